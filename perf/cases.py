@@ -232,20 +232,35 @@ def _tensor(c, H, gen=None):
     return t if c["layout"] == "bhld" else t.transpose(1, 2)
 
 
-def prepare(case, seed):
-    c = case
+def _inputs(c, seed):
+    """The tensors a program has in hand before the call."""
     gen = torch.Generator(device="cuda")
     gen.manual_seed(seed)
+    B, Hq, Hkv, D, T = c["B"], c["Hq"], c["Hkv"], c["D"], c.get("T", 0)
     if c["kind"] in ("decode", "chunk"):
-        return _prepare_serve(c, gen)
+        cap, step = c["sink"] + c["window"], (1,) if c["kind"] == "decode" else (T,)
+        s = {"k_cache": _randn(gen, B, Hkv, cap, D), "v_cache": _randn(gen, B, Hkv, cap, D)}
+        s.update(q=_randn(gen, B, Hq, *(step if c["kind"] == "chunk" else ()), D), k=_randn(gen, B, Hkv, *step, D),
+                 v=_randn(gen, B, Hkv, *step, D))
+        return s
+    s = {"q": _tensor(c, Hq, gen), "k": _tensor(c, Hkv, gen), "v": _tensor(c, Hkv, gen)}
+    if c["kind"] != "prefill":
+        s["do"] = _tensor(c, Hq, gen)
+    if c["doc_mean"]:
+        s["docs"] = _doc_starts(c, seed).cuda()
+    return s
+
+
+def prepare(case, seed):
+    c = case
+    s = dict(_inputs(c, seed), kind=c["kind"])
+    if c["kind"] in ("decode", "chunk"):
+        return _prepare_serve(c, s)
     want_bwd = c["kind"] != "prefill"
-    s = {"kind": c["kind"], "q": _tensor(c, c["Hq"], gen), "k": _tensor(c, c["Hkv"], gen),
-         "v": _tensor(c, c["Hkv"], gen), "o": _tensor(c, c["Hq"]),
-         "lse": torch.empty(c["B"], c["Hq"], c["L"], dtype=torch.float32, device="cuda")}
+    s.update(o=_tensor(c, c["Hq"]), lse=torch.empty(c["B"], c["Hq"], c["L"], dtype=torch.float32, device="cuda"))
     if want_bwd:
-        s.update(do=_tensor(c, c["Hq"], gen), dq=_tensor(c, c["Hq"]), dk=_tensor(c, c["Hkv"]),
-                 dv=_tensor(c, c["Hkv"]))
-    docs = _doc_starts(c, seed).cuda() if c["doc_mean"] else None
+        s.update(dq=_tensor(c, c["Hq"]), dk=_tensor(c, c["Hkv"]), dv=_tensor(c, c["Hkv"]))
+    docs = s.get("docs")
     p = lg.attn_params(c["B"], c["Hq"], c["Hkv"], c["L"], c["D"], c["block"], c["mode"], c["sink"], c["window"],
                        c["stride"], c["local"], window_exact=c["exact"], doc_start=docs)
     s["p"], s["ws"] = p, lg.attn_workspace(p, want_bwd)
@@ -255,21 +270,17 @@ def prepare(case, seed):
     return s
 
 
-def _prepare_serve(c, gen):
+def _prepare_serve(c, s):
     B, Hq, Hkv, D = c["B"], c["Hq"], c["Hkv"], c["D"]
-    cap = c["sink"] + c["window"]
-    p = lg.decode_params(B, Hq, Hkv, D, c["sink"], c["window"], block_tokens=c["block_tokens"])
-    s = {"kind": c["kind"], "p": p, "k_cache": _randn(gen, B, Hkv, cap, D), "v_cache": _randn(gen, B, Hkv, cap, D)}
+    s["p"] = p = lg.decode_params(B, Hq, Hkv, D, c["sink"], c["window"], block_tokens=c["block_tokens"])
     if c["kind"] == "chunk":
         T = c["T"]
-        s.update(q=_randn(gen, B, Hq, T, D), k=_randn(gen, B, Hkv, T, D), v=_randn(gen, B, Hkv, T, D),
-                 o=torch.empty(B, Hq, T, D, dtype=torch.bfloat16, device="cuda"),
+        s.update(o=torch.empty(B, Hq, T, D, dtype=torch.bfloat16, device="cuda"),
                  lse=torch.empty(B, Hq, T, dtype=torch.float32, device="cuda"), n=c["n_min"],
                  ws=lg.chunk_prefill_workspace(p, T, c["n_min"]))
         return s
     n = torch.tensor(_lengths(c), dtype=torch.int64).cuda()
-    s.update(q=_randn(gen, B, Hq, D), k=_randn(gen, B, Hkv, 1, D), v=_randn(gen, B, Hkv, 1, D), n=n, n_before=n - 1,
-             o=torch.empty(B, Hq, D, dtype=torch.bfloat16, device="cuda"),
+    s.update(n=n, n_before=n - 1, o=torch.empty(B, Hq, D, dtype=torch.bfloat16, device="cuda"),
              lse=torch.empty(B, Hq, dtype=torch.float32, device="cuda"), ws=lg.decode_workspace(p))
     # a serving loop's decode: fixed buffers, arguments marshalled once
     s["decode"] = lg.decode_call(p, s["q"], s["k_cache"], s["v_cache"], n, s["o"], s["lse"], s["ws"])
@@ -292,3 +303,107 @@ def run(s):
         return out
     return out + lg.lg_sparse_attn_bwd(p, s["q"], s["k"], s["v"], s["o"], s["lse"], s["do"], dq=s["dq"], dk=s["dk"],
                                        dv=s["dv"], workspace=s["ws"])
+
+
+# ------------------------------------------------------- the same outputs in 64 bits
+
+_MAX_EXACT_FLOPS = 1.5e14    # masked pairs counted: about ten seconds of 64-bit products
+
+
+def _attend(q, k, v, see, do=None):
+    """Rows of masked softmax attention for one head, and what they add to the gradients."""
+    scale = q.shape[-1] ** -0.5
+    x = (q @ k.T).mul_(scale).masked_fill_(~see, -math.inf)
+    lse = torch.logsumexp(x, 1)
+    p = x.sub_(lse[:, None]).exp_()
+    o = p @ v
+    if do is None:
+        return o, lse
+    ds = (do @ v.T).sub_((do * o).sum(1, keepdim=True)).mul_(p).mul_(scale)
+    return o, lse, ds @ k, ds.T @ q, p.T @ do
+
+
+def _seen(c, i, j, doc=None):
+    """Which keys j the queries at positions i see, as the pattern of a training or prefill call says."""
+    bs = c["block"]
+    see = j[None, :] <= i[:, None]
+    if c["mode"] == WINDOW:
+        near = (i[:, None] - j[None, :] < c["window"] if c["exact"] else
+                (i // bs)[:, None] - (j // bs)[None, :] < c["window"] // bs)
+        see &= near | (j < c["sink"])[None, :]
+    elif c["mode"] == STRIDED:
+        see &= ((i // bs)[:, None] - (j // bs)[None, :] < c["local"]) | (j // bs % c["stride"] == 0)[None, :]
+    return see if doc is None else see & (j[None, :] >= doc[:, None])
+
+
+def _exact_attn(c, s):
+    B, Hq, Hkv, L, D, bs, G = c["B"], c["Hq"], c["Hkv"], c["L"], c["D"], c["block"], c["Hq"] // c["Hkv"]
+    grads = "do" in s
+    f64 = dict(dtype=torch.float64, device="cuda")
+    o, lse = torch.empty(B, Hq, L, D, **f64), torch.empty(B, Hq, L, **f64)
+    dq, dk, dv = (torch.zeros(B, H, L, D, **f64) for H in ((Hq, Hkv, Hkv) if grads else (0, 0, 0)))
+    pos = torch.arange(L, device="cuda")
+    rows = 1024 if L <= 65536 else 512
+    for r0 in range(0, L, rows):
+        r1 = min(L, r0 + rows)
+        i = pos[r0:r1]
+        j = pos[:r1]
+        near = r0 - c["window"] - bs if c["mode"] == WINDOW else r0 // bs * bs - c["local"] * bs
+        if c["mode"] == WINDOW:
+            j = j[(j >= near) | (j < c["sink"])]
+        elif c["mode"] == STRIDED:
+            j = j[(j >= near) | (j // bs % c["stride"] == 0)]
+        for b in range(B):
+            see = _seen(c, i, j, s["docs"][b, r0:r1] if "docs" in s else None)
+            for h in range(Hq):
+                kv = (b, h // G, j)
+                got = _attend(s["q"][b, h, r0:r1].double(), s["k"][kv].double(), s["v"][kv].double(), see,
+                              s["do"][b, h, r0:r1].double() if grads else None)
+                o[b, h, r0:r1], lse[b, h, r0:r1] = got[:2]
+                if grads:
+                    dq[b, h, r0:r1] = got[2]
+                    dk[kv] += got[3]
+                    dv[kv] += got[4]
+    return (o, lse, dq, dk, dv) if grads else (o, lse)
+
+
+def _slots(c, n):
+    """The ring slots that hold something after n tokens, and the position of the token in each, oldest first."""
+    sink, window = c["sink"], c["window"]
+    j = torch.cat([torch.arange(min(n, sink)), torch.arange(max(sink, n - window), max(n, sink))]).cuda()
+    return torch.where(j < sink, j, sink + (j - sink) % window), j
+
+
+def _kept(c, i, j):
+    """Which cached positions j a query at position i of a serving call attends."""
+    bs = c["block_tokens"]
+    near = i // bs - j // bs < c["window"] // bs if bs else i - j < c["window"]
+    return (j <= i) & (near | (j < c["sink"]))
+
+
+def _exact_serve(c, s):
+    B, Hq, G, T = c["B"], c["Hq"], c["Hq"] // c["Hkv"], max(1, c["T"])
+    o, lse = torch.empty(s["q"].shape, dtype=torch.float64, device="cuda"), []
+    for b, n in enumerate(_lengths(c)):
+        if c["kind"] == "decode":
+            at = n - 1 if n <= c["sink"] else c["sink"] + (n - 1 - c["sink"]) % c["window"]
+            s["k_cache"][b, :, at], s["v_cache"][b, :, at] = s["k"][b, :, 0], s["v"][b, :, 0]
+        slot, j = _slots(c, n)
+        i = torch.arange(n, n + T, device="cuda") if c["kind"] == "chunk" else torch.tensor([n - 1], device="cuda")
+        every = torch.cat([j, i]) if c["kind"] == "chunk" else j
+        see = _kept(c, i[:, None], every[None, :])
+        for h in range(Hq):
+            k, v = (s[x][b, h // G, slot].double() for x in ("k_cache", "v_cache"))
+            if c["kind"] == "chunk":
+                k, v = torch.cat([k, s["k"][b, h // G].double()]), torch.cat([v, s["v"][b, h // G].double()])
+            got, l = _attend(s["q"][b, h].double().view(T, -1), k, v, see)
+            o[b, h] = got.view(o[b, h].shape)
+            lse.append(l)
+    lse = torch.stack(lse).view(*s["q"].shape[:-1])
+    return (o, lse) if c["kind"] == "chunk" else (o, lse, s["k_cache"].double(), s["v_cache"].double())
+
+
+def exact(case, seed):
+    if work(case)["flops"] > _MAX_EXACT_FLOPS:
+        return None
+    return (_exact_serve if case["kind"] in ("decode", "chunk") else _exact_attn)(case, _inputs(case, seed))
