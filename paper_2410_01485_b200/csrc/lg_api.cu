@@ -84,6 +84,7 @@ lg_status resolve(const lg_attn_params* p, Resolved* r) {
   r->n_qtiles = (p->L + 127) / 128;
   r->n_ktiles = (p->L + 127) / 128;
   r->n_stiles = (p->L + 255) / 256;
+  r->st_row0 = 0;
   r->q_start = 0;
   r->Lq = p->L;
   if (reinterpret_cast<uintptr_t>(p->doc_start) & 3) return LG_ERR_INVALID_ARG;
@@ -180,31 +181,25 @@ WsLayout ws_layout(const Resolved& r, bool want_bwd) {
     off = align_up(off + bytes, 256);
     return o;
   };
-  const size_t nB = r.pat.nB, nnz = static_cast<size_t>(r.nnz);
-  w.row_ptr = take((nB + 1) * 4);
-  w.col_idx = take(nnz * 4);
-  w.col_ptr = take((nB + 1) * 4);
-  w.row_idx = take(nnz * 4);
-  w.qt_cnt = take(r.n_qtiles * 4);
-  w.qt_ent = take(nnz * 4);
-  w.qt_order = take(r.n_qtiles * 4);
+  const size_t nnz = static_cast<size_t>(r.nnz);
+  w.sq_off = take(r.n_stiles * 4);
   w.sq_cnt = take(r.n_stiles * 4);
   w.sq_ent = take(nnz * 4);
   w.sq_order = take(r.n_stiles * 4);
   if (want_bwd) {
-    w.kt_cnt = take(r.n_ktiles * 4);
+    const bool keep = bwd_variant(r) == kBwdKeepDs;
+    w.qt_off = take(static_cast<size_t>(r.n_qtiles) * 4);
+    w.qt_cnt = take(static_cast<size_t>(r.n_qtiles) * 4);
+    w.qt_ent = take(nnz * (keep ? kDqEntInts : 1) * 4);
+    w.qt_order = take(static_cast<size_t>(r.n_qtiles) * 4);
+    w.kt_off = take(static_cast<size_t>(r.n_ktiles) * 4);
+    w.kt_cnt = take(static_cast<size_t>(r.n_ktiles) * 4);
     w.kt_ent = take(nnz * 4);
-    w.kt_order = take(r.n_ktiles * 4);
+    w.kt_order = take(static_cast<size_t>(r.n_ktiles) * 4);
     w.kt_cols = take(static_cast<size_t>(r.n_ktiles) * 2 * 4);
-    w.kt_off = take((static_cast<size_t>(r.n_ktiles) + 1) * 4);
     if (r.doc_start) w.doc_end = take(static_cast<size_t>(r.B) * r.L * 4);
     w.delta = take(static_cast<size_t>(r.B) * r.Hq * align_up(r.L, 128) * 8);   // rows padded to whole tiles   // two planes: -LSE * log2 e and -delta per query row
-    if (bwd_variant(r) == kBwdKeepDs) {
-      w.kt_tile_of = take(nB * 4);
-      w.dq_cnt = take(static_cast<size_t>(r.n_qtiles) * 4);
-      w.dq_ent = take(nnz * kDqEntInts * 4);
-      w.ds_buf = take(ds_buffer_bytes(r));
-    }
+    if (keep) w.ds_buf = take(ds_buffer_bytes(r));
   }
   w.total = off;
   return w;
@@ -212,10 +207,7 @@ WsLayout ws_layout(const Resolved& r, bool want_bwd) {
 
 lg_status launch_index_build(const Resolved& r, int32_t* row_ptr, int32_t* col_idx, int32_t* col_ptr,
                              int32_t* row_idx, cudaStream_t stream) {
-  const int nB = r.pat.nB;
-  index_count_kernel<<<nB, 128, 0, stream>>>(r.pat, row_ptr, col_ptr); note_launch();
-  index_scan_kernel<<<2, 1024, 0, stream>>>(row_ptr, col_ptr, nB); note_launch();
-  index_fill_kernel<<<nB, 64, 0, stream>>>(r.pat, row_ptr, col_idx, col_ptr, row_idx); note_launch();
+  index_fill_kernel<<<r.pat.nB + 1, 64, 0, stream>>>(r.pat, row_ptr, col_idx, col_ptr, row_idx); note_launch();
   return cudaGetLastError() == cudaSuccess ? LG_OK : LG_ERR_CUDA;
 }
 
@@ -232,60 +224,50 @@ unsigned long long pattern_fingerprint(const Resolved& r, bool has_bwd) {
   return h ? h : 1;
 }
 
-// Start of a call that (re)builds the lists: a header that was never initialised is reset, an
-// error word nobody has read yet moves to `latched`, and the fingerprint is withdrawn until the
-// lists are whole again.
-__global__ void header_begin_kernel(WsHeader* h) {
-  if (h->magic != kWsMagic) { h->magic = kWsMagic; h->latched = 0; }
-  else if (h->error_word != 0 && h->latched == 0) h->latched = h->error_word;
-  h->error_word = 0;
-  h->fingerprint = 0;
-}
-__global__ void header_stamp_kernel(WsHeader* h, unsigned long long fp) { h->fingerprint = fp; }
+__global__ void header_begin_kernel(WsHeader* h) { header_begin(h); }
 
 lg_status begin_workspace(uint8_t* ws, cudaStream_t stream) {
   header_begin_kernel<<<1, 1, 0, stream>>>(reinterpret_cast<WsHeader*>(ws)); note_launch();
   return cudaGetLastError() == cudaSuccess ? LG_OK : LG_ERR_CUDA;
 }
 
-// what: bit 0 = the forward's super-tile schedule, bit 1 = the backward's schedules
-lg_status prepare_workspace(const Resolved& r, const WsLayout& w, uint8_t* ws, int what, cudaStream_t stream) {
+lg_status prepare_workspace(const Resolved& r, const WsLayout& w, uint8_t* ws, int what, bool begin,
+                            unsigned long long fp, cudaStream_t stream, const RingCopy* copy) {
   const bool want_fwd = (what & 1) != 0, want_bwd = (what & 2) != 0;
   auto i32 = [&](size_t off) { return reinterpret_cast<int32_t*>(ws + off); };
+  SchedArgs a{};
+  a.p = r.pat;
   // The lists are shared by all sequences of the batch, so documents can only prune them when there
   // is one sequence (the usual case for long packed samples); otherwise they stay the pattern's own.
-  Resolved rl = r;
-  if (r.doc_start && r.B == 1) rl.pat.doc_start = r.doc_start;
-  lg_status s = launch_index_build(rl, i32(w.row_ptr), i32(w.col_idx), i32(w.col_ptr), i32(w.row_idx), stream);
-  if (s != LG_OK) return s;
-  const int R = 128 / r.block;
+  if (r.doc_start && r.B == 1) a.p.doc_start = r.doc_start;
+  WsHeader* header = reinterpret_cast<WsHeader*>(ws);
+  a.header = begin ? header : nullptr;
+  a.R = 128 / r.block;
+  a.L = r.L;
   if (want_fwd) {   // the forward walks super-tiles of 256 rows; the backward passes have their own schedules
-    tile_merge4_kernel<<<(r.n_stiles + 127) / 128, 128, 0, stream>>>(i32(w.row_ptr), i32(w.col_idx), r.pat.nB, 2 * R,
-                                                                     r.n_stiles, i32(w.sq_cnt), i32(w.sq_ent)); note_launch();
-    tile_order_kernel<<<(r.n_stiles + 127) / 128, 128, 0, stream>>>(i32(w.sq_cnt), r.n_stiles, i32(w.sq_order)); note_launch();
+    a.n_stiles = r.n_stiles; a.st_row0 = r.st_row0;
+    a.sq_off = i32(w.sq_off); a.sq_cnt = i32(w.sq_cnt); a.sq_ent = i32(w.sq_ent); a.sq_order = i32(w.sq_order);
   }
   if (want_bwd) {
-    const int nB = r.pat.nB, nt = r.n_ktiles;
-    tile_merge_kernel<<<(r.n_qtiles + 127) / 128, 128, 0, stream>>>(i32(w.row_ptr), i32(w.col_idx), nB, R, r.n_qtiles,
-                                                                    i32(w.qt_cnt), i32(w.qt_ent)); note_launch();
-    tile_order_kernel<<<(r.n_qtiles + 127) / 128, 128, 0, stream>>>(i32(w.qt_cnt), r.n_qtiles, i32(w.qt_order)); note_launch();
-    kv_tile_cols_kernel<<<(nt * R + 127) / 128, 128, 0, stream>>>(i32(w.col_ptr), nB, R, nt, i32(w.kt_cols)); note_launch();
-    kv_tile_len_kernel<<<(nt + 127) / 128, 128, 0, stream>>>(i32(w.col_ptr), i32(w.kt_cols), R, nt, i32(w.kt_off)); note_launch();
-    index_scan_kernel<<<1, 1024, 0, stream>>>(i32(w.kt_off), i32(w.kt_off), nt); note_launch();
-    kv_tile_merge_kernel<<<(nt + 127) / 128, 128, 0, stream>>>(i32(w.col_ptr), i32(w.row_idx), i32(w.kt_cols),
-                                                               i32(w.kt_off), R, nt, i32(w.kt_cnt), i32(w.kt_ent)); note_launch();
-    tile_order_kernel<<<(nt + 127) / 128, 128, 0, stream>>>(i32(w.kt_cnt), nt, i32(w.kt_order)); note_launch();
-    if (bwd_variant(r) == kBwdKeepDs) {   // which dS tiles each query tile reads back
-      kv_tile_of_kernel<<<(nt * R + 127) / 128, 128, 0, stream>>>(i32(w.kt_cols), R, nt, i32(w.kt_tile_of)); note_launch();
-      dq_sched_kernel<<<(r.n_qtiles + 63) / 64, 64, 0, stream>>>(i32(w.row_ptr), i32(w.col_idx), i32(w.col_ptr),
-                                                                  i32(w.row_idx), i32(w.kt_tile_of), i32(w.kt_cols), R, nB,
-                                                                  r.n_qtiles, i32(w.dq_cnt), i32(w.dq_ent)); note_launch();
-    }
+    a.n_qtiles = r.n_qtiles; a.n_ktiles = r.n_ktiles;
+    a.keep_ds = bwd_variant(r) == kBwdKeepDs;
+    a.qt_off = i32(w.qt_off); a.qt_cnt = i32(w.qt_cnt); a.qt_ent = i32(w.qt_ent); a.qt_order = i32(w.qt_order);
+    a.kt_off = i32(w.kt_off); a.kt_cnt = i32(w.kt_cnt); a.kt_ent = i32(w.kt_ent); a.kt_order = i32(w.kt_order);
+    a.kt_cols = i32(w.kt_cols);
     if (r.doc_start) {
-      const int64_t n = static_cast<int64_t>(r.B) * r.L;
-      doc_end_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, stream>>>(r.doc_start, i32(w.doc_end), r.B, r.L); note_launch();
+      a.doc_start = r.doc_start;
+      a.doc_end = i32(w.doc_end);
+      a.n_doc = static_cast<int64_t>(r.B) * r.L;
     }
   }
+  constexpr int kWarps = kSchedThreads / 32;
+  if (copy) a.copy = *copy;
+  const int64_t tiles = static_cast<int64_t>(a.n_stiles) + a.n_qtiles + a.n_ktiles;
+  const int64_t warps = tiles + (a.n_doc + 31) / 32 + (a.copy.n + 31) / 32;
+  if (warps > 0x7fffffffll) return LG_ERR_UNSUPPORTED;
+  sched_build_kernel<<<static_cast<unsigned>((warps + kWarps - 1) / kWarps), kSchedThreads, 0, stream>>>(a); note_launch();
+  a.header = header;
+  sched_order_kernel<<<static_cast<unsigned>((tiles + kWarps - 1) / kWarps), kSchedThreads, 0, stream>>>(a, fp); note_launch();
   return cudaGetLastError() == cudaSuccess ? LG_OK : LG_ERR_CUDA;
 }
 
@@ -325,40 +307,6 @@ lg_status make_tmap(CUtensorMap* out, const void* base, int B, int H, int L, int
 
 
 // ---- chunk served against a sink + window ring ----------------------------------------------
-// Time-ordered copy of what the ring holds, followed by the chunk: K_lin, V_lin [B, Hkv, Lc, D]
-// with Lc = kept + T.  Row v < kept is the cache slot of position
-//   v                                   (v < sink: the sink never moves)
-//   n_before - (kept - sink) + v - sink (the kept window tokens, oldest first),
-// row v >= kept is chunk token v - kept.  One 16-byte copy per thread.
-__global__ void ring_linearise_kernel(const __nv_bfloat16* __restrict__ k_cache, const __nv_bfloat16* __restrict__ v_cache,
-                                      const __nv_bfloat16* __restrict__ k_chunk, const __nv_bfloat16* __restrict__ v_chunk,
-                                      __nv_bfloat16* __restrict__ k_lin, __nv_bfloat16* __restrict__ v_lin, int B, int Hkv,
-                                      int D, int sink, int window, int kept, int T, int64_t n_before) {
-  const int cpr = D / 8;   // 16-byte chunks per row
-  const int Lc = kept + T;
-  const int64_t gid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t total = static_cast<int64_t>(B) * Hkv * Lc * cpr;
-  if (gid >= total) return;
-  const int c = static_cast<int>(gid % cpr);
-  const int v = static_cast<int>((gid / cpr) % Lc);
-  const int64_t bh = gid / (static_cast<int64_t>(cpr) * Lc);
-  const __nv_bfloat16 *ksrc, *vsrc;
-  if (v < kept) {
-    const int64_t pos = v < sink ? v : n_before - (kept - sink) + (v - sink);
-    const int64_t slot = pos < sink ? pos : sink + (pos - sink) % window;
-    const int64_t off = (bh * (sink + window) + slot) * D + c * 8;
-    ksrc = k_cache + off;
-    vsrc = v_cache + off;
-  } else {
-    const int64_t off = (bh * T + (v - kept)) * D + c * 8;
-    ksrc = k_chunk + off;
-    vsrc = v_chunk + off;
-  }
-  const int64_t dst = (bh * Lc + v) * D + c * 8;
-  *reinterpret_cast<uint4*>(k_lin + dst) = *reinterpret_cast<const uint4*>(ksrc);
-  *reinterpret_cast<uint4*>(v_lin + dst) = *reinterpret_cast<const uint4*>(vsrc);
-}
-
 struct ChunkPlan {
   lg_attn_params ap;     // exact-window sink + window attention over the kept tokens and the chunk
   Resolved r;
@@ -400,6 +348,10 @@ static lg_status plan_chunk(const lg_decode_params* p, int32_t T, int64_t n_befo
   lg_status s = resolve(&ap, &c->r);
   if (s != LG_OK) return s;
   c->r.q_start = c->kept;
+  // super-tiles start at the chunk's first 64-token block: with tiles counted from the start of the virtual
+  // sequence a chunk that fits k of them would straddle k + 1, and the grid would hold the empty ones before it
+  c->r.st_row0 = c->kept / ap.block;
+  c->r.n_stiles = (ap.L - c->r.st_row0 * ap.block + 255) / 256;
   c->r.Lq = T;
   // Block-aligned window: every non-sink row v of the virtual sequence (kept tokens, then the chunk) is the
   // token at position v + (n_before - kept), so the block-granular edge of the real positions is a
@@ -509,10 +461,7 @@ lg_status lg_sparse_attn_prepare(const lg_attn_params* p, void* workspace, size_
   if ((s = check_arch()) != LG_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   uint8_t* ws = static_cast<uint8_t*>(workspace);
-  if ((s = begin_workspace(ws, st)) != LG_OK) return s;
-  if ((s = prepare_workspace(r, ws_layout(r, want_bwd != 0), ws, want_bwd ? 3 : 1, st)) != LG_OK) return s;
-  header_stamp_kernel<<<1, 1, 0, st>>>(reinterpret_cast<WsHeader*>(ws), pattern_fingerprint(r, want_bwd != 0)); note_launch();
-  return cudaGetLastError() == cudaSuccess ? LG_OK : LG_ERR_CUDA;
+  return prepare_workspace(r, ws_layout(r, want_bwd != 0), ws, want_bwd ? 3 : 1, true, pattern_fingerprint(r, want_bwd != 0), st);
 }
 
 }  // extern "C"
@@ -537,14 +486,14 @@ lg_status attn_fwd_entry(const lg_attn_params* p, const void* q, const void* k, 
     r.expect_fp2 = pattern_fingerprint(r, true);
     return launch_fwd(r, ws_layout(r, false), q, k, v, o, lse, ws, st);
   }
-  if ((s = begin_workspace(ws, st)) != LG_OK) return s;
   if (per_sequence(r)) {
+    if ((s = begin_workspace(ws, st)) != LG_OK) return s;
     const size_t per = attn_workspace_total(r, false) / r.B;
     for (int b = 0; b < r.B; ++b) {
       const Resolved r1 = one_sequence(r, b, workspace);
       const WsLayout w1 = ws_layout(r1, false);
       uint8_t* wsb = ws + b * per;
-      if ((s = prepare_workspace(r1, w1, wsb, 1, st)) != LG_OK) return s;
+      if ((s = prepare_workspace(r1, w1, wsb, 1, false, 0, st)) != LG_OK) return s;
       s = launch_fwd(r1, w1, seq_ptr(q, b, r.qs[0]), seq_ptr(k, b, r.ks[0]), seq_ptr(v, b, r.vs[0]),
                      seq_ptr(o, b, r.os[0]), lse + static_cast<int64_t>(b) * r.Hq * r.L, wsb, st);
       if (s != LG_OK) return s;
@@ -552,7 +501,7 @@ lg_status attn_fwd_entry(const lg_attn_params* p, const void* q, const void* k, 
     return LG_OK;
   }
   const WsLayout w = ws_layout(r, false);
-  if ((s = prepare_workspace(r, w, ws, 1, st)) != LG_OK) return s;
+  if ((s = prepare_workspace(r, w, ws, 1, true, 0, st)) != LG_OK) return s;
   return launch_fwd(r, w, q, k, v, o, lse, ws, st);
 }
 
@@ -577,14 +526,14 @@ lg_status attn_bwd_entry(const lg_attn_params* p, const void* q, const void* k, 
     r.expect_fp = r.expect_fp2 = pattern_fingerprint(r, true);
     return launch_bwd(r, ws_layout(r, true), q, k, v, o, lse, d_o, dq, dk, dv, ws, st, marks);
   }
-  if ((s = begin_workspace(ws, st)) != LG_OK) return s;
   if (per_sequence(r)) {
+    if ((s = begin_workspace(ws, st)) != LG_OK) return s;
     const size_t per = attn_workspace_total(r, true) / r.B;
     for (int b = 0; b < r.B; ++b) {
       const Resolved r1 = one_sequence(r, b, workspace);
       const WsLayout w1 = ws_layout(r1, true);
       uint8_t* wsb = ws + b * per;
-      if ((s = prepare_workspace(r1, w1, wsb, 2, st)) != LG_OK) return s;
+      if ((s = prepare_workspace(r1, w1, wsb, 2, false, 0, st)) != LG_OK) return s;
       s = launch_bwd(r1, w1, seq_ptr(q, b, r.qs[0]), seq_ptr(k, b, r.ks[0]), seq_ptr(v, b, r.vs[0]),
                      seq_ptr(o, b, r.os[0]), lse + static_cast<int64_t>(b) * r.Hq * r.L, seq_ptr(d_o, b, r.os[0]),
                      seq_ptr(dq, b, r.qs[0]), seq_ptr(dk, b, r.ks[0]), seq_ptr(dv, b, r.vs[0]), wsb, st,
@@ -594,7 +543,7 @@ lg_status attn_bwd_entry(const lg_attn_params* p, const void* q, const void* k, 
     return LG_OK;
   }
   const WsLayout w = ws_layout(r, true);
-  if ((s = prepare_workspace(r, w, ws, 2, st)) != LG_OK) return s;
+  if ((s = prepare_workspace(r, w, ws, 2, true, 0, st)) != LG_OK) return s;
   return launch_bwd(r, w, q, k, v, o, lse, d_o, dq, dk, dv, ws, st, marks);
 }
 
@@ -651,16 +600,15 @@ lg_status lg_chunk_prefill(const lg_decode_params* p, const void* q_chunk, const
   uint8_t* ws = static_cast<uint8_t*>(workspace);
   __nv_bfloat16* k_lin = reinterpret_cast<__nv_bfloat16*>(ws + c.o_k);
   __nv_bfloat16* v_lin = reinterpret_cast<__nv_bfloat16*>(ws + c.o_v);
-  const int64_t threads = static_cast<int64_t>(p->B) * p->Hkv * c.ap.L * (p->D / 8);
-  const int64_t blocks = (threads + 255) / 256;
-  if (blocks > 0x7fffffff) return LG_ERR_UNSUPPORTED;
-  ring_linearise_kernel<<<static_cast<unsigned>(blocks), 256, 0, st>>>(
-      static_cast<const __nv_bfloat16*>(k_cache), static_cast<const __nv_bfloat16*>(v_cache),
-      static_cast<const __nv_bfloat16*>(k_chunk), static_cast<const __nv_bfloat16*>(v_chunk), k_lin, v_lin, p->B,
-      p->Hkv, p->D, p->sink_tokens, p->window_tokens, c.kept, T, n_tokens_before); note_launch();
-  if (cudaGetLastError() != cudaSuccess) return LG_ERR_CUDA;
-  if ((s = begin_workspace(ws, st)) != LG_OK) return s;
-  if ((s = prepare_workspace(c.r, c.w, ws, 1, st)) != LG_OK) return s;
+  RingCopy copy;
+  copy.k_cache = static_cast<const uint4*>(k_cache); copy.v_cache = static_cast<const uint4*>(v_cache);
+  copy.k_chunk = static_cast<const uint4*>(k_chunk); copy.v_chunk = static_cast<const uint4*>(v_chunk);
+  copy.k_lin = reinterpret_cast<uint4*>(k_lin); copy.v_lin = reinterpret_cast<uint4*>(v_lin);
+  copy.n = static_cast<int64_t>(p->B) * p->Hkv * c.ap.L * (p->D / 8);
+  copy.row_chunks = p->D / 8;
+  copy.sink = p->sink_tokens; copy.window = p->window_tokens; copy.kept = c.kept; copy.T = T;
+  copy.n_before = n_tokens_before;
+  if ((s = prepare_workspace(c.r, c.w, ws, 1, true, 0, st, &copy)) != LG_OK) return s;
   return launch_fwd(c.r, c.w, q_chunk, k_lin, v_lin, o, lse, ws, st);
 }
 

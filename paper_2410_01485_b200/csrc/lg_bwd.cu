@@ -37,7 +37,7 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
   a.scale_log2 = r.scale * 1.4426950408889634f;
   a.ds_nnz = r.nnz;
   a.ds_buf = reinterpret_cast<__nv_bfloat16*>(ws + w.ds_buf);
-  a.col_ptr = reinterpret_cast<const int32_t*>(ws + w.col_ptr);
+  a.pat = r.pat;
   constexpr int smem = BwdSmem<D, BS>::kTotal;
   const BwdVariant variant = bwd_variant(r);
 
@@ -94,10 +94,10 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
     // ---- dQ = scale * dS K from the kept tiles --------------------------------------------
     CUtensorMap tk;
     if ((s = make_tmap(&tk, k, r.B, r.Hkv, r.L, D, r.ks, BS)) != LG_OK) return s;
-    a.tile_off = reinterpret_cast<const int32_t*>(ws + w.row_ptr);
-    a.tile_ent = reinterpret_cast<const int32_t*>(ws + w.dq_ent);
+    a.tile_off = reinterpret_cast<const int32_t*>(ws + w.qt_off);
+    a.tile_ent = reinterpret_cast<const int32_t*>(ws + w.qt_ent);
     a.tile_cols = reinterpret_cast<const int32_t*>(ws + w.kt_cols);
-    a.tile_cnt = reinterpret_cast<const int32_t*>(ws + w.dq_cnt);
+    a.tile_cnt = reinterpret_cast<const int32_t*>(ws + w.qt_cnt);
     a.order = reinterpret_cast<const int32_t*>(ws + w.qt_order);
     a.out0 = static_cast<__nv_bfloat16*>(dq);
     a.out1 = nullptr;
@@ -121,7 +121,7 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
     if ((s = make_tmap(&tdo, d_o, r.B, r.Hq, r.L, D, r.os, 128)) != LG_OK) return s;
     if ((s = make_tmap(&tk, k, r.B, r.Hkv, r.L, D, r.ks, BS)) != LG_OK) return s;
     if ((s = make_tmap(&tv, v, r.B, r.Hkv, r.L, D, r.vs, BS)) != LG_OK) return s;
-    a.tile_off = reinterpret_cast<const int32_t*>(ws + w.row_ptr);
+    a.tile_off = reinterpret_cast<const int32_t*>(ws + w.qt_off);
     a.tile_cols = nullptr;
     a.tile_cnt = reinterpret_cast<const int32_t*>(ws + w.qt_cnt);
     a.tile_ent = reinterpret_cast<const int32_t*>(ws + w.qt_ent);

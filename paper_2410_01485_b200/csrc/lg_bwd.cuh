@@ -29,11 +29,12 @@
 #pragma once
 #include <cuda.h>
 #include "lg_common.cuh"
+#include "lg_pattern.h"
 
 namespace lg {
 
 struct BwdArgs {
-  const int32_t* tile_off;   // dQ pass: CSR row_ptr (tile t starts at tile_off[R t]); dK/dV pass: start per tile
+  const int32_t* tile_off;   // where a tile's entries start
   const int32_t* tile_cols;  // dK/dV pass: pattern column of each member of a kv tile (-1: none)
   const int32_t* tile_cnt;
   const int32_t* tile_ent;   // idx * 4 + member mask
@@ -55,7 +56,7 @@ struct BwdArgs {
   float scale, scale_log2;
   // dK/dV pass that also keeps dS (see bwd_dkdv_kernel): dS^T of every block of the pattern goes to ds_buf
   // in tiles of 64 queries x KT keys, KT = the block size: with p = the block's position in the column
-  // lists (col_ptr[column] + rank of the query block in the column), a head's tiles are 2 p and 2 p + 1
+  // lists (col_pos), a head's tiles are 2 p and 2 p + 1
   // (the block's two 64-query halves, 16 KB each) with 128-token blocks and p (8 KB) with 64-token
   // blocks; head (b, h) starts at tile (b * Hq + h) * ds_nnz * (block / 64).  The dQ pass reads them back.
   // Inside a tile the element (key k, query q) sits at byte (q / 8) * 16 KT + k * 16 + (q % 8) * 2: eight
@@ -64,7 +65,7 @@ struct BwdArgs {
   // and a layout in which the 32 key rows of a warp write 512 contiguous bytes per store instruction.
   int64_t ds_nnz;
   __nv_bfloat16* ds_buf;
-  const int32_t* col_ptr;    // column lists of the pattern (dK/dV pass that keeps dS: positions of its blocks)
+  PatternDev pat;            // dK/dV pass that keeps dS: positions of the blocks
   int ahead;                 // dK/dV pass: CTAs that run at a time (see prefetch_successor), 0: no prefetch
   int head_group;            // dK/dV pass: kv heads whose CTAs run side by side (cta_coords); >= gridDim.x: all of them
   int descending;            // dK/dV pass: walk a tile's entries from the last query block down (see the producer)
@@ -206,7 +207,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
   cta_coords(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, cta_x, cta_y);
   const int tile = checked(a.order[cta_y], 0, a.n_tiles - 1, a.error_word, 110);
   const int b = cta_x / a.Hq, h = cta_x % a.Hq, hk = h / a.G;
-  const int ent_off = checked(a.tile_off[tile * R], 0, a.n_list, a.error_word, 111);
+  const int ent_off = checked(a.tile_off[tile], 0, a.n_list, a.error_word, 111);
   const int n_ent = checked(a.tile_cnt[tile], 0, a.n_list - ent_off, a.error_word, 112);
   const int32_t* ent = a.tile_ent + ent_off;
   const int row0 = tile * 128;
@@ -592,18 +593,17 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       // rows of their own again).
       const int e_step = a.descending ? -1 : 1;
       int grp = 0, e = a.descending ? n_ent - 1 : 0;    // (query head within the group, entry) of the next item
-      // positions, in the column lists, of the members' next blocks: the entries that carry a member's bit
-      // are that column's query blocks in the same order
-      auto col_first = [&](int kb) { return (!kSpill || kb < 0) ? 0 : (a.descending ? a.col_ptr[kb + 1] - 1 : a.col_ptr[kb]); };
-      int pos_a = col_first(kb_a), pos_b = col_first(kb_b);
+      // number of a member's dS tile: its block's position in the column lists (col_pos), the query block added
+      // (a member that an entry does not list has no tile; its number is not used)
+      const int pos_a = kSpill ? col_start(a.pat, kb_a) - kb_a : 0, pos_b = (kSpill && kb_b >= 0) ? col_start(a.pat, kb_b) - kb_b : 0;
       auto next_item = [&](int& hq, int& qrow, int& entry, int64_t& ta, int64_t& tb) {
         entry = ent[e];
         hq = hk * a.G + grp;
         qrow = checked(entry >> 2, 0, a.nB - 1, a.error_word, 125) * BS;   // (also the address of the item's statistics)
         const int64_t head_base = (static_cast<int64_t>(b) * a.Hq + hq) * a.ds_nnz;
-        ta = (head_base + pos_a) * (BS / 64);
-        tb = (head_base + pos_b) * (BS / 64);
-        if (++grp == a.G) { grp = 0; pos_a += e_step * (entry & 1); pos_b += e_step * ((entry >> 1) & 1); e += e_step; }
+        ta = (head_base + pos_a + (entry >> 2)) * (BS / 64);
+        tb = (head_base + pos_b + (entry >> 2)) * (BS / 64);
+        if (++grp == a.G) { grp = 0; e += e_step; }
       };
       // Each load is started as soon as its ring slot is free, in the order in which the slots come
       // free: dO of step j (its slot is released when the dV and dP^T products of step j - 2 are done),
@@ -1037,7 +1037,7 @@ bwd_dq_from_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const BwdArgs a,
     const int x = static_cast<int>(w % n_heads), y = static_cast<int>(w / n_heads);
     it.b = x / a.Hq; it.h = x % a.Hq;
     it.t = checked(a.order[y], 0, a.n_tiles - 1, a.error_word, 130);   // query tile (128 rows)
-    const int ent_off = checked(a.tile_off[R * it.t], 0, a.n_list, a.error_word, 131);
+    const int ent_off = checked(a.tile_off[it.t], 0, a.n_list, a.error_word, 131);
     it.n_ent = checked(a.tile_cnt[it.t], 0, a.n_list - ent_off, a.error_word, 132);
     it.ent = a.tile_ent + kDqEntInts * static_cast<int64_t>(ent_off);   // (kv tile, dS tiles of its quarters)
     return it;

@@ -13,7 +13,7 @@ static lg_status launch_fwd_t(const Resolved& r, const WsLayout& w, const void* 
   if ((s = make_tmap(&tk, k, r.B, r.Hkv, r.L, D, r.ks, BS)) != LG_OK) return s;
   if ((s = make_tmap(&tv, v, r.B, r.Hkv, r.L, D, r.vs, BS)) != LG_OK) return s;
   FwdArgs a;
-  a.tile_off = reinterpret_cast<const int32_t*>(ws + w.row_ptr);
+  a.tile_off = reinterpret_cast<const int32_t*>(ws + w.sq_off);
   a.tile_cnt = reinterpret_cast<const int32_t*>(ws + w.sq_cnt);
   a.tile_ent = reinterpret_cast<const int32_t*>(ws + w.sq_ent);
   a.order = reinterpret_cast<const int32_t*>(ws + w.sq_order);
@@ -26,6 +26,7 @@ static lg_status launch_fwd_t(const Resolved& r, const WsLayout& w, const void* 
   for (int i = 0; i < 3; ++i) a.o_strides[i] = r.os[i];
   a.L = r.L; a.Hq = r.Hq; a.G = r.G;
   a.q_start = r.q_start; a.Lq = r.Lq;
+  a.row_origin = r.st_row0 * r.block;
   a.exact_w = r.exact_w; a.ns = r.pat.ns;
   a.win_block = r.win_block; a.win_phase = r.win_phase;
   a.doc_start = r.doc_start;

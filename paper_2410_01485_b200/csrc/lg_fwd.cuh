@@ -26,7 +26,7 @@
 namespace lg {
 
 struct FwdArgs {
-  const int32_t* tile_off;   // row_ptr (CSR): entries of super-tile t start at tile_off[(256 / block) * t]
+  const int32_t* tile_off;   // [n_super_tiles] where a super-tile's entries start
   const int32_t* tile_cnt;   // [n_super_tiles]
   const int32_t* tile_ent;   // kb * 16 + member mask (bit r: pattern row r of the super-tile has the block)
   const int32_t* order;      // [n_super_tiles] launch rank -> super-tile
@@ -39,6 +39,7 @@ struct FwdArgs {
   int L, Hq, G;              // G = Hq / Hkv
   int q_start, Lq;           // queries exist for rows [q_start, q_start + Lq) of the L key positions only
                              // (a chunk served against a cache); Q, O, LSE are indexed by row - q_start
+  int row_origin;            // first row of super-tile 0 (at most q_start)
   int exact_w, ns;           // token-exact window (0: off) and number of sink blocks
   int win_block, win_phase;  // with exact_w: the window edge is block-aligned in shifted coordinates instead --
                              // row i keeps the keys j with (i + phase) / win_block - (j + phase) / win_block
@@ -102,12 +103,11 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   cta_coords(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, cta_x, cta_y);
   const int tile = checked(a.order[cta_y], 0, a.n_tiles - 1, a.error_word, 100);
   const int b = cta_x / a.Hq, h = cta_x % a.Hq, hk = h / a.G;
-  const int ent_off = checked(a.tile_off[tile * R4], 0, a.n_list, a.error_word, 101);
+  const int ent_off = checked(a.tile_off[tile], 0, a.n_list, a.error_word, 101);
   const int n_ent = checked(a.tile_cnt[tile], 0, a.n_list - ent_off, a.error_word, 102);
   const int32_t* ent = a.tile_ent + ent_off;
-  const int row0 = tile * 256;
+  const int row0 = a.row_origin + tile * 256;
   const int n_steps = (BS == 128) ? n_ent : (n_ent + 1) / 2;
-  if (row0 + 256 <= a.q_start) return;   // no query lives in this super-tile (uniform over the CTA)
 
   // entries of the two halves of step j (0: nobody's member, also past the end)
   auto load_ent = [&](int j, int& e0, int& e1) {

@@ -40,7 +40,7 @@ struct Resolved {          // validated, defaulted copy of lg_attn_params
   int win_block, win_phase;  // forward only, with exact_w: block-aligned window edge in coordinates shifted by win_phase (0: off)
   int64_t qs[3], ks[3], vs[3], os[3];
   int n_qtiles, n_ktiles;  // ceil(L / 128)
-  int n_stiles;            // ceil(L / 256): super-tiles of the forward
+  int n_stiles, st_row0;   // super-tiles of the forward (256 rows each), and the pattern row the first one starts at
   int q_start, Lq;         // forward only: queries exist for rows [q_start, q_start + Lq) (0, L by default)
   const int32_t* doc_start;  // device [B, L] or null: first position of each token's document
   unsigned int* error_word;  // status word of the call when it is not the start of `ws` (null: it is)
@@ -53,15 +53,14 @@ lg_status resolve(const lg_attn_params* p, Resolved* r);
 
 // Layout of the attention workspace (all offsets 256-byte aligned).
 struct WsLayout {
-  size_t row_ptr, col_idx, col_ptr, row_idx;     // the CSR / CSC lists
-  size_t qt_cnt, qt_ent, qt_order;               // query-tile schedules (dQ pass)
-  size_t sq_cnt, sq_ent, sq_order;               // super-tile schedules (forward)
-  size_t kt_cnt, kt_ent, kt_order;               // kv-tile schedules (dK/dV pass)
-  size_t kt_cols, kt_off;                        // members of each kv tile, start of its schedule
+  // per schedule: start of each tile's entries, their number, the entries, launch rank -> tile
+  size_t sq_off, sq_cnt, sq_ent, sq_order;       // super-tiles (forward)
+  size_t qt_off, qt_cnt, qt_ent, qt_order;       // query tiles (dQ pass: over kv blocks, or over the kept dS tiles)
+  size_t kt_off, kt_cnt, kt_ent, kt_order;       // kv tiles (dK/dV pass)
+  size_t kt_cols;                                // pattern columns of each kv tile
   size_t doc_end;                                // int32 [B, L]: end of each token's document (bwd with documents only)
   size_t delta;                                  // 2 x float [B, Hq, L]: -LSE * log2 e, then -delta (bwd only)
-  // backward that keeps dS only (0 otherwise): pattern column -> kv tile, the schedule of its dQ pass, the dS^T tiles
-  size_t kt_tile_of, dq_cnt, dq_ent, ds_buf;
+  size_t ds_buf;                                 // dS^T tiles (backward that keeps dS only, 0 otherwise)
   size_t total;
 };
 WsLayout ws_layout(const Resolved& r, bool want_bwd);
@@ -69,9 +68,12 @@ WsLayout ws_layout(const Resolved& r, bool want_bwd);
 // Build CSR/CSC on `stream` into the given device arrays.
 lg_status launch_index_build(const Resolved& r, int32_t* row_ptr, int32_t* col_idx, int32_t* col_ptr,
                              int32_t* row_idx, cudaStream_t stream);
-// Build lists + tile schedules inside a workspace.
-// `what`: bit 0 = the forward's schedule, bit 1 = the backward's schedules.
-lg_status prepare_workspace(const Resolved& r, const WsLayout& w, uint8_t* ws, int what, cudaStream_t stream);
+struct RingCopy;
+// Build the tile schedules inside a workspace.  `what`: bit 0 = the forward's schedule, bit 1 = the backward's
+// schedules; `begin`: also reset the workspace's header first; `fp`: fingerprint to leave in it (0: none);
+// `copy`: a ring to linearise in the same launch (null: none).
+lg_status prepare_workspace(const Resolved& r, const WsLayout& w, uint8_t* ws, int what, bool begin,
+                            unsigned long long fp, cudaStream_t stream, const RingCopy* copy = nullptr);
 
 // bf16 [B, H, L, D] tensor (element strides bs, hs, ls; D contiguous) as a 4-D tensor map with
 // boxes of 64 columns x `box_rows` rows and the 128-byte swizzle.

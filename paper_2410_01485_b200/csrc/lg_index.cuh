@@ -1,78 +1,27 @@
 // Block-index builder: CSR / CSC lists of active blocks of the static pattern (paper
 // Section 3.2: the mask lives in compressed-sparse-row form and is the same for all heads),
-// plus the per-tile schedules the attention kernels walk.
+// and the per-tile schedules the attention kernels walk.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "lg_common.cuh"
 #include "lg_pattern.h"
 
 namespace lg {
 
-// ---- pass 1: per-row and per-column counts -------------------------------------------
-// grid = nB blocks of 128 threads; block b counts row b and column b.
-__global__ void index_count_kernel(PatternDev p, int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_ptr) {
-  const int b = blockIdx.x;
-  int rc = 0, cc = 0;
-  for (int x = threadIdx.x; x < p.nB; x += blockDim.x) {
-    rc += block_active(p, b, x) ? 1 : 0;
-    cc += block_active(p, x, b) ? 1 : 0;
-  }
-  __shared__ int s_r[4], s_c[4];
-  for (int o = 16; o > 0; o >>= 1) {
-    rc += __shfl_xor_sync(0xffffffffu, rc, o);
-    cc += __shfl_xor_sync(0xffffffffu, cc, o);
-  }
-  if ((threadIdx.x & 31) == 0) { s_r[threadIdx.x >> 5] = rc; s_c[threadIdx.x >> 5] = cc; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    row_ptr[b + 1] = s_r[0] + s_r[1] + s_r[2] + s_r[3];
-    col_ptr[b + 1] = s_c[0] + s_c[1] + s_c[2] + s_c[3];
-  }
-}
-
-// ---- pass 2: in-place inclusive scan of ptr[1..n], ptr[0] = 0 (one block, 1024 threads;
-// blockIdx.x selects which of the two arrays) ---------------------------------------------
-__global__ void index_scan_kernel(int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_ptr, int n) {
-  int32_t* ptr = blockIdx.x == 0 ? row_ptr : col_ptr;
-  __shared__ int warp_tot[32];
-  __shared__ int carry;
-  if (threadIdx.x == 0) { carry = 0; ptr[0] = 0; }
-  __syncthreads();
-  for (int base = 0; base < n; base += 1024) {
-    const int i = base + threadIdx.x;
-    int v = i < n ? ptr[i + 1] : 0;
-    for (int o = 1; o < 32; o <<= 1) {
-      int t = __shfl_up_sync(0xffffffffu, v, o);
-      if ((threadIdx.x & 31) >= o) v += t;
-    }
-    if ((threadIdx.x & 31) == 31) warp_tot[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      int w = warp_tot[threadIdx.x];
-      for (int o = 1; o < 32; o <<= 1) {
-        int t = __shfl_up_sync(0xffffffffu, w, o);
-        if (threadIdx.x >= o) w += t;
-      }
-      warp_tot[threadIdx.x] = w;
-    }
-    __syncthreads();
-    const int prefix = carry + ((threadIdx.x >> 5) ? warp_tot[(threadIdx.x >> 5) - 1] : 0);
-    if (i < n) ptr[i + 1] = v + prefix;
-    __syncthreads();
-    if (threadIdx.x == 0) carry += warp_tot[31];
-    __syncthreads();
-  }
-}
-
-// ---- pass 3: fill.  grid = nB blocks of 64 threads: warp 0 writes row b (ascending kb),
-// warp 1 writes column b (ascending qb), by ordered ballot compaction. ---------------------
-__global__ void index_fill_kernel(PatternDev p, const int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_idx,
-                                  const int32_t* __restrict__ col_ptr, int32_t* __restrict__ row_idx) {
+// ---- CSR / CSC lists (lg_build_block_index) ---------------------------------------------------
+// grid = nB + 1 blocks of 64 threads: block b writes row_ptr[b], col_ptr[b] (closed forms), and below nB warp 0
+// writes row b (ascending kb) and warp 1 column b (ascending qb), by ordered ballot compaction.
+__global__ void index_fill_kernel(PatternDev p, int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_idx,
+                                  int32_t* __restrict__ col_ptr, int32_t* __restrict__ row_idx) {
   const int b = blockIdx.x;
   const int lane = threadIdx.x & 31;
   const bool is_row = (threadIdx.x >> 5) == 0;
-  int32_t* out = is_row ? col_idx + row_ptr[b] : row_idx + col_ptr[b];
+  const int start = is_row ? row_start(p, b) : col_start(p, b);
+  if (lane == 0) (is_row ? row_ptr : col_ptr)[b] = start;
+  if (b == p.nB) return;
+  int32_t* out = (is_row ? col_idx : row_idx) + start;
   int written = 0;
   for (int base = 0; base < p.nB; base += 32) {
     const int x = base + lane;
@@ -83,208 +32,269 @@ __global__ void index_fill_kernel(PatternDev p, const int32_t* __restrict__ row_
   }
 }
 
-// ---- tile schedules ---------------------------------------------------------------------
-// A tile groups R consecutive pattern rows (or columns).  Its schedule is the ascending
-// union of their lists; entry = idx * 4 + member_mask (bit r set: member r of the tile has
-// the block).  Entries of tile t start at ptr[R * t]; cnt[t] says how many there are.
-// One thread per tile.
-__global__ void tile_merge_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx, int nB, int R,
-                                  int n_tiles, int32_t* __restrict__ tile_cnt, int32_t* __restrict__ tile_ent) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_tiles) return;
-  const int r0 = t * R;
-  int32_t* out = tile_ent + ptr[r0];
-  int n = 0;
-  if (R == 1 || r0 + 1 >= nB) {
-    for (int e = ptr[r0]; e < ptr[r0 + 1]; ++e) out[n++] = idx[e] * 4 + 1;
-  } else {  // R == 2: merge two ascending lists
-    int a = ptr[r0], ae = ptr[r0 + 1], c = ptr[r0 + 1], ce = ptr[r0 + 2];
-    while (a < ae || c < ce) {
-      const int va = a < ae ? idx[a] : 0x7fffffff;
-      const int vc = c < ce ? idx[c] : 0x7fffffff;
-      if (va == vc) { out[n++] = va * 4 + 3; ++a; ++c; }
-      else if (va < vc) { out[n++] = va * 4 + 1; ++a; }
-      else { out[n++] = vc * 4 + 2; ++c; }
-    }
-  }
-  tile_cnt[t] = n;
+// ---- schedules -------------------------------------------------------------------------------
+// Everything the attention kernels walk, in two launches: sched_build_kernel writes the entries of every tile (one
+// warp per tile, straight from the block predicate -- the places come from the closed forms of lg_pattern.h, so
+// nothing has to be counted or scanned first), sched_order_kernel ranks the tiles longest first.
+//   super-tile (forward, 256 query rows = up to 4 pattern rows): ascending kv blocks, kb * 16 + member mask
+//   query tile (dQ pass that recomputes, 128 rows):              ascending kv blocks, kb * 4 + member mask
+//   kv tile (dK/dV pass, R pattern columns):                     ascending query blocks, qb * 4 + member mask
+//   query tile (dQ pass that reads the kept dS):                 ascending kv tiles, see dq_entries below
+// (member bit r: pattern row / column r of the tile has the block).
+
+// A chunk served against a sink + window ring: time-ordered copy of what the ring holds, followed by the chunk,
+// K_lin, V_lin [B, Hkv, kept + T, D].  Row v < kept is the cache slot of position
+//   v                                   (v < sink: the sink never moves)
+//   n_before - (kept - sink) + v - sink (the kept window tokens, oldest first),
+// row v >= kept is chunk token v - kept.
+struct RingCopy {
+  const uint4 *k_cache, *v_cache, *k_chunk, *v_chunk;
+  uint4 *k_lin, *v_lin;
+  int64_t n;                 // 16-byte chunks of K_lin (0: no copy)
+  int row_chunks;            // of a row: D / 8
+  int sink, window, kept, T;
+  int64_t n_before;
+};
+
+struct SchedArgs {
+  PatternDev p;
+  WsHeader* header;          // reset first (null: done by the caller)
+  int R;                     // pattern rows / columns per 128 tokens
+  int n_stiles, st_row0;     // super-tiles, and the pattern row the first one starts at
+  int n_qtiles, n_ktiles;    // 0: no schedule of that kind
+  int keep_ds;               // query tiles: the schedule over the kept dS instead of the recomputing pass's
+  int32_t *sq_off, *sq_cnt, *sq_ent, *sq_order;
+  int32_t *qt_off, *qt_cnt, *qt_ent, *qt_order;
+  int32_t *kt_off, *kt_cnt, *kt_ent, *kt_order, *kt_cols;
+  const int32_t* doc_start;  // with documents and a backward: doc_end[i] is derived for n_doc tokens, L per sequence
+  int32_t* doc_end;
+  int64_t n_doc;
+  int L;
+  RingCopy copy;
+};
+
+// Start of a call that (re)builds the lists: a header that was never initialised is reset, an
+// error word nobody has read yet moves to `latched`, and the fingerprint is withdrawn until the
+// lists are whole again.
+__device__ __forceinline__ void header_begin(WsHeader* h) {
+  if (h->magic != kWsMagic) { h->magic = kWsMagic; h->latched = 0; }
+  else if (h->error_word != 0 && h->latched == 0) h->latched = h->error_word;
+  h->error_word = 0;
+  h->fingerprint = 0;
 }
 
-// The same for tiles of up to four pattern rows (the forward's super-tiles of 256 query rows):
-// entry = idx * 16 + member mask.
-__global__ void tile_merge4_kernel(const int32_t* __restrict__ ptr, const int32_t* __restrict__ idx, int nB, int R,
-                                   int n_tiles, int32_t* __restrict__ tile_cnt, int32_t* __restrict__ tile_ent) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_tiles) return;
-  const int r0 = t * R;
-  int32_t* out = tile_ent + ptr[r0];
-  int cur[4], end[4];
+// oldest block the documents leave to query block qb (see block_active: block kb is dropped when it ends at or
+// before the start of the block's earliest document)
+__device__ __forceinline__ int doc_first_block(const PatternDev& p, int qb) {
+  return p.doc_start ? max(p.doc_start[qb * p.block], 0) / p.block : 0;
+}
+__device__ __forceinline__ bool pattern_active(const PatternDev& p, int qb, int kb) {
+  if (kb > qb) return false;
+  if (p.mode == 0) return true;
+  if (p.mode == 1) return kb < p.ns || qb - kb < p.nw;
+  return qb - kb < p.nl || kb % p.stride == 0;
+}
+
+// The ascending union of the lists of pattern rows r0 .. r0 + n - 1 (n <= 4) as `kb * mul + member mask`; one warp.
+__device__ __forceinline__ int merge_rows(const PatternDev& p, int r0, int n, int mul, int32_t* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  int first[4], lo = 0x7fffffff;
+#pragma unroll
   for (int r = 0; r < 4; ++r) {
-    const bool have = r < R && r0 + r < nB;
-    cur[r] = have ? ptr[r0 + r] : 0;
-    end[r] = have ? ptr[r0 + r + 1] : 0;
+    first[r] = (r < n && r0 + r < p.nB) ? doc_first_block(p, r0 + r) : 0x7fffffff;
+    lo = min(lo, first[r]);
   }
-  int n = 0;
-  for (;;) {
-    int lo = 0x7fffffff;
-    for (int r = 0; r < 4; ++r)
-      if (cur[r] < end[r]) lo = min(lo, idx[cur[r]]);
-    if (lo == 0x7fffffff) break;
+  const int hi = min(r0 + n, p.nB);                     // the youngest row's diagonal
+  const int win0 = p.mode == 1 ? r0 - p.nw + 1 : 0;     // sink + window: nothing between the sink and the oldest row's window
+  int written = 0;
+  for (int base = lo & ~31; base < hi; base += 32) {
+    if (p.mode == 1 && base >= p.ns && base + 32 <= win0) base = win0 & ~31;
+    const int kb = base + lane;
     int mask = 0;
-    for (int r = 0; r < 4; ++r)
-      if (cur[r] < end[r] && idx[cur[r]] == lo) { mask |= 1 << r; ++cur[r]; }
-    out[n++] = lo * 16 + mask;
+    if (kb < hi) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+        if (kb >= first[r] && pattern_active(p, r0 + r, kb)) mask |= 1 << r;   // (first[r] = INT_MAX: no such row)
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, mask != 0);
+    if (mask) out[written + __popc(m & ((1u << lane) - 1))] = kb * mul + mask;
+    written += __popc(m);
   }
-  tile_cnt[t] = n;
+  return written;
 }
 
-// Launch order: tiles with more work first.  order[rank] = tile; rank by (count desc, tile asc).
-__global__ void tile_order_kernel(const int32_t* __restrict__ tile_cnt, int n_tiles, int32_t* __restrict__ order) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_tiles) return;
-  const int c = tile_cnt[t];
-  int rank = 0;
-  for (int u = 0; u < n_tiles; ++u) {
-    const int cu = tile_cnt[u];
-    rank += (cu > c || (cu == c && u < t)) ? 1 : 0;
-  }
-  order[rank] = t;
-}
-
-// ---- kv tiles of the dK/dV pass ------------------------------------------------------------
-// A kv tile holds R pattern columns (R = 128 / block).  With R = 2 the two columns of a tile
-// should have similar lists: a comb column of the strided pattern is attended by every later
-// query block and its neighbour by a handful, so pairing neighbours would leave half of every
-// MMA idle.  Columns are therefore ranked by list length (longest first, ties by index) and
-// consecutive ranks share a tile.  cols[R * t + m] = pattern column of member m (-1: none).
-__global__ void kv_tile_cols_kernel(const int32_t* __restrict__ col_ptr, int nB, int R, int n_tiles,
-                                    int32_t* __restrict__ cols) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c < n_tiles * R && c >= nB) cols[c] = -1;          // padding member of the last tile
-  if (c >= nB) return;
-  if (R == 1) { cols[c] = c; return; }
-  const int len = col_ptr[c + 1] - col_ptr[c];
-  int rank = 0;
-  for (int u = 0; u < nB; ++u) {
-    const int lu = col_ptr[u + 1] - col_ptr[u];
-    rank += (lu > len || (lu == len && u < c)) ? 1 : 0;
-  }
-  cols[rank] = c;
-}
-
-// upper bound of a tile's schedule length, written to off[t + 1] (off[0] = 0) for the scan
-__global__ void kv_tile_len_kernel(const int32_t* __restrict__ col_ptr, const int32_t* __restrict__ cols, int R,
-                                   int n_tiles, int32_t* __restrict__ off) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_tiles) return;
-  int n = 0;
-  for (int m = 0; m < R; ++m) {
-    const int c = cols[R * t + m];
-    if (c >= 0) n += col_ptr[c + 1] - col_ptr[c];
-  }
-  off[t + 1] = n;
-  if (t == 0) off[0] = 0;
-}
-
-// ascending union of the members' CSC lists; entry = query block * 4 + member mask
-__global__ void kv_tile_merge_kernel(const int32_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
-                                     const int32_t* __restrict__ cols, const int32_t* __restrict__ off, int R,
-                                     int n_tiles, int32_t* __restrict__ tile_cnt, int32_t* __restrict__ tile_ent) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_tiles) return;
-  int32_t* out = tile_ent + off[t];
-  const int ca = cols[R * t], cb = (R == 2) ? cols[R * t + 1] : -1;
-  int a = ca >= 0 ? col_ptr[ca] : 0, ae = ca >= 0 ? col_ptr[ca + 1] : 0;
-  int c = cb >= 0 ? col_ptr[cb] : 0, ce = cb >= 0 ? col_ptr[cb + 1] : 0;
-  int n = 0;
-  while (a < ae || c < ce) {
-    const int va = a < ae ? row_idx[a] : 0x7fffffff;
-    const int vc = c < ce ? row_idx[c] : 0x7fffffff;
-    if (va == vc) { out[n++] = va * 4 + 3; ++a; ++c; }
-    else if (va < vc) { out[n++] = va * 4 + 1; ++a; }
-    else { out[n++] = vc * 4 + 2; ++c; }
-  }
-  tile_cnt[t] = n;
-}
-
-// tile_of[kb] = kv tile of pattern column kb
-__global__ void kv_tile_of_kernel(const int32_t* __restrict__ cols, int R, int n_tiles, int32_t* __restrict__ tile_of) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= n_tiles * R) return;
-  const int kb = cols[c];
-  if (kb >= 0) tile_of[kb] = c / R;
-}
-
-// ---- schedule of the dQ pass that reads the kept dS tiles -------------------------------------
-// The dK/dV pass leaves one dS tile per block of the pattern and 64-row half of its query block, numbered by
-// the block's position p in the column lists (col_ptr[c] + rank of the query block in column c):
-// 128-token blocks: tiles 2 p and 2 p + 1 (128 keys x 64 queries each); 64-token blocks: tile p (64 keys x
-// 64 queries).  A query tile of 128 rows needs, for every kv tile T with an active column in the row(s) of
-// its query block(s), the four quarters (64-row half m, 64-key half n) of its 128 x 128 product; entry =
+// Entries of query tile t for the dQ pass that reads the kept dS tiles.  The dK/dV pass leaves one dS tile per
+// block of the pattern and 64-row half of its query block, numbered by the block's position p in the column
+// lists (col_pos): 128-token blocks: tiles 2 p and 2 p + 1 (128 keys x 64 queries each); 64-token blocks: tile p
+// (64 keys x 64 queries).  A query tile of 128 rows needs, for every kv tile T with an active column in the row(s)
+// of its query block(s), the four quarters (64-row half m, 64-key half n) of its 128 x 128 product; entry =
 // (T, tile of (m, n) at 1 + 2 n + m), -1 where the pattern has no block (that quarter of dS is zero).  With
-// 128-token blocks only n = 0 is used: the tiles of the two halves.  One thread per query tile; entries at
-// dq_ent[kDqEntInts * (row_ptr[R t] + i)], kv tiles ascending.
-__global__ void dq_sched_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
-                                const int32_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
-                                const int32_t* __restrict__ tile_of, const int32_t* __restrict__ cols, int R, int nB,
-                                int n_qtiles, int32_t* __restrict__ dq_cnt, int32_t* __restrict__ dq_ent) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n_qtiles) return;
+// 128-token blocks only n = 0 is used: the tiles of the two halves.  One warp, kv tiles ascending.
+__device__ __forceinline__ int dq_entries(const PatternDev& p, int R, int n_ktiles, int t, int32_t* __restrict__ out) {
   constexpr int E = kDqEntInts;
-  int32_t* out = dq_ent + E * static_cast<int64_t>(row_ptr[R * t]);
-  int n = 0;
-  for (int m = 0; m < R; ++m) {          // distinct kv tiles of the tile's query blocks, kept ascending
-    const int qb = R * t + m;
-    if (qb >= nB) break;
-    for (int x = row_ptr[qb]; x < row_ptr[qb + 1]; ++x) {
-      const int T = tile_of[col_idx[x]];
-      int pos = 0;
-      while (pos < n && out[E * pos] < T) ++pos;
-      if (pos < n && out[E * pos] == T) continue;
-      for (int y = n; y > pos; --y) out[E * y] = out[E * (y - 1)];
-      out[E * pos] = T;
-      ++n;
+  const int lane = threadIdx.x & 31;
+  int first[2];
+#pragma unroll
+  for (int m = 0; m < 2; ++m) first[m] = (m < R && R * t + m < p.nB) ? doc_first_block(p, R * t + m) : 0x7fffffff;
+  const bool in_order = R == 1 || n_long_cols(p) == 0;   // tile T holds columns R T, R T + 1
+  const int lo = in_order ? min(first[0], first[1]) / R : 0, hi = in_order ? min(t + 1, n_ktiles) : n_ktiles;
+  int written = 0;
+  for (int base = lo & ~31; base < hi; base += 32) {
+    const int T = base + lane;
+    int q[4] = {-1, -1, -1, -1};
+    bool any = false;
+    if (T < hi) {
+#pragma unroll
+      for (int n = 0; n < 2; ++n) {
+        if (n >= R || R * T + n >= p.nB) continue;
+        const int c = kv_col(p, R, R * T + n);
+#pragma unroll
+        for (int m = 0; m < 2; ++m) {
+          const int qb = R * t + m;
+          if (m >= R || c < first[m] || !pattern_active(p, qb, c)) continue;   // (first[m] = INT_MAX: no such row)
+          q[2 * n + m] = col_pos(p, qb, c);
+          any = true;
+        }
+      }
+      if (R == 1 && any) { q[1] = 2 * q[0] + 1; q[0] = 2 * q[0]; }
     }
+    const unsigned m = __ballot_sync(0xffffffffu, any);
+    if (any) {
+      int32_t* e = out + E * (written + __popc(m & ((1u << lane) - 1)));
+      e[0] = T;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) e[1 + i] = q[i];
+    }
+    written += __popc(m);
   }
-  auto find = [&](int c, int qb) {       // position of block (row qb, column c) in the column lists, or -1
-    if (c < 0 || qb >= nB) return -1;
-    int lo = col_ptr[c], hi = col_ptr[c + 1];
-    const int end = hi;
-    while (lo < hi) {
-      const int mid = (lo + hi) >> 1;
-      if (row_idx[mid] < qb) lo = mid + 1; else hi = mid;
-    }
-    return (lo < end && row_idx[lo] == qb) ? lo : -1;
-  };
-  for (int i = 0; i < n; ++i) {
-    const int T = out[E * i];
-    if (R == 1) {
-      const int p = find(cols[T], t);
-      out[E * i + 1] = p >= 0 ? 2 * p : -1;
-      out[E * i + 2] = p >= 0 ? 2 * p + 1 : -1;
-      out[E * i + 3] = out[E * i + 4] = -1;
-    } else {
-      for (int nn = 0; nn < 2; ++nn)
-        for (int m = 0; m < 2; ++m) out[E * i + 1 + 2 * nn + m] = find(cols[2 * T + nn], 2 * t + m);
-    }
-  }
-  dq_cnt[t] = n;
+  return written;
 }
 
-// doc_end[b][j] = end (one past the last token) of the document token j belongs to, from
-// doc_start[b][i] = first token of token i's document (non-decreasing): the first i > j whose
-// document starts after j, found by bisection, or L.
-__global__ void doc_end_kernel(const int32_t* __restrict__ doc_start, int32_t* __restrict__ doc_end, int B, int L) {
-  const int64_t gid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (gid >= static_cast<int64_t>(B) * L) return;
-  const int j = static_cast<int>(gid % L);
-  const int32_t* ds = doc_start + (gid - j);
+// The ascending union of the lists of a kv tile's columns as `qb * 4 + member mask`; one warp.
+__device__ __forceinline__ int merge_cols(const PatternDev& p, int ca, int cb, int32_t* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const int lo = cb >= 0 ? min(ca, cb) : ca;
+  int hi = ca + col_len(p, ca);
+  if (cb >= 0) hi = max(hi, cb + col_len(p, cb));
+  int written = 0;
+  for (int base = lo & ~31; base < hi; base += 32) {
+    const int qb = base + lane;
+    int mask = 0;
+    if (qb < hi) {
+      const int first = doc_first_block(p, qb);
+      if (ca >= first && pattern_active(p, qb, ca)) mask |= 1;
+      if (cb >= first && cb >= 0 && pattern_active(p, qb, cb)) mask |= 2;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, mask != 0);
+    if (mask) out[written + __popc(m & ((1u << lane) - 1))] = qb * 4 + mask;
+    written += __popc(m);
+  }
+  return written;
+}
+
+// end (one past the last token) of the document token j belongs to, from doc_start[i] = first token of token i's
+// document (non-decreasing): the first i > j whose document starts after j, found by bisection, or L.
+__device__ __forceinline__ int doc_end_of(const int32_t* __restrict__ ds, int j, int L) {
   int lo = j, hi = L;            // ds[lo] <= j (its own document); ds[hi] > j, with ds[L] taken as +inf
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
     if (ds[mid] > j) hi = mid; else lo = mid;
   }
-  doc_end[gid] = hi;
+  return hi;
+}
+
+// one 16-byte chunk of K and of V
+__device__ __forceinline__ void ring_linearise(const RingCopy& r, int64_t i) {
+  const int Lc = r.kept + r.T;
+  const int c = static_cast<int>(i % r.row_chunks), v = static_cast<int>((i / r.row_chunks) % Lc);
+  const int64_t bh = i / (static_cast<int64_t>(r.row_chunks) * Lc);
+  if (v < r.kept) {
+    const int64_t pos = v < r.sink ? v : r.n_before - (r.kept - r.sink) + (v - r.sink);
+    const int64_t slot = pos < r.sink ? pos : r.sink + (pos - r.sink) % r.window;
+    const int64_t off = (bh * (r.sink + r.window) + slot) * r.row_chunks + c;
+    r.k_lin[i] = r.k_cache[off];
+    r.v_lin[i] = r.v_cache[off];
+  } else {
+    const int64_t off = (bh * r.T + (v - r.kept)) * r.row_chunks + c;
+    r.k_lin[i] = r.k_chunk[off];
+    r.v_lin[i] = r.v_chunk[off];
+  }
+}
+
+constexpr int kSchedThreads = 256;   // warps are independent of one another
+
+// Latency-bound integer work: a warp per tile looks at 32 blocks at a time (the one-thread-per-tile merges this
+// replaces took 30 us of a 520 us chunk call and 260 us of a 4.8 ms step over packed documents).
+__global__ void __launch_bounds__(kSchedThreads) sched_build_kernel(const SchedArgs a) {
+  if (blockIdx.x == 0 && threadIdx.x == 0 && a.header) header_begin(a.header);
+  const int lane = threadIdx.x & 31;
+  int64_t w = static_cast<int64_t>(blockIdx.x) * (kSchedThreads / 32) + (threadIdx.x >> 5);
+  if (w < a.n_stiles) {
+    const int t = static_cast<int>(w), r0 = a.st_row0 + 2 * a.R * t;
+    const int off = row_start(a.p, r0) - row_start(a.p, a.st_row0);
+    const int n = merge_rows(a.p, r0, 2 * a.R, 16, a.sq_ent + off);
+    if (lane == 0) { a.sq_off[t] = off; a.sq_cnt[t] = n; }
+    return;
+  }
+  w -= a.n_stiles;
+  if (w < a.n_qtiles) {
+    const int t = static_cast<int>(w), off = row_start(a.p, a.R * t);
+    const int n = a.keep_ds ? dq_entries(a.p, a.R, a.n_ktiles, t, a.qt_ent + static_cast<int64_t>(kDqEntInts) * off)
+                            : merge_rows(a.p, a.R * t, a.R, 4, a.qt_ent + off);
+    if (lane == 0) { a.qt_off[t] = off; a.qt_cnt[t] = n; }
+    return;
+  }
+  w -= a.n_qtiles;
+  if (w < a.n_ktiles) {
+    const int t = static_cast<int>(w), k = a.R * t, off = kv_start(a.p, a.R, k);
+    const int ca = kv_col(a.p, a.R, k), cb = (a.R == 2 && k + 1 < a.p.nB) ? kv_col(a.p, a.R, k + 1) : -1;   // -1: no second column
+    const int n = merge_cols(a.p, ca, cb, a.kt_ent + off);
+    if (lane == 0) {
+      a.kt_off[t] = off; a.kt_cnt[t] = n;
+      a.kt_cols[a.R * t] = ca;
+      if (a.R == 2) a.kt_cols[2 * t + 1] = cb;
+    }
+    return;
+  }
+  w -= a.n_ktiles;
+  int64_t i = w * 32 + lane;
+  if (i < a.n_doc) {
+    const int j = static_cast<int>(i % a.L);
+    a.doc_end[i] = doc_end_of(a.doc_start + (i - j), j, a.L);
+    return;
+  }
+  i -= (a.n_doc + 31) / 32 * 32;
+  if (i >= 0 && i < a.copy.n) ring_linearise(a.copy, i);   // (a few schedule warps beside a copy: one launch for both)
+}
+
+// rank of tile t by (count descending, tile ascending); one warp
+__device__ __forceinline__ int rank_of(const int32_t* __restrict__ cnt, int n, int t) {
+  const int c = cnt[t];
+  int rank = 0;
+  for (int u = threadIdx.x & 31; u < n; u += 32) {
+    const int cu = cnt[u];
+    rank += (cu > c || (cu == c && u < t)) ? 1 : 0;
+  }
+  return __reduce_add_sync(0xffffffffu, rank);
+}
+
+// Launch order: tiles with more work first (order[rank] = tile).  The last launch of a build: the header gets the
+// fingerprint the lists are known by (0: none).
+__global__ void __launch_bounds__(kSchedThreads) sched_order_kernel(const SchedArgs a, unsigned long long fp) {
+  if (blockIdx.x == 0 && threadIdx.x == 0 && fp != 0) a.header->fingerprint = fp;
+  int w = blockIdx.x * (kSchedThreads / 32) + (threadIdx.x >> 5);
+  const int32_t* cnt[3] = {a.sq_cnt, a.qt_cnt, a.kt_cnt};
+  int32_t* order[3] = {a.sq_order, a.qt_order, a.kt_order};
+  const int n[3] = {a.n_stiles, a.n_qtiles, a.n_ktiles};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    if (w < n[i]) {
+      const int rank = rank_of(cnt[i], n[i], w);
+      if ((threadIdx.x & 31) == 0) order[i][rank] = w;
+      return;
+    }
+    w -= n[i];
+  }
 }
 
 }  // namespace lg
