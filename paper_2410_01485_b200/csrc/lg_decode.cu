@@ -37,7 +37,7 @@ struct DecodeArgs {
   const __nv_bfloat16* k_cache;  // [B, Hkv, C, D]
   const __nv_bfloat16* v_cache;
   const int64_t* n_tokens;       // [B]
-  float* part;                   // [B, Hkv*HG, nsplit, 8 heads, (D + 2)] : O, m, l
+  float* part;                   // records: O of 8 heads [8][D], then their (m, l) pairs [8][2]
   __nv_bfloat16* o;              // [B, Hq, D]
   float* lse;                    // [B, Hq] or null
   int Hq, Hkv, G, HG, C, nsplit;
@@ -279,8 +279,8 @@ __device__ __forceinline__ void decode_run_segment(const DecodeArgs& a, uint8_t*
         if (d == 0 && a.lse) a.lse[qh] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
       }
     } else {
-      out[head * kRec + d] = acc;
-      if (d == 0) { out[head * kRec + D] = m; out[head * kRec + D + 1] = l; }
+      out[idx] = acc;
+      if (d == 0) { out[kDecHeads * D + 2 * head] = m; out[kDecHeads * D + 2 * head + 1] = l; }
     }
   }
 }
@@ -317,15 +317,18 @@ __device__ __forceinline__ int decode_tiles_of(const DecodeArgs& a, int b) {
   return (nvalid + kDecTile - 1) / kDecTile;
 }
 
-// cum[b] = tiles of the sequences before b, b = 0 .. B (block of kDecThreads threads; ends with a barrier)
-__device__ __forceinline__ void decode_build_cum(const DecodeArgs& a, int* cum) {
+// cum[b] = tiles of the sequences before b, b = 0 .. B (block of kDecThreads threads; ends with a barrier).
+// Returns whether some sequence holds no token.
+__device__ __forceinline__ bool decode_build_cum(const DecodeArgs& a, int* cum) {
   __shared__ int warp_sum[kDecWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ipt = (a.B + kDecThreads - 1) / kDecThreads;
   const int b0 = tid * ipt;
-  int local = 0;
-  for (int i = 0; i < ipt; ++i)
-    if (b0 + i < a.B) local += decode_tiles_of(a, b0 + i);
+  const int first = b0 < a.B ? decode_tiles_of(a, b0) : 0;   // usually all of the thread's sequences
+  int local = first;
+  bool empty = b0 < a.B && first == 0;
+  for (int i = 1; i < ipt; ++i)
+    if (b0 + i < a.B) { const int n = decode_tiles_of(a, b0 + i); local += n; empty |= n == 0; }
   int incl = local;
   for (int o = 1; o < 32; o <<= 1) {
     const int t = __shfl_up_sync(0xffffffffu, incl, o);
@@ -334,67 +337,83 @@ __device__ __forceinline__ void decode_build_cum(const DecodeArgs& a, int* cum) 
   if (lane == 31) warp_sum[warp] = incl;
   __syncthreads();
   int run = incl - local;
-  for (int w = 0; w < warp; ++w) run += warp_sum[w];
-  for (int i = 0; i < ipt; ++i)
-    if (b0 + i < a.B) { cum[b0 + i] = run; run += decode_tiles_of(a, b0 + i); }
+#pragma unroll
+  for (int w = 0; w < kDecWarps; ++w) run += w < warp ? warp_sum[w] : 0;
+  if (b0 < a.B) {
+    cum[b0] = run;
+    run += first;
+    for (int i = 1; i < ipt; ++i)
+      if (b0 + i < a.B) { cum[b0 + i] = run; run += decode_tiles_of(a, b0 + i); }
+  }
   if (tid == kDecThreads - 1) cum[a.B] = run;   // the last thread's running total is the grand total
-  __syncthreads();
+  return __syncthreads_or(empty) != 0;
 }
 
-// Merge the records of unit (b, k): CTAs first_cta .. first_cta + n_rec - 1, in that order
-// (whichever CTA happens to run this, the summation order is the same).  kDecThreads threads.
+// Merge the records of unit (b, k): CTAs first_cta .. first_cta + n_rec - 1, in that order (whichever CTA happens
+// to run this, the summation order is the same).  kDecThreads threads; `scratch`: shared memory, 8 (n_rec + 1)
+// pairs of floats.  The records sit in L2, so what this takes is round trips: one for all (max, sum) pairs, one
+// for eight records' values at a time (read record by record it was a chain of 2 n_rec dependent round trips:
+// one sequence of 8 kv heads, 16 records a unit, 24.5 -> 12.2 us for the kernel).
 template <int D>
-__device__ __forceinline__ void decode_merge_unit(const DecodeArgs& a, int b, int k, int64_t u, int first_cta,
+__device__ __forceinline__ void decode_merge_unit(const DecodeArgs& a, float* scratch, int b, int k, int64_t u, int first_cta,
                                                   int n_rec, int64_t total, int n_cta) {
   constexpr int kRec = D + 2;
-  const int kvh = k / a.HG, hg = k % a.HG;
+  static_assert(kDecWarps == kDecHeads, "a warp per head");
+  const int kvh = k / a.HG, hg = k % a.HG, tid = threadIdx.x, lane = tid & 31;
   const float* recs = a.part + (static_cast<int64_t>(first_cta) + u) * (kDecHeads * kRec);
   // a CTA with an empty slice (possible only with fewer tiles than CTAs) wrote no record
   const bool sparse_slices = total < n_cta;
-  auto empty_slice = [&](int c) { return total * c / n_cta == total * (c + 1) / n_cta; };
-  // Each thread owns kOut outputs (all handled together so that the loads of one record are in
-  // flight at once: the records sit in L2 and a dependent chain of loads would dominate).
-  constexpr int kOut = kDecHeads * D / kDecThreads;
-  int head[kOut], dd[kOut];
-  float m[kOut], acc[kOut], l[kOut];
-#pragma unroll
-  for (int j = 0; j < kOut; ++j) {
-    const int idx = threadIdx.x + j * kDecThreads;
-    head[j] = idx / D;
-    dd[j] = idx % D;
-    m[j] = -INFINITY;
-    acc[j] = 0.f;
-    l[j] = 0.f;
+  auto absent = [&](int c) { return sparse_slices && total * c / n_cta == total * (c + 1) / n_cta; };
+  float2* ml = reinterpret_cast<float2*>(scratch);           // [n_rec][8]: (max, sum), then x becomes the record's weight
+  __syncthreads();                                           // scratch: whoever used this shared memory is done
+  for (int e = tid; e < n_rec * kDecHeads; e += kDecThreads) {
+    const int i = e / kDecHeads;
+    ml[e] = absent(first_cta + i) ? make_float2(-INFINITY, 0.f)
+                                  : __ldcg(reinterpret_cast<const float2*>(recs + static_cast<int64_t>(i) * (kDecHeads * kRec) +
+                                                                           kDecHeads * D) + e % kDecHeads);
   }
-  for (int i = 0; i < n_rec; ++i) {
-    if (sparse_slices && empty_slice(first_cta + i)) continue;
+  __syncthreads();
+  {
+    const int head = tid >> 5;
+    float m = -INFINITY, l = 0.f;
+    for (int i = lane; i < n_rec; i += 32) m = fmaxf(m, ml[i * kDecHeads + head].x);
 #pragma unroll
-    for (int j = 0; j < kOut; ++j) m[j] = fmaxf(m[j], __ldcg(recs + (i * kDecHeads + head[j]) * kRec + D));
-  }
-  for (int i = 0; i < n_rec; ++i) {
-    if (sparse_slices && empty_slice(first_cta + i)) continue;
-    float rm[kOut], rl[kOut], ro[kOut];
-#pragma unroll
-    for (int j = 0; j < kOut; ++j) {
-      const float* rec = recs + (i * kDecHeads + head[j]) * kRec;
-      rm[j] = __ldcg(rec + D);
-      rl[j] = __ldcg(rec + D + 1);
-      ro[j] = __ldcg(rec + dd[j]);
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    const float mu = m == -INFINITY ? 0.f : m;
+    for (int i = lane; i < n_rec; i += 32) {
+      const float f = fast_exp2(ml[i * kDecHeads + head].x - mu);
+      l += f * ml[i * kDecHeads + head].y;
+      ml[i * kDecHeads + head].x = f;
     }
 #pragma unroll
-    for (int j = 0; j < kOut; ++j) {
-      const float f = fast_exp2(rm[j] - (m[j] == -INFINITY ? 0.f : m[j]));
-      acc[j] += f * ro[j];
-      l[j] += f * rl[j];
-    }
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) ml[n_rec * kDecHeads + head] = make_float2(m, l);
   }
+  __syncthreads();
+  for (int idx = tid * 4; idx < kDecHeads * D; idx += kDecThreads * 4) {   // four values of one head
+    const int head = idx / D, gh = hg * kDecHeads + head;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i0 = 0; i0 < n_rec; i0 += 8) {
+      float4 r[8];
 #pragma unroll
-  for (int j = 0; j < kOut; ++j) {
-    const int gh = hg * kDecHeads + head[j];
+      for (int x = 0; x < 8; ++x)
+        r[x] = (i0 + x < n_rec && !absent(first_cta + i0 + x))
+                   ? __ldcg(reinterpret_cast<const float4*>(recs + static_cast<int64_t>(i0 + x) * (kDecHeads * kRec) + idx))
+                   : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        const float f = i0 + x < n_rec ? ml[(i0 + x) * kDecHeads + head].x : 0.f;
+        acc.x += f * r[x].x; acc.y += f * r[x].y; acc.z += f * r[x].z; acc.w += f * r[x].w;
+      }
+    }
     if (gh >= a.G) continue;
+    const float m = ml[n_rec * kDecHeads + head].x, l = ml[n_rec * kDecHeads + head].y;
     const int64_t qh = static_cast<int64_t>(b) * a.Hq + kvh * a.G + gh;
-    a.o[qh * D + dd[j]] = __float2bfloat16(l[j] > 0.f ? acc[j] / l[j] : 0.f);
-    if (dd[j] == 0 && a.lse) a.lse[qh] = l[j] > 0.f ? (m[j] + log2f(l[j])) * 0.6931471805599453f : -INFINITY;
+    uint2 out;
+    out.x = l > 0.f ? pack_bf16(acc.x / l, acc.y / l) : 0u;
+    out.y = l > 0.f ? pack_bf16(acc.z / l, acc.w / l) : 0u;
+    *reinterpret_cast<uint2*>(a.o + qh * D + idx % D) = out;
+    if (idx % D == 0 && a.lse) a.lse[qh] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
   }
 }
 
@@ -404,7 +423,11 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
   constexpr int kPipeBytes = kDecWarps * kDecStages * 2 * kDecTile * D * 2;
   constexpr int kRec = D + 2;
   int* cum = reinterpret_cast<int*>(dsmem + kPipeBytes);
-  decode_build_cum(a, cum);
+  // overlapped with the kernel before (an append, or the decode of the step before): append + decode of 16 sequences
+  // over 4224 slots, 64 / 8 heads, 54.9 -> 48.7 us a step, of one sequence 28.7 -> 13.7 us with the merge below
+  pdl_trigger();
+  pdl_wait();
+  const bool any_empty = decode_build_cum(a, cum);
   const int ups = a.Hkv * a.HG;
   const int64_t total = static_cast<int64_t>(cum[a.B]) * ups;
   __shared__ int s_merge[3];
@@ -416,11 +439,11 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
     return static_cast<int>(c);
   };
   // units of sequences without tokens get their (empty) result here, spread over the CTAs
-  for (int e = 0; e < a.B; ++e) {
+  for (int e = 0; any_empty && e < a.B; ++e) {
     if (cum[e + 1] != cum[e]) continue;
     for (int k = 0; k < ups; ++k) {
       const int64_t u = static_cast<int64_t>(e) * ups + k;
-      if (u % gridDim.x == blockIdx.x) decode_merge_unit<D>(a, e, k, u, 0, 0, total, gridDim.x);
+      if (u % gridDim.x == blockIdx.x) decode_merge_unit<D>(a, reinterpret_cast<float*>(dsmem), e, k, u, 0, 0, total, gridDim.x);
     }
   }
   const int64_t f0 = start_of(blockIdx.x), f1 = start_of(blockIdx.x + 1);
@@ -469,7 +492,7 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
     __syncthreads();
     if (s_merge[0]) {
       __threadfence();
-      decode_merge_unit<D>(a, b, k, u, s_merge[1], s_merge[2], total, gridDim.x);
+      decode_merge_unit<D>(a, reinterpret_cast<float*>(dsmem), b, k, u, s_merge[1], s_merge[2], total, gridDim.x);
       if (threadIdx.x == 0) a.unit_count[u] = 0u;
     }
   }
@@ -486,14 +509,15 @@ __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeArgs a) {
     const int head = idx / D, d = idx % D;
     const int gh = hg * kDecHeads + head;
     if (gh >= a.G) continue;
+    const float* ml = part + kDecHeads * D + 2 * head;
     float m = -INFINITY;
-    for (int s = 0; s < a.nsplit; ++s) m = fmaxf(m, part[(s * kDecHeads + head) * kRec + D]);
+    for (int s = 0; s < a.nsplit; ++s) m = fmaxf(m, ml[s * kDecHeads * kRec]);
     const float mu = m == -INFINITY ? 0.f : m;
     float acc = 0.f, l = 0.f;
     for (int s = 0; s < a.nsplit; ++s) {
-      const float f = fast_exp2(part[(s * kDecHeads + head) * kRec + D] - mu);
-      acc += f * part[(s * kDecHeads + head) * kRec + d];
-      l += f * part[(s * kDecHeads + head) * kRec + D + 1];
+      const float f = fast_exp2(ml[s * kDecHeads * kRec] - mu);
+      acc += f * part[s * kDecHeads * kRec + idx];
+      l += f * ml[s * kDecHeads * kRec + 1];
     }
     const int64_t qh = static_cast<int64_t>(b) * a.Hq + kvh * a.G + gh;
     a.o[qh * D + d] = __float2bfloat16(l > 0.f ? acc / l : 0.f);
@@ -508,6 +532,7 @@ __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeArgs a) {
 __global__ void ring_append_kernel(__nv_bfloat16* k_cache, __nv_bfloat16* v_cache, const __nv_bfloat16* k_new,
                                    const __nv_bfloat16* v_new, const int64_t* n_before, int B, int Hkv, int D, int T,
                                    int sink, int window) {
+  pdl_trigger();
   const int per_row = D / 8;
   const int64_t gid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   const int64_t row_id = gid / per_row;
@@ -517,6 +542,7 @@ __global__ void ring_append_kernel(__nv_bfloat16* k_cache, __nv_bfloat16* v_cach
   const int t = static_cast<int>(row_id % T);
   const int64_t bh = row_id / T;
   const int b = static_cast<int>(bh / Hkv);
+  pdl_wait();
   const int64_t n0 = n_before[b];
   if (n0 < 0) return;                                  // a negative count addresses nothing: the sequence is skipped
   const int64_t j = n0 + t, last = n0 + T - 1;
@@ -623,11 +649,10 @@ lg_status lg_kv_ring_append(const lg_decode_params* p, void* k_cache, void* v_ca
   const int64_t threads = static_cast<int64_t>(p->B) * p->Hkv * T_new * (p->D / 8);
   const int64_t blocks = (threads + 255) / 256;
   if (blocks > 0x7fffffff) return LG_ERR_UNSUPPORTED;
-  ring_append_kernel<<<static_cast<unsigned>(blocks), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-      static_cast<__nv_bfloat16*>(k_cache), static_cast<__nv_bfloat16*>(v_cache),
-      static_cast<const __nv_bfloat16*>(k_new), static_cast<const __nv_bfloat16*>(v_new), n_tokens_before, p->B,
-      p->Hkv, p->D, T_new, p->sink_tokens, p->window_tokens); note_launch();
-  return cudaGetLastError() == cudaSuccess ? LG_OK : LG_ERR_CUDA;
+  return launch_overlapped(ring_append_kernel, dim3(static_cast<unsigned>(blocks)), 256, 0, static_cast<cudaStream_t>(stream),
+                           static_cast<__nv_bfloat16*>(k_cache), static_cast<__nv_bfloat16*>(v_cache),
+                           static_cast<const __nv_bfloat16*>(k_new), static_cast<const __nv_bfloat16*>(v_new), n_tokens_before,
+                           p->B, p->Hkv, p->D, T_new, p->sink_tokens, p->window_tokens) == cudaSuccess ? LG_OK : LG_ERR_CUDA;
 }
 
 size_t lg_sparse_decode_workspace_bytes(const lg_decode_params* p) {
@@ -703,12 +728,8 @@ lg_status lg_sparse_decode(const lg_decode_params* p, const void* q, const void*
     a.unit_count = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(workspace) + sizeof(WsHeader));
     a.part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + sizeof(WsHeader) + count_bytes);
     const int smem_flat = kDecWarps * kDecStages * 2 * kDecTile * p->D * 2 + (p->B + 1) * static_cast<int>(sizeof(int));
-    if (p->D == 128) {
-      decode_stream_kernel<128><<<static_cast<unsigned>(n_cta), kDecWarps * 32, smem_flat, st>>>(a); note_launch();
-    } else {
-      decode_stream_kernel<64><<<static_cast<unsigned>(n_cta), kDecWarps * 32, smem_flat, st>>>(a); note_launch();
-    }
-    return cudaGetLastError() == cudaSuccess ? LG_OK : LG_ERR_CUDA;
+    return launch_overlapped(p->D == 128 ? decode_stream_kernel<128> : decode_stream_kernel<64>, dim3(static_cast<unsigned>(n_cta)),
+                             kDecWarps * 32, smem_flat, st, a) == cudaSuccess ? LG_OK : LG_ERR_CUDA;
   }
   if (a.Hkv * a.HG > 65535 || p->B > 65535) return LG_ERR_UNSUPPORTED;
   if (cudaMemsetAsync(workspace, 0, sizeof(WsHeader), st) != cudaSuccess) return LG_ERR_CUDA;

@@ -32,6 +32,21 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // lg_debug_kernel_launches); nothing in the library depends on it.
 void note_launch();
 
+// Launch of a kernel that calls pdl_wait() (lg_common.cuh) before it touches global memory: it may start while the
+// kernel before it on the stream drains.
+template <typename... Params, typename... Args>
+inline cudaError_t launch_overlapped(void (*kern)(Params...), dim3 grid, int block, int smem, cudaStream_t stream, Args&&... args) {
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
+  note_launch();
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+}
+
 struct Resolved {          // validated, defaulted copy of lg_attn_params
   int B, Hq, Hkv, L, D, block, mode, G;
   PatternDev pat;
