@@ -365,6 +365,11 @@ __device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
 }
+// bits lo .. hi - 1 (0 <= lo, hi <= 32; none when hi <= lo): a mask whose bits are tested at compile-time places costs
+// a fraction of an instruction per element (they reach the predicates several at a time), a pair of compares two
+__device__ __forceinline__ uint32_t bit_range(int lo, int hi) {
+  return hi <= lo ? 0u : (0xffffffffu << lo) & (0xffffffffu >> (32 - hi));
+}
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));

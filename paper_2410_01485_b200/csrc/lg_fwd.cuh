@@ -10,11 +10,16 @@
 //   warp 8          : TMA producer (Q once, then the K and V rings)
 //   warps 9 / 10    : issue the tcgen05.mma of slot 0 / 1 (warp-uniform code, one elected lane;
 //                     the two warps sit on different scheduler partitions of the SM)
-// Tensor memory: S of slot s, half h at columns 128 s + 64 h (P is written as bf16 over the
+// Tensor memory, D = 128: S of slot s, half h at columns 128 s + 64 h (P is written as bf16 over the
 // first 32 of them), O of slot s at 256 + 128 s.  Per slot the issue order is
 //   S_0(0) S_1(0) | PV_0(0) S_0(1) | PV_1(0) S_1(1) | PV_0(1) S_0(2) | ...
 // so the two halves of a slot form a double buffer: while the softmax works on one half the
-// tensor pipe computes the other, and the second slot fills what is left.  The online softmax
+// tensor pipe computes the other, and the second slot fills what is left.
+// D = 64: the products of a half take 320 cycles of the tensor pipe where its exponentials take 512 of
+// the exponential unit, so the element-wise chain sets the pace, and what fills the unit is more rows in
+// work.  Two CTAs share an SM: each has half the tensor memory, one score buffer per slot (S of slot s at
+// 64 s, O at 128 + 64 s; S(0) | PV(0) S(1) | PV(1) S(2) | ...) and 80 registers per thread, hence the half
+// is worked 32 columns at a time (3 x 16 / 4 heads x 6001 tokens, window 1024: 169 -> 150 us).  The online softmax
 // advances half by half.  A row's reference (the maximum its probabilities are expressed relative
 // to) only moves, and O is only rescaled, when a half's probabilities sum to more than 2^8;
 // until then they are relative to the older reference, which fp32 / bf16 hold easily, and the
@@ -53,6 +58,8 @@ struct FwdArgs {
 constexpr int kFwdTmaWarp = 8, kFwdMmaWarp0 = 9;
 constexpr int kFwdThreads = 11 * 32;
 constexpr float kFwdMaxProb = 256.0f;   // a half's probabilities may grow to this (relative to the row's reference) before the reference moves
+template <int D> constexpr int kFwdBufs = D == 64 ? 1 : 2;        // score buffers per slot
+template <int D> constexpr int kFwdCtasPerSm = D == 64 ? 2 : 1;
 template <int D>
 struct FwdSmem {
   static constexpr int kBox = 128 * 128;               // one 64-column box of 128 rows
@@ -66,7 +73,7 @@ struct FwdSmem {
 };
 
 template <int D, int BS>
-__global__ void __launch_bounds__(kFwdThreads, 1)
+__global__ void __launch_bounds__(kFwdThreads, kFwdCtasPerSm<D>)
 fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
            const __grid_constant__ CUtensorMap tm_v, const FwdArgs a) {
   using SM = FwdSmem<D>;
@@ -74,8 +81,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   constexpr int RS = R4 / 2;                    // pattern rows per slot
   constexpr uint32_t kSlotMask = (1u << RS) - 1u;
   constexpr int kTile = SM::kTile;
-  constexpr uint32_t kColS = 0, kColO = 256;
-  // SF / PF / OD are indexed [slot * 2 + half].  A parity wait is only meaningful while the barrier
+  constexpr int NB = kFwdBufs<D>;
+  constexpr uint32_t kColS = 0, kSlotS = 64 * NB, kColO = 2 * kSlotS, kTmemCols = kColO + 2 * D;
+  // SF / PF / OD are indexed [slot * 2 + buffer].  A parity wait is only meaningful while the barrier
   // is at most one phase behind the waiter; per half buffer that holds by construction (the S
   // product that re-fills a half is queued behind the P V product that read it), which is why
   // "O is complete" is tracked per half as well.
@@ -85,6 +93,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SM::oBar);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + B_COUNT);
   static_assert(B_COUNT * 8 + 8 <= 256, "barrier area too small");
+  static_assert(kFwdCtasPerSm<D> * (SM::kTotal + 1024) <= 228 * 1024 && kFwdCtasPerSm<D> * kTmemCols <= 512, "does not fit an SM");
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // same value, known to be warp-uniform
   if ((smem_u32(smem) & 1023u) != 0) {   // the swizzled tiles need 1024-byte alignment
@@ -129,7 +138,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     tmem_slot[1] = abort_word;
   }
   if (warp == kFwdMmaWarp0) {
-    tmem_alloc(tmem_slot, 512);
+    tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -137,7 +146,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   if (tmem_slot[1] != 0) {   // after a failed wait the rest of the grid does nothing: the call ends in seconds, not minutes
-    if (warp == kFwdMmaWarp0) tmem_dealloc(tmem, 512);
+    if (warp == kFwdMmaWarp0) tmem_dealloc(tmem, kTmemCols);
     return;
   }
 
@@ -200,56 +209,61 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const uint32_t hi = desc_hi(1024);
     const uint32_t q_lo = desc_lo(smem_u32(sQ), 16) + s * (kTile >> 4), k_lo = desc_lo(smem_u32(sK), 16);
     const uint32_t v_mn_lo = desc_lo(smem_u32(sV), SM::kBox);
-    const uint32_t t_s = tmem + kColS + s * 128, t_o = tmem + kColO + s * 128;
+    const uint32_t t_s = tmem + kColS + s * kSlotS, t_o = tmem + kColO + s * D;
     bool ok = mbar_wait(bars + B_Q, 0, a.error_word, 7);
     int n_pv = 0;                 // P V products issued (accumulate flag)
     int pf0 = 0, pf1 = 0;         // uses of the two half buffers whose P V product was issued (barrier phases)
     int ce0 = 0, ce1 = 0, ne0, ne1, nn0, nn1;
     load_ent(0, ne0, ne1);
     load_ent(1, nn0, nn1);
+    bool k_seen = false;          // the K tile of the step whose S products are being issued has arrived
 #pragma unroll 1
-    for (int j = -1; j < n_steps; ++j) {   // step -1 only issues the S products of step 0
-      bool v_seen = false, k_seen = false;
+    for (int j = -1; j < n_steps; ++j) {   // step -1 only issues S products of step 0
+      bool v_seen = false;
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
-        const int ce = hf ? ce1 : ce0, ne = hf ? ne1 : ne0;
-        if ((static_cast<uint32_t>(ce) >> (s * RS)) & kSlotMask) {           // P V of half hf of step j
+        const int buf = NB == 2 ? hf : 0;
+        if ((static_cast<uint32_t>(hf ? ce1 : ce0) >> (s * RS)) & kSlotMask) {           // P V of half hf of step j
           const int sv = j & 1;
           if (!v_seen) { ok = ok && mbar_wait(bars + B_VF + sv, (j / 2) & 1, a.error_word, 9); v_seen = true; }
-          ok = ok && mbar_wait(bars + B_PF + s * 2 + hf, (hf ? pf1 : pf0) & 1, a.error_word, 10);
+          ok = ok && mbar_wait(bars + B_PF + s * 2 + buf, (buf ? pf1 : pf0) & 1, a.error_word, 10);
           if (ok) {
             tc_fence_after();
             const uint32_t b_lo = v_mn_lo + sv * (kTile >> 4) + hf * 4 * (2048 >> 4);
 #pragma unroll
             for (int kk = 0; kk < 4; ++kk)
-              if (lead) mma_ts2(t_o, t_s + hf * 64 + kk * 8, b_lo + kk * (2048 >> 4), hi, idesc_o, (n_pv > 0) || (kk > 0));
+              if (lead) mma_ts2(t_o, t_s + buf * 64 + kk * 8, b_lo + kk * (2048 >> 4), hi, idesc_o, (n_pv > 0) || (kk > 0));
           }
-          if (lead) mma_commit(bars + B_OD + s * 2 + hf);
+          if (lead) mma_commit(bars + B_OD + s * 2 + buf);
           ++n_pv;
-          if (hf) ++pf1; else ++pf0;
+          if (buf) ++pf1; else ++pf0;
         }
         if (hf == 1 && j >= 0) {
           if (!v_seen) ok = ok && mbar_wait(bars + B_VF + (j & 1), (j / 2) & 1, a.error_word, 9);
           if (lead) mma_commit(bars + B_VE + (j & 1));
         }
-        if ((static_cast<uint32_t>(ne) >> (s * RS)) & kSlotMask) {           // S of half hf of step j + 1
-          const int sk = (j + 1) % 3;
-          if (!k_seen) { ok = ok && mbar_wait(bars + B_KF + sk, ((j + 1) / 3) & 1, a.error_word, 8); k_seen = true; }
+        // the S product that takes the buffer next: the same half of step j + 1, or (one buffer) the next half
+        const int jn = (NB == 2 || hf == 1) ? j + 1 : j, hn = NB == 2 ? hf : 1 - hf;
+        const int ne = NB == 2 ? (hf ? ne1 : ne0) : (hf ? ne0 : ce1);
+        if (hn == 0) k_seen = false;
+        if ((static_cast<uint32_t>(ne) >> (s * RS)) & kSlotMask) {
+          const int sk = jn % 3;
+          if (!k_seen) { ok = ok && mbar_wait(bars + B_KF + sk, (jn / 3) & 1, a.error_word, 8); k_seen = true; }
           if (ok) {
             tc_fence_after();
-            const uint32_t b_lo = k_lo + sk * (kTile >> 4) + hf * kHalfRows;
+            const uint32_t b_lo = k_lo + sk * (kTile >> 4) + hn * kHalfRows;
 #pragma unroll
             for (int k = 0; k < D / 16; ++k) {
               constexpr int kB = SM::kBox >> 4;
               const uint32_t off = (k >> 2) * kB + (k & 3) * 2;
-              if (lead) mma_ss2(t_s + hf * 64, q_lo + off, b_lo + off, hi, idesc_s, k > 0);
+              if (lead) mma_ss2(t_s + buf * 64, q_lo + off, b_lo + off, hi, idesc_s, k > 0);
             }
           }
-          if (lead) mma_commit(bars + B_SF + s * 2 + hf);
+          if (lead) mma_commit(bars + B_SF + s * 2 + buf);
         }
-        if (hf == 1 && j + 1 < n_steps) {
-          if (!k_seen) ok = ok && mbar_wait(bars + B_KF + (j + 1) % 3, ((j + 1) / 3) & 1, a.error_word, 8);
-          if (lead) mma_commit(bars + B_KE + (j + 1) % 3);
+        if (hn == 1 && jn >= 0 && jn < n_steps) {
+          if (!k_seen) ok = ok && mbar_wait(bars + B_KF + jn % 3, (jn / 3) & 1, a.error_word, 8);
+          if (lead) mma_commit(bars + B_KE + jn % 3);
         }
       }
       ce0 = ne0; ce1 = ne1;
@@ -265,7 +279,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const int qi = row0 + s * 128 + r;
     const int member = s * RS + (BS == 128 ? 0 : (r >> 6));  // pattern row of the super-tile
     const uint32_t lane_addr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-    const uint32_t my_s = lane_addr + kColS + s * 128, my_o = lane_addr + kColO + s * 128;
+    const uint32_t my_s = lane_addr + kColS + s * kSlotS, my_o = lane_addr + kColO + s * D;
     // lowest key position this row may see outside what the pattern already excludes: the start of its
     // document (0 without documents)
     const int dstart = (a.doc_start && qi < a.L && qi >= a.q_start) ? a.doc_start[static_cast<int64_t>(b) * a.L + qi] : 0;
@@ -275,8 +289,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
                            : qi - a.exact_w + 1;
     float m_ref = -INFINITY;   // reference maximum (scaled, log2 domain) the probabilities are relative to
     float l_run = 0.f;
-    int p0 = 0, p1 = 0;        // P tiles published per half buffer (barrier phases)
-    // every P V product issued so far has completed (at most one per half can still be running)
+    int p0 = 0, p1 = 0;        // P tiles published per score buffer (barrier phases)
+    // every P V product issued so far has completed (at most one per buffer can still be running)
     auto wait_o = [&](uint32_t site) {
       bool w = true;
       if (p0 > 0) w = mbar_wait_warp(bars + B_OD + s * 2, (p0 - 1) & 1, a.error_word, site);
@@ -302,36 +316,49 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         const int lo = min(max(lo_abs - key0, 0), 64);
 
         const bool masked = __any_sync(0xffffffffu, lim < 64 || lo > 0);   // (voted before the wait: off the chain)
-        ok = mbar_wait_warp(bars + B_SF + s * 2 + hf, (hf ? p1 : p0) & 1, a.error_word, 12);
+        const int buf = NB == 2 ? hf : 0;
+        ok = mbar_wait_warp(bars + B_SF + s * 2 + buf, (buf ? p1 : p0) & 1, a.error_word, 12);
         if (!ok) break;
         tc_fence_after();
-        uint32_t v[64];
-        tmem_ld32(my_s + hf * 64, v);
-        tmem_ld32(my_s + hf * 64 + 32, v + 32);
-        tmem_ld_wait();
-        if (masked) {
+        constexpr int C = 32 * NB;                   // columns in registers at a time
+        uint32_t v[C];
+        auto load_cols = [&](int c0) {               // columns c0 .. c0 + C - 1 of the half
 #pragma unroll
-          for (int x = 0; x < 64; ++x)
-            v[x] = (x < lim && x >= lo) ? v[x] : 0xff800000u;   // -inf: the exponential below gives exactly 0
-        }
+          for (int x = 0; x < C; x += 32) tmem_ld32(my_s + buf * 64 + c0 + x, v + x);
+          tmem_ld_wait();
+          if (masked) {
+#pragma unroll
+            for (int y = 0; y < C; y += 32) {
+              const uint32_t seen = bit_range(min(max(lo - c0 - y, 0), 32), min(max(lim - c0 - y, 0), 32));
+#pragma unroll
+              for (int x = 0; x < 32; ++x)
+                v[y + x] = (seen >> x) & 1 ? v[y + x] : 0xff800000u;   // -inf: the exponential below gives exactly 0
+            }
+          }
+        };
         // Probabilities relative to the reference as it stands; the row maximum is only looked at when
         // that cannot be right: the row has no reference yet, or the sum of the half's probabilities
         // (an upper bound of each of them) passes 2^8.  Otherwise every probability is below 2^8 and the
         // reference stays -- the maximum, its 32 instructions per row and the vote are off the common path.
         uint32_t preg[32];
         float psum;
+        bool loaded = false;                         // with one chunk, v still holds the half when it is worked again
         auto exp_half = [&](float neg_m) {
           float q0 = 0.f, q1 = 0.f, q2 = 0.f, q3 = 0.f;   // independent partial sums
 #pragma unroll
-          for (int x = 0; x < 64; x += 4) {
-            const float x0 = fmaf(__uint_as_float(v[x]), a.scale_log2, neg_m);
-            const float x1 = fmaf(__uint_as_float(v[x + 1]), a.scale_log2, neg_m);
-            const float x2 = fmaf(__uint_as_float(v[x + 2]), a.scale_log2, neg_m);
-            const float x3 = fmaf(__uint_as_float(v[x + 3]), a.scale_log2, neg_m);
-            const float e0 = fast_exp2(x0), e1 = fast_exp2(x1), e2 = fast_exp2(x2), e3 = fast_exp2(x3);
-            q0 += e0; q1 += e1; q2 += e2; q3 += e3;
-            preg[x >> 1] = pack_bf16(e0, e1);
-            preg[(x >> 1) + 1] = pack_bf16(e2, e3);
+          for (int c0 = 0; c0 < 64; c0 += C) {
+            if (NB == 1 || !loaded) { load_cols(c0); loaded = true; }
+#pragma unroll
+            for (int x = 0; x < C; x += 4) {
+              const float x0 = fmaf(__uint_as_float(v[x]), a.scale_log2, neg_m);
+              const float x1 = fmaf(__uint_as_float(v[x + 1]), a.scale_log2, neg_m);
+              const float x2 = fmaf(__uint_as_float(v[x + 2]), a.scale_log2, neg_m);
+              const float x3 = fmaf(__uint_as_float(v[x + 3]), a.scale_log2, neg_m);
+              const float e0 = fast_exp2(x0), e1 = fast_exp2(x1), e2 = fast_exp2(x2), e3 = fast_exp2(x3);
+              q0 += e0; q1 += e1; q2 += e2; q3 += e3;
+              preg[(c0 + x) >> 1] = pack_bf16(e0, e1);
+              preg[((c0 + x) >> 1) + 1] = pack_bf16(e2, e3);
+            }
           }
           psum = (q0 + q2) + (q1 + q3);
         };
@@ -341,17 +368,19 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         // and cannot appear: masked scores are -inf, whose exponential is 0)
         const bool look = unset ? (lim > lo) : !(psum <= kFwdMaxProb);
         if (__any_sync(0xffffffffu, look)) {
-          float mx;
-          {
+          float mx = -INFINITY;
+#pragma unroll
+          for (int c0 = 0; c0 < 64; c0 += C) {
+            if (NB == 1) load_cols(c0);
             float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
 #pragma unroll
-            for (int x = 0; x < 64; x += 8) {
+            for (int x = 0; x < C; x += 8) {
               m0 = max3(m0, __uint_as_float(v[x + 0]), __uint_as_float(v[x + 1]));
               m1 = max3(m1, __uint_as_float(v[x + 2]), __uint_as_float(v[x + 3]));
               m2 = max3(m2, __uint_as_float(v[x + 4]), __uint_as_float(v[x + 5]));
               m3 = max3(m3, __uint_as_float(v[x + 6]), __uint_as_float(v[x + 7]));
             }
-            mx = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
+            mx = max3(mx, fmaxf(m0, m1), fmaxf(m2, m3));
           }
           // the rows that asked move their reference to the maximum seen so far (the others keep theirs)
           const float m_new = fmaxf(m_ref, mx * a.scale_log2);
@@ -375,12 +404,12 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
           exp_half((m_ref == -INFINITY) ? 0.f : -m_ref);
         }
         l_run += psum;
-        tmem_st32(my_s + hf * 64, preg);   // P over the first columns of this half's S
+        tmem_st32(my_s + buf * 64, preg);   // P over the first columns of this half's S
         tmem_st_wait();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(bars + B_PF + s * 2 + hf);
-        if (hf) ++p1; else ++p0;
+        if (lane == 0) mbar_arrive(bars + B_PF + s * 2 + buf);
+        if (buf) ++p1; else ++p0;
       }
     }
     // ---- epilogue: O / l -> bf16, LSE ------------------------------------------------------
@@ -409,7 +438,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == kFwdMmaWarp0) tmem_dealloc(tmem, 512);
+  if (warp == kFwdMmaWarp0) tmem_dealloc(tmem, kTmemCols);
 }
 
 }  // namespace lg
