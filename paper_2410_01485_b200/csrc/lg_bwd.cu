@@ -59,7 +59,13 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
     dim3 grid(r.B * r.Hkv, r.n_ktiles);
     a.ahead = sm_count();   // one CTA per SM
     a.head_group = head_group(r, r.B * r.Hkv);
-    a.n_long = r.n_ktiles;
+    const int n_kv = r.B * r.Hkv, per_tile = 128 / r.block;
+    a.n_long = 0;
+    a.long_group = n_kv;
+    if (r.mode == LG_MODE_SINK_WINDOW) {   // the sink tiles of all heads before everything else
+      a.n_long = (r.pat.ns + per_tile - 1) / per_tile;
+      if (a.n_long > r.n_ktiles) a.n_long = r.n_ktiles;
+    }
     a.descending = r.mode != LG_MODE_SINK_WINDOW;   // combs and full causal attention
     if (r.mode == LG_MODE_STRIDED_LOCAL && r.pat.stride > 1) {
       // the comb columns (every stride-th) are the longest and share kv tiles among themselves: those tiles,
@@ -68,11 +74,11 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
       // attention a tile streams each row for all query heads of its group; four kv heads at a time were
       // measured best there (64 / 8 heads at 128K, dS kept: 40.5-41.7 -> 39.8-39.9 ms, two at a time 40.8-41.1;
       // recomputing dQ pass: 34.4-34.9 -> 33.9-35.2 ms, two at a time 34.9-35.7).
-      const int n_comb = (r.pat.nB + r.pat.stride - 1) / r.pat.stride, per_tile = 128 / r.block;
+      const int n_comb = (r.pat.nB + r.pat.stride - 1) / r.pat.stride;
       a.n_long = (n_comb + per_tile - 1) / per_tile;
       if (a.n_long > r.n_ktiles) a.n_long = r.n_ktiles;
       const int comb_group = r.Hq == r.Hkv ? kHeadGroupCombs : kHeadGroupCombsGqa;
-      a.head_group = r.B * r.Hkv > comb_group ? comb_group : r.B * r.Hkv;
+      a.long_group = n_kv > comb_group ? comb_group : n_kv;
     }
     if (a.ahead < 0) return LG_ERR_CUDA;
     if (variant == kBwdKeepDs) {

@@ -67,9 +67,9 @@ struct BwdArgs {
   __nv_bfloat16* ds_buf;
   PatternDev pat;            // dK/dV pass that keeps dS: positions of the blocks
   int ahead;                 // dK/dV pass: CTAs that run at a time (see prefetch_successor), 0: no prefetch
-  int head_group;            // dK/dV pass: kv heads whose CTAs run side by side (cta_coords); >= gridDim.x: all of them
+  int head_group;            // kv heads (dQ pass: heads) whose CTAs run side by side (cta_coords); >= gridDim.x: all of them
+  int n_long, long_group;    // dK/dV pass: the first n_long launch ranks take long_group kv heads at a time (cta_coords2)
   int descending;            // dK/dV pass: walk a tile's entries from the last query block down (see the producer)
-  int n_long;                // dK/dV pass: launch ranks taken in head groups (cta_coords2); >= gridDim.y: all of them
 };
 template <int BS> constexpr int kDsTileBytes = BS * 64 * 2;
 
@@ -520,7 +520,7 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   unsigned int abort_word = 0;
   if (tid == 0) abort_word = *reinterpret_cast<volatile unsigned int*>(a.error_word);
   int cta_x, cta_y;   // (batch, kv head) and launch rank of this CTA's kv tile
-  cta_coords2(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, a.n_long, cta_x, cta_y);
+  cta_coords2(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.long_group, a.n_long, a.head_group, cta_x, cta_y);
   const int tile = checked(a.order[cta_y], 0, a.n_tiles - 1, a.error_word, 120);
   const int b = cta_x / a.Hkv, hk = cta_x % a.Hkv;
   const int ent_off = checked(a.tile_off[tile], 0, a.n_list, a.error_word, 121);
@@ -621,7 +621,7 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const int64_t w = static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x + a.ahead;
         if (w >= static_cast<int64_t>(gridDim.x) * gridDim.y) return;
         int x2, y2;
-        cta_coords2(w, gridDim.x, gridDim.y, a.head_group, a.n_long, x2, y2);
+        cta_coords2(w, gridDim.x, gridDim.y, a.long_group, a.n_long, a.head_group, x2, y2);
         const int t2 = checked(a.order[y2], 0, a.n_tiles - 1, a.error_word, 126);
         const int b2 = x2 / a.Hkv, hk2 = x2 % a.Hkv;
 #pragma unroll
@@ -822,7 +822,7 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       const int col0 = half * kKvHalf + g * C;                 // my first column within the step's 128 queries
       const int entry = sEnt[(j & 1) * 2 + (BS == 64 ? col0 / 64 : 0)];
       const int q0 = (entry >> 2) * BS + (BS == 128 ? col0 : col0 % 64);
-      const bool on = (entry >> member) & 1;
+      const bool on = (entry >> member) & 1;                   // (the same for all rows of a warp)
       const int xmin = on ? min(max(kj - q0, 0), C) : C;      // columns xmin <= c < xmax are visible
       const int hi_abs = (a.exact_w > 0 && kb_mine >= a.ns) ? min(dend, kj + a.exact_w) : dend;   // first query that no longer sees me
       const int xmax = min(max(hi_abs - q0, 0), C);
@@ -833,6 +833,20 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
+      if (!on) {
+        // The tile's other column alone sees these queries (most steps of a sink or comb column whose neighbour is
+        // an ordinary one): P and dS of mine are zero without being computed.
+        const uint32_t zero[C / 2] = {};
+        tmem_st16(s_addr, zero);
+        ew_publish(bars + B_PF + half);
+        ok = mbar_wait_warp(bars + B_DPF + half, j & 1, a.error_word, 2);
+        if (!ok) break;
+        tc_fence_after();
+        tmem_st16(dp_addr, zero);
+        ew_publish(bars + B_DSF + half);
+        if (lane == 0) mbar_arrive(bars + B_STE + (j & 1));
+        continue;
+      }
       float p[C];
       {
         uint32_t sreg[C];
@@ -840,6 +854,8 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         for (int c = 0; c < C; c += 32) tmem_ld32(s_addr + c, sreg + c);
         tmem_ld_wait();
         const bool masked = __any_sync(0xffffffffu, xmin > 0 || xmax < C);
+        static_assert(C == 32, "one mask word");
+        const uint32_t seen = bit_range(xmin, xmax);
 #pragma unroll
         for (int c = 0; c < C; c += 4) {
           const float4 l4 = st_l[c >> 2];
@@ -852,10 +868,10 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
           // the power cap the instructions of a polynomial on the FMA pipe cost more than the unit's cycles)
           float v0 = fast_exp2(x0), v1 = fast_exp2(x1), v2 = fast_exp2(x2), v3 = fast_exp2(x3);
           if (masked) {
-            v0 = (c >= xmin && c < xmax) ? v0 : 0.f;
-            v1 = (c + 1 >= xmin && c + 1 < xmax) ? v1 : 0.f;
-            v2 = (c + 2 >= xmin && c + 2 < xmax) ? v2 : 0.f;
-            v3 = (c + 3 >= xmin && c + 3 < xmax) ? v3 : 0.f;
+            v0 = (seen >> c) & 1 ? v0 : 0.f;
+            v1 = (seen >> (c + 1)) & 1 ? v1 : 0.f;
+            v2 = (seen >> (c + 2)) & 1 ? v2 : 0.f;
+            v3 = (seen >> (c + 3)) & 1 ? v3 : 0.f;
           }
           p[c] = v0;
           p[c + 1] = v1;

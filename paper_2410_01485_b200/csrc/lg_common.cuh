@@ -325,14 +325,19 @@ __device__ __forceinline__ void cta_coords(long long w, int n_x, int n_y, int gr
   x = grp * group + rem % size;
   y = rem / size;
 }
-// The same with two regions of launch ranks: the first n_long ranks in groups of `group` heads, the rest with
-// all heads side by side (a strided pattern's few long comb tiles per head, and the many short ones behind
-// them, which fill the tail whatever head the last long tile belongs to).
-__device__ __forceinline__ void cta_coords2(long long w, int n_x, int n_y, int group, int n_long, int& x, int& y) {
+// The same with two regions of launch ranks, each with a group size of its own: the first n_long ranks, which hold
+// the tiles that are much longer than the rest, and the ranks behind them.
+//   strided pattern: the few comb tiles per head a few heads at a time, the many short ones, which fill the tail
+//     whatever head the last long tile belongs to, with all heads side by side;
+//   sink + window (dK/dV pass): the sink tiles, which every query block sees, of all heads first, the others in
+//     groups.  Inside a group alone the longest-first order does not hold over the grid: the last group's sink tiles
+//     started when most of the work was done, and the pass waited for them (3 x 4 kv heads, 6001 tokens, window
+//     1024: SMs busy for 52 % of the pass).
+__device__ __forceinline__ void cta_coords2(long long w, int n_x, int n_y, int long_group, int n_long, int group, int& x, int& y) {
   const long long first = static_cast<long long>(n_x) * n_long;
-  if (n_long >= n_y || w < first) { cta_coords(w, n_x, n_long < n_y ? n_long : n_y, group, x, y); return; }
-  x = static_cast<int>((w - first) % n_x);
-  y = n_long + static_cast<int>((w - first) / n_x);
+  if (w < first) { cta_coords(w, n_x, n_long, long_group, x, y); return; }
+  cta_coords(w - first, n_x, n_y - n_long, group, x, y);
+  y += n_long;
 }
 
 // ---- small math helpers --------------------------------------------------------------
