@@ -265,10 +265,12 @@ lg_status prepare_workspace(const Resolved& r, const WsLayout& w, uint8_t* ws, i
   const int64_t tiles = static_cast<int64_t>(a.n_stiles) + a.n_qtiles + a.n_ktiles;
   const int64_t warps = tiles + (a.n_doc + 31) / 32 + (a.copy.n + 31) / 32;
   if (warps > 0x7fffffffll) return LG_ERR_UNSUPPORTED;
-  sched_build_kernel<<<static_cast<unsigned>((warps + kWarps - 1) / kWarps), kSchedThreads, 0, stream>>>(a); note_launch();
+  if (launch_kernel(true, sched_build_kernel, dim3(static_cast<unsigned>((warps + kWarps - 1) / kWarps)), kSchedThreads, 0, stream, a) != cudaSuccess)
+    return LG_ERR_CUDA;
   a.header = header;
-  sched_order_kernel<<<static_cast<unsigned>((tiles + kWarps - 1) / kWarps), kSchedThreads, 0, stream>>>(a, fp); note_launch();
-  return cudaGetLastError() == cudaSuccess ? LG_OK : LG_ERR_CUDA;
+  if (launch_kernel(true, sched_order_kernel, dim3(static_cast<unsigned>((tiles + kWarps - 1) / kWarps)), kSchedThreads, 0, stream, a, fp) != cudaSuccess)
+    return LG_ERR_CUDA;
+  return LG_OK;
 }
 
 // ---- tensor maps ---------------------------------------------------------------------

@@ -10,15 +10,19 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
                               uint8_t* ws, cudaStream_t stream, cudaEvent_t* marks) {
   lg_status s;
   float* stat = reinterpret_cast<float*>(ws + w.delta);
+  const BwdVariant variant = bwd_variant(r);
+  const bool overlap = launch_attn_overlapped(r);
   if (marks) cudaEventRecord(marks[0], stream);
   {
     const int Lp = static_cast<int>(align_up(r.L, 128));
     const int n_bh = r.B * r.Hq;
-    const int rows_per_block = 256 / (D / 8) * kDeltaRowsPerThread;
+    const int rows_per_block = 8 * kDeltaRowsPerWarp<D>;
     dim3 grid((Lp + rows_per_block - 1) / rows_per_block, n_bh < 65535 ? n_bh : 65535);
-    delta_kernel<D><<<grid, 256, 0, stream>>>(
-        static_cast<const __nv_bfloat16*>(o), static_cast<const __nv_bfloat16*>(d_o), lse, stat, r.os[0], r.os[1],
-        r.os[2], r.Hq, n_bh, r.L, Lp, static_cast<int64_t>(n_bh) * Lp); note_launch();
+    // (zeros: the tile that stands in for a half of a query tile a kv tile has no entry for)
+    uint4* zeros = variant == kBwdKeepDs ? reinterpret_cast<uint4*>(ws + w.ds_buf + ds_buffer_bytes(r) - 128 * 64 * 2) : nullptr;
+    if (launch_kernel(true, delta_kernel<D>, grid, 256, 0, stream, static_cast<const __nv_bfloat16*>(o),
+                          static_cast<const __nv_bfloat16*>(d_o), lse, stat, zeros, r.os[0], r.os[1], r.os[2], r.Hq, n_bh, r.L, Lp,
+                          static_cast<int64_t>(n_bh) * Lp) != cudaSuccess) return LG_ERR_CUDA;
   }
   if (marks) cudaEventRecord(marks[1], stream);
   BwdArgs a;
@@ -39,7 +43,6 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
   a.ds_buf = reinterpret_cast<__nv_bfloat16*>(ws + w.ds_buf);
   a.pat = r.pat;
   constexpr int smem = BwdSmem<D, BS>::kTotal;
-  const BwdVariant variant = bwd_variant(r);
 
   // ---- dK / dV pass -------------------------------------------------------------------
   {
@@ -82,17 +85,11 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
     }
     if (a.ahead < 0) return LG_ERR_CUDA;
     if (variant == kBwdKeepDs) {
-      // the tile of zeros that stands in for a half of a query tile a kv tile has no entry for
-      if (cudaMemsetAsync(ws + w.ds_buf + ds_buffer_bytes(r) - 128 * 64 * 2, 0, 128 * 64 * 2, stream) != cudaSuccess) return LG_ERR_CUDA;
-      auto kern = bwd_dkdv_kernel<D, BS, true>;
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-        return LG_ERR_CUDA;
-      kern<<<grid, kKvThreads, smem, stream>>>(tq, tk, tv, tdo, a); note_launch();
+      static std::atomic<bool> allowed[kMaxDevices];
+      if (launch_big_smem(overlap, allowed, bwd_dkdv_kernel<D, BS, true>, grid, kKvThreads, smem, stream, tq, tk, tv, tdo, a) != cudaSuccess) return LG_ERR_CUDA;
     } else {
-      auto kern = bwd_dkdv_kernel<D, BS, false>;
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-        return LG_ERR_CUDA;
-      kern<<<grid, kKvThreads, smem, stream>>>(tq, tk, tv, tdo, a); note_launch();
+      static std::atomic<bool> allowed[kMaxDevices];
+      if (launch_big_smem(overlap, allowed, bwd_dkdv_kernel<D, BS, false>, grid, kKvThreads, smem, stream, tq, tk, tv, tdo, a) != cudaSuccess) return LG_ERR_CUDA;
     }
     if (marks) cudaEventRecord(marks[2], stream);
   }
@@ -108,15 +105,14 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
     a.out0 = static_cast<__nv_bfloat16*>(dq);
     a.out1 = nullptr;
     for (int i = 0; i < 3; ++i) { a.s0[i] = r.qs[i]; a.s1[i] = 0; }
-    auto kern = bwd_dq_from_ds_kernel<D, BS>;
     constexpr int smem_q = DqDsSmem<D>::kTotal;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_q) != cudaSuccess)
-      return LG_ERR_CUDA;
     const int n_sm = sm_count();
     if (n_sm <= 0) return LG_ERR_CUDA;
     const long long n_items = static_cast<long long>(r.B) * r.Hq * r.n_qtiles;
     const int n_cta = static_cast<int>(n_items < n_sm ? n_items : n_sm);   // one CTA per SM, each working every n_cta-th item
-    kern<<<n_cta, kDq2Threads, smem_q, stream>>>(tk, a, r.B * r.Hq, r.n_qtiles); note_launch();
+    static std::atomic<bool> allowed[kMaxDevices];
+    if (launch_big_smem(overlap, allowed, bwd_dq_from_ds_kernel<D, BS>, dim3(n_cta), kDq2Threads, smem_q, stream, tk, a, r.B * r.Hq, r.n_qtiles) != cudaSuccess)
+      return LG_ERR_CUDA;
     if (marks) cudaEventRecord(marks[3], stream);
     return cudaGetLastError() == cudaSuccess ? LG_OK : LG_ERR_CUDA;
   }
@@ -136,11 +132,9 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
     a.out1 = nullptr;
     for (int i = 0; i < 3; ++i) { a.s0[i] = r.qs[i]; a.s1[i] = 0; }
     a.head_group = head_group(r, r.B * r.Hq);
-    auto kern = bwd_dq_kernel<D, BS>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
+    static std::atomic<bool> allowed[kMaxDevices];
+    if (launch_big_smem(overlap, allowed, bwd_dq_kernel<D, BS>, dim3(r.B * r.Hq, r.n_qtiles), kDqThreads, smem, stream, tq, tk, tv, tdo, a) != cudaSuccess)
       return LG_ERR_CUDA;
-    dim3 grid(r.B * r.Hq, r.n_qtiles);
-    kern<<<grid, kDqThreads, smem, stream>>>(tq, tk, tv, tdo, a); note_launch();
     if (marks) cudaEventRecord(marks[3], stream);
   }
   return cudaGetLastError() == cudaSuccess ? LG_OK : LG_ERR_CUDA;

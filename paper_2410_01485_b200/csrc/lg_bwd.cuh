@@ -75,34 +75,50 @@ template <int BS> constexpr int kDsTileBytes = BS * 64 * 2;
 
 // ---- stat = -(LSE * log2 e) and -rowsum(dO * O), stored negated (they are only ever subtracted),
 // each in a plane of its own: the dK/dV pass fetches four neighbouring queries' values of one kind
-// with a single 16-byte shared-memory load ---------------------------------------------------------
-constexpr int kDeltaRowsPerThread = 4;   // rows a thread works, their loads issued together
+// with a single 16-byte shared-memory load.  Bound by the HBM reads of O and dO.  A warp works consecutive rows,
+// kDeltaUnroll load instructions of each tensor in flight (read once: no place in the L1), and its results leave in
+// one store per plane.  The first block also fills the tile of zeros of the dQ pass that reads dS back (a memset
+// of its own was a launch). ------------------------------------------------------------------------
+constexpr int kDeltaUnroll = 8;
+template <int D> constexpr int kDeltaRowsPerWarp = kDeltaUnroll * 32 / (D / 8);
+__device__ __forceinline__ uint4 ld_once(const void* p) {
+  uint4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
 template <int D>
-__global__ void delta_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfloat16* __restrict__ d_o,
-                             const float* __restrict__ lse, float* __restrict__ stat, int64_t sb, int64_t sh,
-                             int64_t sl, int Hq, int n_bh, int L, int Lp, int64_t plane) {
+__global__ void __launch_bounds__(256)
+delta_kernel(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse, float* stat, uint4* zero_tile, int64_t sb,
+             int64_t sh, int64_t sl, int Hq, int n_bh, int L, int Lp, int64_t plane) {
+  pdl_trigger();
+  pdl_wait();
   // grid.x walks the padded rows of a head (rows i >= L exist only in `stat`, as zeros), grid.y the heads
-  constexpr int TPR = D / 8;   // threads per row, 16 bytes each
-  constexpr int U = kDeltaRowsPerThread;
-  const int rows = blockDim.x / TPR;                       // rows per pass of the block
-  const int i0 = blockIdx.x * (rows * U) + threadIdx.x / TPR;
-  const int ch = threadIdx.x % TPR;
+  constexpr int TPR = D / 8, RPI = 32 / TPR;               // threads per row, 16 bytes each; rows per load instruction
+  constexpr int U = kDeltaUnroll, ROWS = kDeltaRowsPerWarp<D>;
+  static_assert(ROWS <= 32, "a lane per row");
+  if (zero_tile && blockIdx.x == 0 && blockIdx.y == 0)
+    for (int x = threadIdx.x; x < 128 * 64 * 2 / 16; x += 256) zero_tile[x] = make_uint4(0, 0, 0, 0);
+  const int lane = threadIdx.x & 31;
+  const int i0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * ROWS;   // the warp's first row
+  if (i0 >= Lp) return;
   for (int bh = blockIdx.y; bh < n_bh; bh += gridDim.y) {
     const int h = bh % Hq, b = bh / Hq;
+    const int64_t off = b * sb + h * sh + (lane % TPR) * 8;
     uint4 ov[U], dv[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = i0 + u * rows;
+      const int i = i0 + u * RPI + lane / TPR;
       ov[u] = dv[u] = make_uint4(0, 0, 0, 0);
       if (i < L) {
-        const int64_t off = b * sb + h * sh + static_cast<int64_t>(i) * sl + ch * 8;
-        ov[u] = *reinterpret_cast<const uint4*>(o + off);
-        dv[u] = *reinterpret_cast<const uint4*>(d_o + off);
+        ov[u] = ld_once(o + off + static_cast<int64_t>(i) * sl);
+        dv[u] = ld_once(d_o + off + static_cast<int64_t>(i) * sl);
       }
     }
+    const int mine = i0 + lane;                              // the row whose values this lane stores (lane < ROWS)
+    const float l = (lane < ROWS && mine < L) ? lse[static_cast<int64_t>(bh) * L + mine] : 0.f;
+    float sum = 0.f;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int i = i0 + u * rows;
       const __nv_bfloat162* op = reinterpret_cast<const __nv_bfloat162*>(&ov[u]);
       const __nv_bfloat162* dp = reinterpret_cast<const __nv_bfloat162*>(&dv[u]);
       float acc = 0.f;
@@ -113,11 +129,13 @@ __global__ void delta_kernel(const __nv_bfloat16* __restrict__ o, const __nv_bfl
       }
 #pragma unroll
       for (int s = TPR / 2; s > 0; s >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
-      if (i < Lp && ch == 0) {
-        const int64_t row = static_cast<int64_t>(bh) * Lp + i;
-        stat[row] = i < L ? -lse[static_cast<int64_t>(bh) * L + i] * 1.4426950408889634f : 0.f;
-        stat[plane + row] = -acc;
-      }
+      const float t = __shfl_sync(0xffffffffu, acc, (lane % RPI) * TPR);   // row u RPI + lane % RPI
+      if (lane / RPI == u) sum = t;
+    }
+    if (lane < ROWS && mine < Lp) {
+      const int64_t row = static_cast<int64_t>(bh) * Lp + mine;
+      stat[row] = mine < L ? -l * 1.4426950408889634f : 0.f;
+      stat[plane + row] = -sum;
     }
   }
 }
@@ -190,6 +208,8 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
   static_assert(B_COUNT * 8 + 8 <= SM::kBarBytes, "barrier area too small");
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // same value, known to be warp-uniform
+  pdl_trigger();
+  pdl_wait();
   if ((smem_u32(smem) & 1023u) != 0) {   // the swizzled tiles need 1024-byte alignment
     if (tid == 0) atomicCAS(a.error_word, 0u, (2u << 24) | 20u);
     return;
@@ -505,6 +525,8 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   static_assert((B_COUNT + 3) * 8 + 64 <= SM::kBarBytes, "barrier area too small");
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // same value, known to be warp-uniform
+  pdl_trigger();
+  pdl_wait();
   if ((smem_u32(smem) & 1023u) != 0) {
     if (tid == 0) atomicCAS(a.error_word, 0u, (2u << 24) | 10u);
     return;
@@ -1018,6 +1040,8 @@ bwd_dq_from_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const BwdArgs a,
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + B_COUNT);
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  pdl_trigger();
+  pdl_wait();
   if ((smem_u32(smem) & 1023u) != 0) {
     if (tid == 0) atomicCAS(a.error_word, 0u, (2u << 24) | 80u);
     return;

@@ -649,7 +649,7 @@ lg_status lg_kv_ring_append(const lg_decode_params* p, void* k_cache, void* v_ca
   const int64_t threads = static_cast<int64_t>(p->B) * p->Hkv * T_new * (p->D / 8);
   const int64_t blocks = (threads + 255) / 256;
   if (blocks > 0x7fffffff) return LG_ERR_UNSUPPORTED;
-  return launch_overlapped(ring_append_kernel, dim3(static_cast<unsigned>(blocks)), 256, 0, static_cast<cudaStream_t>(stream),
+  return launch_kernel(true, ring_append_kernel, dim3(static_cast<unsigned>(blocks)), 256, 0, static_cast<cudaStream_t>(stream),
                            static_cast<__nv_bfloat16*>(k_cache), static_cast<__nv_bfloat16*>(v_cache),
                            static_cast<const __nv_bfloat16*>(k_new), static_cast<const __nv_bfloat16*>(v_new), n_tokens_before,
                            p->B, p->Hkv, p->D, T_new, p->sink_tokens, p->window_tokens) == cudaSuccess ? LG_OK : LG_ERR_CUDA;
@@ -728,7 +728,7 @@ lg_status lg_sparse_decode(const lg_decode_params* p, const void* q, const void*
     a.unit_count = reinterpret_cast<unsigned int*>(static_cast<uint8_t*>(workspace) + sizeof(WsHeader));
     a.part = reinterpret_cast<float*>(static_cast<uint8_t*>(workspace) + sizeof(WsHeader) + count_bytes);
     const int smem_flat = kDecWarps * kDecStages * 2 * kDecTile * p->D * 2 + (p->B + 1) * static_cast<int>(sizeof(int));
-    return launch_overlapped(p->D == 128 ? decode_stream_kernel<128> : decode_stream_kernel<64>, dim3(static_cast<unsigned>(n_cta)),
+    return launch_kernel(true, p->D == 128 ? decode_stream_kernel<128> : decode_stream_kernel<64>, dim3(static_cast<unsigned>(n_cta)),
                              kDecWarps * 32, smem_flat, st, a) == cudaSuccess ? LG_OK : LG_ERR_CUDA;
   }
   if (a.Hkv * a.HG > 65535 || p->B > 65535) return LG_ERR_UNSUPPORTED;

@@ -34,10 +34,9 @@ static lg_status launch_fwd_t(const Resolved& r, const WsLayout& w, const void* 
   a.head_group = head_group(r, r.B * r.Hq);
   auto kern = fwd_kernel<D, BS>;
   constexpr int smem = FwdSmem<D>::kTotal;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return LG_ERR_CUDA;
+  static std::atomic<bool> allowed[kMaxDevices];
   dim3 grid(r.B * r.Hq, r.n_stiles);
-  kern<<<grid, kFwdThreads, smem, stream>>>(tq, tk, tv, a); note_launch();
-  return cudaGetLastError() == cudaSuccess ? LG_OK : LG_ERR_CUDA;
+  return launch_big_smem(launch_attn_overlapped(r), allowed, kern, grid, kFwdThreads, smem, stream, tq, tk, tv, a) == cudaSuccess ? LG_OK : LG_ERR_CUDA;
 }
 
 lg_status launch_fwd(const Resolved& r, const WsLayout& w, const void* q, const void* k, const void* v, void* o,

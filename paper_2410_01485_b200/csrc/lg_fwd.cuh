@@ -96,6 +96,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   static_assert(kFwdCtasPerSm<D> * (SM::kTotal + 1024) <= 228 * 1024 && kFwdCtasPerSm<D> * kTmemCols <= 512, "does not fit an SM");
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // same value, known to be warp-uniform
+  pdl_trigger();
+  pdl_wait();
   if ((smem_u32(smem) & 1023u) != 0) {   // the swizzled tiles need 1024-byte alignment
     if (tid == 0) atomicCAS(a.error_word, 0u, (2u << 24) | 1u);
     return;

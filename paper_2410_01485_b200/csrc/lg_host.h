@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/lg.h"
 #include "lg_pattern.h"
 
@@ -32,19 +34,38 @@ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // lg_debug_kernel_launches); nothing in the library depends on it.
 void note_launch();
 
-// Launch of a kernel that calls pdl_wait() (lg_common.cuh) before it touches global memory: it may start while the
-// kernel before it on the stream drains.
+constexpr int kMaxDevices = 64;   // devices whose properties are looked up once
+
+// Launch of a kernel that calls pdl_wait() (lg_common.cuh) before it touches global memory: with `overlap` it may
+// start while the kernel before it on the stream drains.
 template <typename... Params, typename... Args>
-inline cudaError_t launch_overlapped(void (*kern)(Params...), dim3 grid, int block, int smem, cudaStream_t stream, Args&&... args) {
+inline cudaError_t launch_kernel(bool overlap, void (*kern)(Params...), dim3 grid, int block, int smem, cudaStream_t stream, const Args&... args) {
   cudaLaunchAttribute attr;
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid; cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-  cfg.attrs = &attr; cfg.numAttrs = 1;
-  note_launch();
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+  cfg.attrs = &attr; cfg.numAttrs = overlap ? 1 : 0;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
+  if (e == cudaSuccess) note_launch();
+  return e;
+}
+
+// The same for a kernel that needs more dynamic shared memory than a launch may ask for by default (allowed once per
+// device; a call on every launch cost the host a microsecond).
+template <typename... Params, typename... Args>
+inline cudaError_t launch_big_smem(bool overlap, std::atomic<bool>* allowed /* [kMaxDevices] of this kernel */, void (*kern)(Params...), dim3 grid,
+                                   int block, int smem, cudaStream_t stream, const Args&... args) {
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const bool known = dev < kMaxDevices && allowed[dev].load(std::memory_order_acquire);
+  if (known && launch_kernel(overlap, kern, grid, block, smem, stream, args...) == cudaSuccess) return cudaSuccess;
+  if (known) cudaGetLastError();   // (a device that was reset has forgotten it)
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+  if (dev < kMaxDevices) allowed[dev].store(true, std::memory_order_release);
+  return launch_kernel(overlap, kern, grid, block, smem, stream, args...);
 }
 
 struct Resolved {          // validated, defaulted copy of lg_attn_params
@@ -106,6 +127,14 @@ int sm_count();   // SMs of the current device, < 0 on failure
 int head_group(const Resolved& r, int n_x);
 size_t ds_buffer_bytes(const Resolved& r);
 
+
+// Whether the attention kernels of a problem are launched overlapped: up to two waves of the forward.  Their prologues
+// and launch latencies then weigh something (2 heads x 512 tokens fwd + bwd 36.9 -> 35.9 us, steps of 40-50 us by
+// 4-18 %).  Large ones gain nothing and lose 1-2 % (full causal, 32 heads x 16K: 8.55 -> 8.63 ms): CTAs that
+// arrive as SMs fall free are spread over the chip in another order than those of an ordinary launch.
+inline bool launch_attn_overlapped(const Resolved& r) {
+  return static_cast<long long>(r.B) * r.Hq * r.n_stiles <= 2 * 148;
+}
 
 lg_status check_arch();
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }

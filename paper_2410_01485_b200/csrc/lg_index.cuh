@@ -226,6 +226,8 @@ constexpr int kSchedThreads = 256;   // warps are independent of one another
 // Latency-bound integer work: a warp per tile looks at 32 blocks at a time (the one-thread-per-tile merges this
 // replaces took 30 us of a 520 us chunk call and 260 us of a 4.8 ms step over packed documents).
 __global__ void __launch_bounds__(kSchedThreads) sched_build_kernel(const SchedArgs a) {
+  pdl_trigger();
+  pdl_wait();
   if (blockIdx.x == 0 && threadIdx.x == 0 && a.header) header_begin(a.header);
   const int lane = threadIdx.x & 31;
   int64_t w = static_cast<int64_t>(blockIdx.x) * (kSchedThreads / 32) + (threadIdx.x >> 5);
@@ -281,6 +283,8 @@ __device__ __forceinline__ int rank_of(const int32_t* __restrict__ cnt, int n, i
 // Launch order: tiles with more work first (order[rank] = tile).  The last launch of a build: the header gets the
 // fingerprint the lists are known by (0: none).
 __global__ void __launch_bounds__(kSchedThreads) sched_order_kernel(const SchedArgs a, unsigned long long fp) {
+  pdl_trigger();
+  pdl_wait();
   if (blockIdx.x == 0 && threadIdx.x == 0 && fp != 0) a.header->fingerprint = fp;
   int w = blockIdx.x * (kSchedThreads / 32) + (threadIdx.x >> 5);
   const int32_t* cnt[3] = {a.sq_cnt, a.qt_cnt, a.kt_cnt};
