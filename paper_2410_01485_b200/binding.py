@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from typing import Optional, Tuple
 
 import torch
@@ -102,13 +103,30 @@ def _check(code: int, what: str):
         raise LgError(code, what)
 
 
+try:   # the handle alone: building a torch.cuda.Stream object for it costs three microseconds of a call
+    from torch._C import _cuda_getCurrentRawStream as _raw_stream, _cuda_getDevice as _device
+except ImportError:
+    _raw_stream = None
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    if _raw_stream is None or not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(_device())
 
 
-def _strides3(t: torch.Tensor):
-    assert t.dim() == 4 and t.stride(3) == 1, "expect [B, H, L, D] with contiguous D"
-    return (C.c_int64 * 3)(t.stride(0), t.stride(1), t.stride(2))
+_pack_strides = struct.Struct("=12q").pack_into      # q_strides .. o_strides, which lie side by side
+_STRIDES_AT = AttnParams.q_strides.offset
+assert AttnParams.o_strides.offset == _STRIDES_AT + 72
+
+
+def _set_strides(p: AttnParams, q, k, v, o):
+    """Strides of the four tensors [B, H, L, D] into p (one packed write: field by field it took 8 us); returns them."""
+    qs, ks, vs, os_ = q.stride(), k.stride(), v.stride(), o.stride()
+    assert len(qs) == len(ks) == len(vs) == len(os_) == 4 and qs[3] == ks[3] == vs[3] == os_[3] == 1, \
+        "expect [B, H, L, D] with contiguous D"
+    _pack_strides(p, _STRIDES_AT, qs[0], qs[1], qs[2], ks[0], ks[1], ks[2], vs[0], vs[1], vs[2], os_[0], os_[1], os_[2])
+    return qs, ks, vs, os_
 
 
 def attn_params(B, Hq, Hkv, L, D, block, mode, sink_tokens=0, window_tokens=0, stride_blocks=0, local_blocks=0,
@@ -193,7 +211,7 @@ def lg_sparse_attn_fwd(p: AttnParams, q, k, v, o=None, lse=None, workspace=None)
     o = torch.empty_like(q) if o is None else o
     lse = torch.empty(q.shape[:3], dtype=torch.float32, device=q.device) if lse is None else lse
     ws = attn_workspace(p, False, q.device) if workspace is None else workspace
-    p.q_strides, p.k_strides, p.v_strides, p.o_strides = _strides3(q), _strides3(k), _strides3(v), _strides3(o)
+    _set_strides(p, q, k, v, o)
     _check(lib.lg_sparse_attn_fwd(C.byref(p), q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(),
                                   lse.data_ptr(), ws.data_ptr(), ws.numel(), _stream()), "lg_sparse_attn_fwd")
     return o, lse
@@ -206,9 +224,9 @@ def lg_sparse_attn_bwd(p: AttnParams, q, k, v, o, lse, d_o, dq=None, dk=None, dv
     dk = torch.empty_like(k) if dk is None else dk
     dv = torch.empty_like(v) if dv is None else dv
     ws = attn_workspace(p, True, q.device) if workspace is None else workspace
-    assert d_o.stride() == o.stride() and dq.stride() == q.stride()
-    assert dk.stride() == k.stride() and dv.stride() == v.stride()
-    p.q_strides, p.k_strides, p.v_strides, p.o_strides = _strides3(q), _strides3(k), _strides3(v), _strides3(o)
+    qs, ks, vs, os_ = _set_strides(p, q, k, v, o)
+    assert d_o.stride() == os_ and dq.stride() == qs
+    assert dk.stride() == ks and dv.stride() == vs
     _check(lib.lg_sparse_attn_bwd(C.byref(p), q.data_ptr(), k.data_ptr(), v.data_ptr(), o.data_ptr(),
                                   lse.data_ptr(), d_o.data_ptr(), dq.data_ptr(), dk.data_ptr(), dv.data_ptr(),
                                   ws.data_ptr(), ws.numel(), _stream()), "lg_sparse_attn_bwd")
@@ -219,7 +237,7 @@ def lg_sparse_attn_bwd_marked(p: AttnParams, q, k, v, o, lse, d_o, dq, dk, dv, w
     """As lg_sparse_attn_bwd; records the caller's four torch.cuda.Event objects (timing enabled, each
     recorded once before so that its handle exists) around the delta, dK/dV and dQ kernels.  Does not
     synchronise: read event durations after the stream has passed them."""
-    p.q_strides, p.k_strides, p.v_strides, p.o_strides = _strides3(q), _strides3(k), _strides3(v), _strides3(o)
+    _set_strides(p, q, k, v, o)
     assert len(events) == 4
     ev = (C.c_void_p * 4)(*[e.cuda_event for e in events])
     _check(load_library().lg_sparse_attn_bwd_marked(
