@@ -12,6 +12,8 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
   float* stat = reinterpret_cast<float*>(ws + w.delta);
   const BwdVariant variant = bwd_variant(r);
   const bool overlap = launch_attn_overlapped(r);
+  const KvSplit split = kv_split(r);
+  unsigned int* tickets = split.len > 0 ? reinterpret_cast<unsigned int*>(ws + w.kv_ticket) : nullptr;
   if (marks) cudaEventRecord(marks[0], stream);
   {
     const int Lp = static_cast<int>(align_up(r.L, 128));
@@ -21,7 +23,8 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
     // (zeros: the tile that stands in for a half of a query tile a kv tile has no entry for)
     uint4* zeros = variant == kBwdKeepDs ? reinterpret_cast<uint4*>(ws + w.ds_buf + ds_buffer_bytes(r) - 128 * 64 * 2) : nullptr;
     if (launch_kernel(true, delta_kernel<D>, grid, 256, 0, stream, static_cast<const __nv_bfloat16*>(o),
-                          static_cast<const __nv_bfloat16*>(d_o), lse, stat, zeros, r.os[0], r.os[1], r.os[2], r.Hq, n_bh, r.L, Lp,
+                          static_cast<const __nv_bfloat16*>(d_o), lse, stat, zeros, tickets,
+                          split.n_ranks * r.B * r.Hkv, r.os[0], r.os[1], r.os[2], r.Hq, n_bh, r.L, Lp,
                           static_cast<int64_t>(n_bh) * Lp) != cudaSuccess) return LG_ERR_CUDA;
   }
   if (marks) cudaEventRecord(marks[1], stream);
@@ -84,13 +87,18 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
       a.long_group = n_kv > comb_group ? comb_group : n_kv;
     }
     if (a.ahead < 0) return LG_ERR_CUDA;
-    if (variant == kBwdKeepDs) {
-      static std::atomic<bool> allowed[kMaxDevices];
-      if (launch_big_smem(overlap, allowed, bwd_dkdv_kernel<D, BS, true>, grid, kKvThreads, smem, stream, tq, tk, tv, tdo, a) != cudaSuccess) return LG_ERR_CUDA;
-    } else {
-      static std::atomic<bool> allowed[kMaxDevices];
-      if (launch_big_smem(overlap, allowed, bwd_dkdv_kernel<D, BS, false>, grid, kKvThreads, smem, stream, tq, tk, tv, tdo, a) != cudaSuccess) return LG_ERR_CUDA;
-    }
+    a.split = split;
+    a.kv_part = reinterpret_cast<float4*>(ws + w.kv_part);
+    a.kv_ticket = tickets;
+    if (split.len > 0) grid.y = split.first_place[split.n_regions];
+    auto launch = [&](auto kern, std::atomic<bool>* allowed) {
+      return launch_big_smem(overlap, allowed, kern, grid, kKvThreads, smem, stream, tq, tk, tv, tdo, a);
+    };
+    static std::atomic<bool> allowed[4][kMaxDevices];
+    const cudaError_t e = variant == kBwdKeepDs
+        ? (split.len > 0 ? launch(bwd_dkdv_kernel<D, BS, true, true>, allowed[0]) : launch(bwd_dkdv_kernel<D, BS, true, false>, allowed[1]))
+        : (split.len > 0 ? launch(bwd_dkdv_kernel<D, BS, false, true>, allowed[2]) : launch(bwd_dkdv_kernel<D, BS, false, false>, allowed[3]));
+    if (e != cudaSuccess) return LG_ERR_CUDA;
     if (marks) cudaEventRecord(marks[2], stream);
   }
   if (variant == kBwdKeepDs) {

@@ -67,6 +67,9 @@ struct BwdArgs {
   __nv_bfloat16* ds_buf;
   PatternDev pat;            // dK/dV pass that keeps dS: positions of the blocks
   int ahead;                 // dK/dV pass: CTAs that run at a time (see prefetch_successor), 0: no prefetch
+  KvSplit split;             // dK/dV pass: kv tiles cut into pieces
+  float4* kv_part;           // partial sums of the pieces, [place][B * Hkv][dV | dK][D / 4][128 keys]
+  unsigned int* kv_ticket;   // [rank][B * Hkv] pieces delivered (zeroed by the delta pass)
   int head_group;            // kv heads (dQ pass: heads) whose CTAs run side by side (cta_coords); >= gridDim.x: all of them
   int n_long, long_group;    // dK/dV pass: the first n_long launch ranks take long_group kv heads at a time (cta_coords2)
   int descending;            // dK/dV pass: walk a tile's entries from the last query block down (see the producer)
@@ -78,7 +81,7 @@ template <int BS> constexpr int kDsTileBytes = BS * 64 * 2;
 // with a single 16-byte shared-memory load.  Bound by the HBM reads of O and dO.  A warp works consecutive rows,
 // kDeltaUnroll load instructions of each tensor in flight (read once: no place in the L1), and its results leave in
 // one store per plane.  The first block also fills the tile of zeros of the dQ pass that reads dS back (a memset
-// of its own was a launch). ------------------------------------------------------------------------
+// of its own was a launch) and clears the arrivals of split kv tiles. ------------------------------------------------------------------------
 constexpr int kDeltaUnroll = 8;
 template <int D> constexpr int kDeltaRowsPerWarp = kDeltaUnroll * 32 / (D / 8);
 __device__ __forceinline__ uint4 ld_once(const void* p) {
@@ -88,8 +91,9 @@ __device__ __forceinline__ uint4 ld_once(const void* p) {
 }
 template <int D>
 __global__ void __launch_bounds__(256)
-delta_kernel(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse, float* stat, uint4* zero_tile, int64_t sb,
-             int64_t sh, int64_t sl, int Hq, int n_bh, int L, int Lp, int64_t plane) {
+delta_kernel(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse, float* stat, uint4* zero_tile,
+             unsigned int* tickets, int n_tickets, int64_t sb, int64_t sh, int64_t sl, int Hq, int n_bh, int L, int Lp,
+             int64_t plane) {
   pdl_trigger();
   pdl_wait();
   // grid.x walks the padded rows of a head (rows i >= L exist only in `stat`, as zeros), grid.y the heads
@@ -98,6 +102,8 @@ delta_kernel(const __nv_bfloat16* o, const __nv_bfloat16* d_o, const float* lse,
   static_assert(ROWS <= 32, "a lane per row");
   if (zero_tile && blockIdx.x == 0 && blockIdx.y == 0)
     for (int x = threadIdx.x; x < 128 * 64 * 2 / 16; x += 256) zero_tile[x] = make_uint4(0, 0, 0, 0);
+  if (blockIdx.x == 0 && blockIdx.y == 0)
+    for (int x = threadIdx.x; x < n_tickets; x += 256) tickets[x] = 0;
   const int lane = threadIdx.x & 31;
   const int i0 = (blockIdx.x * 8 + (threadIdx.x >> 5)) * ROWS;   // the warp's first row
   if (i0 >= Lp) return;
@@ -498,6 +504,44 @@ constexpr int kKvHalf = 64;                                // queries of a half-
 constexpr int kKvNB = 128 / kKvHalf;                       // half-steps per step = score buffers in rotation = teams
 constexpr int kKvCols = kKvHalf / (kKvTeamWarps / 4);      // queries of a half-step per element-wise thread
 
+// The pieces of a split kv tile: the CTA that delivers the last one adds them, in their order whichever CTA that is, and
+// writes dK and dV.  Piece i of the tile sits at place first + i * stride.  The whole CTA calls, after its own
+// piece's stores have been fenced and a CTA barrier; flag: a word of shared memory.  Bound by the reads of the partial
+// sums (128 KB a piece at D = 128) from the L2.
+template <int D, int BS>
+__device__ __forceinline__ void kv_add_pieces(const BwdArgs& a, uint32_t* flag, int x, int rank, int first, int stride,
+                                              int n_segs, int kb_a, int kb_b, int b, int hk) {
+  const int heads = static_cast<int>(gridDim.x);
+  if (threadIdx.x == 0) {
+    __threadfence();
+    *flag = atomicAdd(a.kv_ticket + static_cast<int64_t>(rank) * heads + x, 1u) + 1u == static_cast<unsigned>(n_segs) ? 1u : 0u;
+  }
+  __syncthreads();
+  if (*flag == 0) return;
+  __threadfence();
+  constexpr int kSlot = 2 * (D / 4) * 128;                       // float4 of a piece
+  for (int u = threadIdx.x; u < 2 * (D / 8) * 128; u += blockDim.x) {   // eight columns of a key
+    const int r = u % 128, c8 = u / 128;                         // (c8 runs over dV's columns, then dK's)
+    const int member = BS == 64 ? r / 64 : 0, kb = member ? kb_b : kb_a, key = kb * BS + (BS == 64 ? r % 64 : r);
+    if (kb < 0 || key >= a.L) continue;
+    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+#pragma unroll 4
+    for (int i = 0; i < n_segs; ++i) {
+      const float4* p = a.kv_part + (static_cast<int64_t>(first + i * stride) * heads + x) * kSlot + c8 * 2 * 128 + r;
+      const float4 v = __ldcg(p), w = __ldcg(p + 128);
+      lo.x += v.x; lo.y += v.y; lo.z += v.z; lo.w += v.w;
+      hi.x += w.x; hi.y += w.y; hi.z += w.z; hi.w += w.w;
+    }
+    const bool is_dk = c8 >= D / 8;
+    const float m = is_dk ? a.scale : 1.0f;
+    const int64_t* st = is_dk ? a.s0 : a.s1;
+    uint4 out;
+    out.x = pack_bf16(lo.x * m, lo.y * m); out.y = pack_bf16(lo.z * m, lo.w * m);
+    out.z = pack_bf16(hi.x * m, hi.y * m); out.w = pack_bf16(hi.z * m, hi.w * m);
+    *reinterpret_cast<uint4*>((is_dk ? a.out0 : a.out1) + b * st[0] + hk * st[1] + static_cast<int64_t>(key) * st[2] + (c8 % (D / 8)) * 8) = out;
+  }
+}
+
 // kSpill: the pass also writes dS^T (bf16) of every half-step to global memory (BwdArgs::ds_buf), so
 // that the dQ pass is one product per step, dQ += dS K, instead of recomputing S and dP
 // (bwd_dq_from_ds_kernel).  Every element-wise thread stores the 64 bytes it holds (32 queries of its
@@ -505,7 +549,7 @@ constexpr int kKvCols = kKvHalf / (kKvTeamWarps / 4);      // queries of a half-
 // instruction covers 512 contiguous bytes.  (Staging the tiles in shared memory for a TMA store cost
 // a shared-memory ring stage of Q, a proxy fence and two barrier round trips per half-step; storing
 // rows of a [key][query] layout from registers touched 32 separate cache lines per instruction.)
-template <int D, int BS, bool kSpill>
+template <int D, int BS, bool kSpill, bool kSplit>
 __global__ void __launch_bounds__(kKvThreads, 1)
 bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                 const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_do, const BwdArgs a) {
@@ -542,7 +586,19 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   unsigned int abort_word = 0;
   if (tid == 0) abort_word = *reinterpret_cast<volatile unsigned int*>(a.error_word);
   int cta_x, cta_y;   // (batch, kv head) and launch rank of this CTA's kv tile
-  cta_coords2(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.long_group, a.n_long, a.head_group, cta_x, cta_y);
+  int place = 0, seg = 0, seg_stride = 0;                  // split kv tiles: my place, which piece of the tile it is, places between pieces
+  if constexpr (kSplit) {
+    cta_x = static_cast<int>(blockIdx.x);
+    place = static_cast<int>(blockIdx.y);
+    int reg = 0;
+    while (reg + 1 < a.split.n_regions && place >= a.split.first_place[reg + 1]) ++reg;
+    // the pieces of a region in turn, the tiles side by side: CTAs that run together walk the same rows
+    seg_stride = a.split.first_rank[reg + 1] - a.split.first_rank[reg];
+    seg = (place - a.split.first_place[reg]) / seg_stride;
+    cta_y = a.split.first_rank[reg] + (place - a.split.first_place[reg]) % seg_stride;
+  } else {
+    cta_coords2(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.long_group, a.n_long, a.head_group, cta_x, cta_y);
+  }
   const int tile = checked(a.order[cta_y], 0, a.n_tiles - 1, a.error_word, 120);
   const int b = cta_x / a.Hkv, hk = cta_x % a.Hkv;
   const int ent_off = checked(a.tile_off[tile], 0, a.n_list, a.error_word, 121);
@@ -551,7 +607,11 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   // key blocks of the tile's members (with 64-token blocks the two members need not be neighbours)
   const int kb_a = checked(a.tile_cols[R * tile], 0, a.nB - 1, a.error_word, 123);
   const int kb_b = (R == 2) ? checked(a.tile_cols[R * tile + 1], -1, a.nB - 1, a.error_word, 124) : -1;
-  const int n_items = n_ent * a.G;
+  const int all_items = n_ent * a.G;
+  const int n_segs = (kSplit && all_items > a.split.len) ? (all_items + a.split.len - 1) / a.split.len : 1;
+  if (seg >= n_segs) return;                               // an empty place (uniform over the CTA)
+  const int item0 = kSplit ? static_cast<int>(static_cast<int64_t>(all_items) * seg / n_segs) : 0;
+  const int n_items = kSplit ? static_cast<int>(static_cast<int64_t>(all_items) * (seg + 1) / n_segs) - item0 : all_items;
   const int n_hs = (BS == 128) ? kKvNB * n_items : (kKvNB == 2 ? n_items : (n_items + 1) / 2);    // half-steps
   const int n_steps = (n_hs + kKvNB - 1) / kKvNB;          // 128-row tiles streamed
   // half-step hs belongs to step hs / kKvNB and is its last one when:
@@ -614,7 +674,8 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       // 127 -> 92 GB of DRAM reads in the pass; its operands are 5 GB, but tiles that start later are on
       // rows of their own again).
       const int e_step = a.descending ? -1 : 1;
-      int grp = 0, e = a.descending ? n_ent - 1 : 0;    // (query head within the group, entry) of the next item
+      int grp = kSplit ? item0 % a.G : 0, e = kSplit ? item0 / a.G : 0;   // (query head within the group, entry) of the next item
+      if (a.descending) e = n_ent - 1 - e;
       // number of a member's dS tile: its block's position in the column lists (col_pos), the query block added
       // (a member that an entry does not list has no tile; its number is not used)
       const int pos_a = kSpill ? col_start(a.pat, kb_a) - kb_a : 0, pos_b = (kSpill && kb_b >= 0) ? col_start(a.pat, kb_b) - kb_b : 0;
@@ -639,7 +700,7 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       // again by the time they are wanted: + 25 % of DRAM reads in the profile), they are in the L2 by then.
       // A hint only: nothing waits for it and a wrong guess costs two tile reads.
       auto prefetch_successor = [&]() {
-        if (a.ahead <= 0) return;
+        if (kSplit || a.ahead <= 0) return;
         const int64_t w = static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x + a.ahead;
         if (w >= static_cast<int64_t>(gridDim.x) * gridDim.y) return;
         int x2, y2;
@@ -965,7 +1026,24 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       // products that are now done), 4 KB per warp, so that the stores cover whole rows (store_acc_64cols).
       constexpr int kParts = D / 64, kGroups = kKvEwWarps / 4;
       const int ge = warp >> 2;
-      if (kb_mine >= 0) {
+      if (kSplit && n_segs > 1) {
+        // a piece of a split tile: the sums as they stand, 512 contiguous bytes per store instruction of a warp
+        float4* part = a.kv_part + (static_cast<int64_t>(place) * gridDim.x + cta_x) * (2 * (D / 4) * 128) + (warp & 3) * 32 + lane;
+#pragma unroll
+        for (int pi = ge; pi < 2 * kParts; pi += kGroups) {
+#pragma unroll
+          for (int c = 0; c < 64; c += 32) {
+            uint32_t reg[32];
+            tmem_ld32(lane_addr + (pi >= kParts ? kColDK : kColDV) + (pi % kParts) * 64 + c, reg);
+            tmem_ld_wait();
+#pragma unroll
+            for (int x = 0; x < 32; x += 4)
+              part[(pi * 16 + (c + x) / 4) * 128] = make_float4(__uint_as_float(reg[x]), __uint_as_float(reg[x + 1]),
+                                                                __uint_as_float(reg[x + 2]), __uint_as_float(reg[x + 3]));
+          }
+        }
+        __threadfence();
+      } else if (kb_mine >= 0) {
 #pragma unroll
         for (int pi = ge; pi < 2 * kParts; pi += kGroups) {      // warp-uniform
           const bool is_dk = pi >= kParts;
@@ -992,6 +1070,8 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   tc_fence_before();
   __syncthreads();
   if (warp == kKvMmaWarpA) tmem_dealloc(tmem, 512);
+  if (kSplit && n_segs > 1)
+    kv_add_pieces<D, BS>(a, tmem_slot, cta_x, cta_y, place - seg * seg_stride, seg_stride, n_segs, kb_a, kb_b, b, hk);
 }
 
 // ============================== dQ from the kept dS ===========================================

@@ -83,6 +83,7 @@ struct Resolved {          // validated, defaulted copy of lg_attn_params
   int lists_prepared;        // the caller says the workspace already holds this pattern's lists
   unsigned long long expect_fp, expect_fp2;   // fingerprints the kernels accept in the header (0: no check)
   int64_t nnz;
+  int kv_total;              // kv heads (times batch) of the whole problem: B * Hkv, more when the call works a group of its heads
 };
 
 lg_status resolve(const lg_attn_params* p, Resolved* r);
@@ -97,6 +98,7 @@ struct WsLayout {
   size_t doc_end;                                // int32 [B, L]: end of each token's document (bwd with documents only)
   size_t delta;                                  // 2 x float [B, Hq, L]: -LSE * log2 e, then -delta (bwd only)
   size_t ds_buf;                                 // dS^T tiles (backward that keeps dS only, 0 otherwise)
+  size_t kv_part, kv_ticket;                     // dK/dV pass with split kv tiles: partial sums, arrivals per tile
   size_t total;
 };
 WsLayout ws_layout(const Resolved& r, bool want_bwd);
@@ -136,6 +138,9 @@ inline bool launch_attn_overlapped(const Resolved& r) {
   return static_cast<long long>(r.B) * r.Hq * r.n_stiles <= 2 * 148;
 }
 
+// How the dK/dV pass cuts its longest kv tiles (len = 0: not at all): see kv_split.
+KvSplit kv_split(const Resolved& r);
+
 lg_status check_arch();
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
@@ -151,6 +156,8 @@ lg_status attn_fwd_entry(const lg_attn_params* p, const void* q, const void* k, 
                          void* workspace, size_t workspace_bytes, void* stream, unsigned int* status_word);
 lg_status attn_bwd_entry(const lg_attn_params* p, const void* q, const void* k, const void* v, const void* o,
                          const float* lse, const void* d_o, void* dq, void* dk, void* dv, void* workspace,
-                         size_t workspace_bytes, void* stream, cudaEvent_t* marks, unsigned int* status_word);
+                         size_t workspace_bytes, void* stream, cudaEvent_t* marks, unsigned int* status_word,
+                         int kv_total = 0 /* kv heads of the whole problem when this is a group of them */);
+size_t attn_workspace_bytes(const lg_attn_params* p, int want_bwd, int kv_total);
 
 }  // namespace lg

@@ -11,6 +11,7 @@ namespace {
 struct GroupPlan {
   lg_attn_params pg;      // the group's problem: kv_per kv heads with their query heads, strides of the whole tensors
   int n_groups, kv_per, q_per;
+  int kv_total;           // kv heads of the whole problem
   size_t ws_per;          // workspace slice of one group
 };
 
@@ -33,7 +34,8 @@ lg_status plan_groups(const lg_attn_params* p, int head_groups, GroupPlan* g) {
     g->pg.q_strides[i] = g->pg.o_strides[i] = sq[i];
     g->pg.k_strides[i] = g->pg.v_strides[i] = sk[i];
   }
-  const size_t one = lg_sparse_attn_workspace_bytes(&g->pg, 1);
+  g->kv_total = r.doc_start && r.B > 1 ? r.Hkv : r.B * r.Hkv;   // (documents: sequence by sequence)
+  const size_t one = attn_workspace_bytes(&g->pg, 1, g->kv_total);
   if (one == 0) return LG_ERR_INVALID_ARG;
   g->ws_per = align_up(one, 256);
   return LG_OK;
@@ -117,7 +119,7 @@ lg_status lg_sparse_attn_fwd_bwd_host(const lg_attn_params* p, const void* q_hos
       if (result == LG_OK)
         result = attn_bwd_entry(&g.pg, qd, kd, vd, od, lsed, dod, off(dev->dq, q0, head_bytes),
                                 off(dev->dk, kv0, head_bytes), off(dev->dv, kv0, head_bytes), wsg, g.ws_per, s_cmp,
-                                nullptr, status);
+                                nullptr, status, g.kv_total);
     }
     ck(cudaEventRecord(ev_cmp, s_cmp));
     ck(cudaStreamWaitEvent(s_out, ev_cmp, 0));

@@ -126,4 +126,27 @@ __host__ __device__ __forceinline__ int kv_start(const PatternDev& p, int R, int
   return static_cast<int>(m * p.nB - p.stride * (m * (m - 1) / 2) + short_cols_sum(p, k - m));
 }
 
+// Query blocks that see a kv tile, i.e. the union of its columns' runs.
+__host__ __device__ __forceinline__ int kv_tile_len(const PatternDev& p, int R, int t) {
+  const int a = kv_col(p, R, R * t), na = col_len(p, a);
+  if (R == 1 || 2 * t + 1 >= p.nB) return na;
+  const int b = kv_col(p, R, 2 * t + 1), nb = col_len(p, b);
+  const int lo = a < b ? a : b, first_end = lo == a ? a + na : b + nb, second = lo == a ? b : a;
+  const int end = (a + na > b + nb) ? a + na : b + nb;
+  return second <= first_end ? end - lo : na + nb;
+}
+
+// The dK/dV pass gives a kv tile to one CTA, which walks it for every query head of the group.  Where that leaves the
+// chip waiting for the longest tiles they are cut: a tile of n items (query block x query head) into
+// ceil(n / len) nearly equal pieces, one CTA each, whose partial sums the CTA that finishes last adds in the order
+// of the pieces.  The launch ranks 0, 1, ... (tiles longest first) fall into regions; a rank of region i has places
+// for segs[i] pieces (a power of two; places beyond a tile's pieces stay empty).
+constexpr int kKvMaxRegions = 6, kKvMaxSegs = 32;
+struct KvSplit {
+  int len;                        // 0: no tile is cut
+  int n_regions;
+  int first_rank[kKvMaxRegions + 1], first_place[kKvMaxRegions + 1], segs[kKvMaxRegions];
+  int n_ranks, n_places;          // of the regions that cut (segs > 1): ranks, and places of pieces
+};
+
 }  // namespace lg
