@@ -447,7 +447,7 @@ static bool per_sequence(const Resolved& r) { return r.doc_start != nullptr && r
 static Resolved one_sequence(const Resolved& r, int b, void* workspace) {
   Resolved r1 = r;
   r1.B = 1;
-  r1.kv_total = r.Hkv;
+  r1.kv_total = r.kv_total / r.B;   // (of the whole problem's sequence: r.Hkv, more when r is a group of its heads)
   r1.doc_start = r.doc_start + static_cast<int64_t>(b) * r.L;
   r1.error_word = r.error_word ? r.error_word : static_cast<unsigned int*>(workspace);
   return r1;

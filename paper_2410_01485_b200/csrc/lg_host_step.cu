@@ -34,7 +34,7 @@ lg_status plan_groups(const lg_attn_params* p, int head_groups, GroupPlan* g) {
     g->pg.q_strides[i] = g->pg.o_strides[i] = sq[i];
     g->pg.k_strides[i] = g->pg.v_strides[i] = sk[i];
   }
-  g->kv_total = r.doc_start && r.B > 1 ? r.Hkv : r.B * r.Hkv;   // (documents: sequence by sequence)
+  g->kv_total = r.B * r.Hkv;
   const size_t one = attn_workspace_bytes(&g->pg, 1, g->kv_total);
   if (one == 0) return LG_ERR_INVALID_ARG;
   g->ws_per = align_up(one, 256);

@@ -76,3 +76,21 @@ def test_head_groups_of_the_host_step_split_like_the_whole(lg):
         torch.cuda.synchronize()
         for name, t in ref.items():
             assert torch.equal(out[name], t.cpu()), (groups, name)
+
+
+@pytest.mark.parametrize("groups", [4, 2])
+def test_head_groups_with_documents_in_several_sequences(lg, groups):
+    """Documents in a batch of two (run sequence by sequence), 16 / 4 heads: a whole sequence is cut into pieces of 48
+    items, two or four kv heads on their own would be cut into 24 or 16."""
+    cfg = replace(synth.CFG1, name="doc_groups", B=2, L=6000, D=64, Hq=16, Hkv=4, block=64, sink_tokens=64, window_tokens=1024)
+    ds = torch.stack([synth.make_doc_start(cfg.L, seed=30 + b, mean_len=5000) for b in range(2)]).cuda()
+    p = lg.params_of(cfg, doc_start=ds)
+    inp = synth.make_attn_inputs(cfg, "cuda", seed=14, with_do=True)
+    o, lse = lg.lg_sparse_attn_fwd(p, inp["q"], inp["k"], inp["v"])
+    ref = dict(zip(("o", "lse", "dq", "dk", "dv"), (o, lse) + lg.lg_sparse_attn_bwd(p, inp["q"], inp["k"], inp["v"], o, lse, inp["do"])))
+    host = {k: v.cpu().pin_memory() for k, v in inp.items()}
+    out = {n: torch.zeros(t.shape, dtype=t.dtype).pin_memory() for n, t in ref.items()}
+    lg.sparse_attn_fwd_bwd_host(lg.params_of(cfg, doc_start=ds), host, out, head_groups=groups)
+    torch.cuda.synchronize()
+    for name, t in ref.items():
+        assert torch.equal(out[name], t.cpu()), (groups, name)
