@@ -3,10 +3,8 @@
 #include <stdlib.h>
 #include <string.h>
 
-#include <algorithm>
 #include <atomic>
 #include <mutex>
-#include <vector>
 
 #include "lg_common.cuh"
 #include "lg_host.h"
@@ -41,7 +39,13 @@ static lg_status fix_strides(const int64_t in[3], int H, int L, int D, int64_t o
   return LG_OK;
 }
 
-lg_status resolve(const lg_attn_params* p, Resolved* r) {
+// Packed documents with several sequences: the block lists are shared by the sequences of a call, and documents prune
+// them per sequence; with documents and B > 1 a call therefore runs sequence by sequence, each with its own lists in
+// its own slice of the workspace (long packed samples fill the GPU one at a time).  The status
+// word of the call stays the first word of the whole workspace.
+static bool per_sequence(const Resolved& r) { return r.doc_start != nullptr && r.B > 1; }
+
+lg_status resolve(const lg_attn_params* p, Resolved* r, bool want_bwd, int kv_total) {
   if (!p || !r) return LG_ERR_INVALID_ARG;
   if (p->B < 1 || p->Hq < 1 || p->Hkv < 1 || p->L < 1 || p->Hq % p->Hkv != 0) return LG_ERR_INVALID_ARG;
   if (p->block != 64 && p->block != 128) return LG_ERR_INVALID_ARG;
@@ -112,8 +116,10 @@ lg_status resolve(const lg_attn_params* p, Resolved* r) {
     }
   }
   r->nnz = nnz;
-  r->kv_total = p->B * p->Hkv;
+  r->kv_total = kv_total > 0 ? kv_total : p->B * p->Hkv;
   if (nnz > 0x3fffffff || pt.nB > (1 << 20)) return LG_ERR_UNSUPPORTED;
+  // (documents in several sequences: the pass runs once per sequence)
+  r->split = want_bwd ? kv_split(pt, r->n_ktiles, r->G, nnz, per_sequence(*r) ? r->kv_total / r->B : r->kv_total) : KvSplit{};
   return LG_OK;
 }
 
@@ -176,53 +182,6 @@ BwdVariant bwd_variant(const Resolved& r) {
   return (can_keep && static_cast<double>(ds_buffer_bytes(r)) <= keep_ds_limit()) ? kBwdKeepDs : kBwdTwoPass;
 }
 
-// Cut the longest kv tiles?  In units of half-steps (64 queries x 128 keys): a CTA costs about 8 of them besides its
-// own (prologue, first loads, epilogue), so an even share of the pass is (all + 8 per CTA) / SMs.  Tiles are cut when
-// the longest one alone exceeds 1.1 such shares, into pieces of half a share, at least 16 (shorter pieces cost more in
-// overhead than they balance).  Measured, whole step: 3 x 16 / 4 heads x 6001 tokens, window 1024, D = 64: 604 -> 564
-// us; 16 / 4 heads x 4096 tokens, full causal with documents: 369 -> 313 us.
-// The rule looks at the whole problem, so that a step worked in groups of heads gives the same bits.
-KvSplit kv_split(const Resolved& r) {
-  KvSplit k{};
-  constexpr int kSms = 148, kCta = 8, kMinLen = 16;
-  const int R = 128 / r.block, per_item = r.block / 64;       // half-steps of an item
-  const int64_t per_entry = static_cast<int64_t>(r.G) * per_item;
-  // a bound first, without looking at the tiles: none is longer than twice the rows, and two columns share entries
-  if (per_entry * r.pat.nB * 2 * kSms <= r.nnz / R * per_entry * r.kv_total) return k;
-  int64_t all = 0, longest = 0;
-  std::vector<int> len(r.n_ktiles);
-  for (int t = 0; t < r.n_ktiles; ++t) {
-    len[t] = kv_tile_len(r.pat, R, t);
-    all += len[t];
-    if (len[t] > longest) longest = len[t];
-  }
-  longest *= per_entry;
-  const int64_t share = (all * per_entry + static_cast<int64_t>(kCta) * r.n_ktiles) * r.kv_total / kSms;
-  if (10 * (longest + kCta) <= 11 * (share + kCta)) return k;
-  int64_t piece = share / 2 > kMinLen ? share / 2 : kMinLen;   // half-steps
-  if (piece * kKvMaxSegs < longest) piece = (longest + kKvMaxSegs - 1) / kKvMaxSegs;
-  const int64_t items = (piece + per_item - 1) / per_item;
-  if (items * per_item >= longest) return k;
-  k.len = static_cast<int>(items);
-  std::sort(len.begin(), len.end(), [](int a, int b) { return a > b; });   // the launch order (documents only shorten tiles)
-  for (int y = 0; y < r.n_ktiles; ++y) {
-    const int64_t n = (static_cast<int64_t>(len[y]) * r.G + items - 1) / items;
-    int segs = 1;
-    while (segs < n) segs *= 2;
-    if (k.n_regions == 0 || segs != k.segs[k.n_regions - 1]) {
-      k.first_rank[k.n_regions] = y;
-      k.first_place[k.n_regions] = k.n_regions == 0 ? 0
-          : k.first_place[k.n_regions - 1] + (y - k.first_rank[k.n_regions - 1]) * k.segs[k.n_regions - 1];
-      k.segs[k.n_regions++] = segs;
-    }
-  }
-  k.first_rank[k.n_regions] = r.n_ktiles;
-  k.first_place[k.n_regions] = k.first_place[k.n_regions - 1] + (r.n_ktiles - k.first_rank[k.n_regions - 1]) * k.segs[k.n_regions - 1];
-  for (int i = 0; i < k.n_regions; ++i)
-    if (k.segs[i] > 1) { k.n_ranks = k.first_rank[i + 1]; k.n_places = k.first_place[i + 1]; }
-  return k;
-}
-
 WsLayout ws_layout(const Resolved& r, bool want_bwd) {
   WsLayout w{};
   size_t off = sizeof(WsHeader);
@@ -250,7 +209,7 @@ WsLayout ws_layout(const Resolved& r, bool want_bwd) {
     if (r.doc_start) w.doc_end = take(static_cast<size_t>(r.B) * r.L * 4);
     w.delta = take(static_cast<size_t>(r.B) * r.Hq * align_up(r.L, 128) * 8);   // rows padded to whole tiles   // two planes: -LSE * log2 e and -delta per query row
     if (keep) w.ds_buf = take(ds_buffer_bytes(r));
-    const KvSplit split = kv_split(r);
+    const KvSplit& split = r.split;
     if (split.len > 0) {
       const size_t heads = static_cast<size_t>(r.B) * r.Hkv;
       w.kv_part = take(heads * split.n_places * 2 * 128 * r.D * 4);
@@ -437,17 +396,9 @@ __global__ void wait_selftest_kernel(unsigned int* error_word, long long limit_c
   }
 }
 
-// ---- packed documents with several sequences ------------------------------------------------
-// The block lists are shared by the sequences of a call, and documents prune them per sequence;
-// with documents and B > 1 a call therefore runs sequence by sequence, each with its own lists in
-// its own slice of the workspace (long packed samples fill the GPU one at a time).  The status
-// word of the call stays the first word of the whole workspace.
-static bool per_sequence(const Resolved& r) { return r.doc_start != nullptr && r.B > 1; }
-
 static Resolved one_sequence(const Resolved& r, int b, void* workspace) {
   Resolved r1 = r;
   r1.B = 1;
-  r1.kv_total = r.kv_total / r.B;   // (of the whole problem's sequence: r.Hkv, more when r is a group of its heads)
   r1.doc_start = r.doc_start + static_cast<int64_t>(b) * r.L;
   r1.error_word = r.error_word ? r.error_word : static_cast<unsigned int*>(workspace);
   return r1;
@@ -460,8 +411,7 @@ static size_t attn_workspace_total(const Resolved& r, bool want_bwd) {
 
 size_t attn_workspace_bytes(const lg_attn_params* p, int want_bwd, int kv_total) {
   Resolved r;
-  if (resolve(p, &r) != LG_OK) return 0;
-  if (kv_total > 0) r.kv_total = kv_total;
+  if (resolve(p, &r, want_bwd != 0, kv_total) != LG_OK) return 0;
   return attn_workspace_total(r, want_bwd != 0);
 }
 
@@ -515,7 +465,7 @@ lg_status lg_sparse_attn_prepare(const lg_attn_params* p, void* workspace, size_
                                  void* stream) {
   LG_RANGE("lg_sparse_attn_prepare");
   Resolved r;
-  lg_status s = resolve(p, &r);
+  lg_status s = resolve(p, &r, want_bwd != 0);
   if (s != LG_OK) return s;
   if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255)) return LG_ERR_INVALID_ARG;
   if (per_sequence(r)) return LG_ERR_UNSUPPORTED;   // lists per sequence: those calls build them themselves
@@ -572,9 +522,8 @@ lg_status attn_bwd_entry(const lg_attn_params* p, const void* q, const void* k, 
                          size_t workspace_bytes, void* stream, cudaEvent_t* marks, unsigned int* status_word,
                          int kv_total) {
   Resolved r;
-  lg_status s = resolve(p, &r);
+  lg_status s = resolve(p, &r, true, kv_total);
   if (s != LG_OK) return s;
-  if (kv_total > 0) r.kv_total = kv_total;
   r.error_word = status_word;
   if (!q || !k || !v || !o || !lse || !d_o || !dq || !dk || !dv || !workspace) return LG_ERR_INVALID_ARG;
   if (!aligned16(q) || !aligned16(k) || !aligned16(v) || !aligned16(o) || !aligned16(lse) || !aligned16(d_o) ||

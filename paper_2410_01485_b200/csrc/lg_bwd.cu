@@ -12,7 +12,7 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
   float* stat = reinterpret_cast<float*>(ws + w.delta);
   const BwdVariant variant = bwd_variant(r);
   const bool overlap = launch_attn_overlapped(r);
-  const KvSplit split = kv_split(r);
+  const KvSplit& split = r.split;
   unsigned int* tickets = split.len > 0 ? reinterpret_cast<unsigned int*>(ws + w.kv_ticket) : nullptr;
   if (marks) cudaEventRecord(marks[0], stream);
   {

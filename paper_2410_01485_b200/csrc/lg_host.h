@@ -84,9 +84,12 @@ struct Resolved {          // validated, defaulted copy of lg_attn_params
   unsigned long long expect_fp, expect_fp2;   // fingerprints the kernels accept in the header (0: no check)
   int64_t nnz;
   int kv_total;              // kv heads (times batch) of the whole problem: B * Hkv, more when the call works a group of its heads
+  KvSplit split;             // how the dK/dV pass cuts its kv tiles (calls with a backward; see kv_split)
 };
 
-lg_status resolve(const lg_attn_params* p, Resolved* r);
+// want_bwd: the call runs, prepares or sizes a backward; kv_total: kv heads of the whole problem when `p` is a group of
+// them (0: p is the whole)
+lg_status resolve(const lg_attn_params* p, Resolved* r, bool want_bwd = false, int kv_total = 0);
 
 // Layout of the attention workspace (all offsets 256-byte aligned).
 struct WsLayout {
@@ -137,9 +140,6 @@ size_t ds_buffer_bytes(const Resolved& r);
 inline bool launch_attn_overlapped(const Resolved& r) {
   return static_cast<long long>(r.B) * r.Hq * r.n_stiles <= 2 * 148;
 }
-
-// How the dK/dV pass cuts its longest kv tiles (len = 0: not at all): see kv_split.
-KvSplit kv_split(const Resolved& r);
 
 lg_status check_arch();
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }

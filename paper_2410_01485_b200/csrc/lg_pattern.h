@@ -149,4 +149,57 @@ struct KvSplit {
   int n_ranks, n_places;          // of the regions that cut (segs > 1): ranks, and places of pieces
 };
 
+
+// Cut the longest kv tiles?  In units of half-steps (64 queries x 128 keys): a CTA costs about 8 of them besides its
+// own (prologue, first loads, epilogue), so an even share of the pass is (all + 8 per CTA) / SMs.  Tiles are cut when
+// the longest one alone exceeds 1.1 such shares, into pieces of half a share, at least 16 (shorter pieces cost more in
+// overhead than they balance).  Measured, whole step: 3 x 16 / 4 heads x 6001 tokens, window 1024, D = 64: 604 -> 564
+// us; 16 / 4 heads x 4096 tokens, full causal with documents: 369 -> 313 us.
+// kv_total: kv heads (times batch) of the whole problem, so that a step worked in groups of heads gives the same bits.
+// A call evaluates this once (resolve); it walks the tiles at most twice and allocates nothing (evaluated three times
+// with a sorted copy of the lengths, a backward call over 2 heads x 128K tokens, window 4096, took 75 us of host time; 26).
+inline KvSplit kv_split(const PatternDev& p, int n_ktiles, int G, int64_t nnz, int kv_total) {
+  KvSplit k{};
+  constexpr int kSms = 148, kCta = 8, kMinLen = 16;
+  const int R = 128 / p.block, per_item = p.block / 64;        // half-steps of an item
+  const int64_t per_entry = static_cast<int64_t>(G) * per_item;
+  // a bound first, without looking at the tiles: none is longer than twice the rows, and two columns share entries
+  if (per_entry * p.nB * 2 * kSms <= nnz / R * per_entry * kv_total) return k;
+  int64_t all = 0, longest = 0;
+  for (int t = 0; t < n_ktiles; ++t) {
+    const int len = kv_tile_len(p, R, t);
+    all += len;
+    if (len > longest) longest = len;
+  }
+  longest *= per_entry;
+  const int64_t share = (all * per_entry + static_cast<int64_t>(kCta) * n_ktiles) * kv_total / kSms;
+  if (10 * (longest + kCta) <= 11 * (share + kCta)) return k;
+  int64_t piece = share / 2 > kMinLen ? share / 2 : kMinLen;   // half-steps
+  if (piece * kKvMaxSegs < longest) piece = (longest + kKvMaxSegs - 1) / kKvMaxSegs;
+  const int64_t items = (piece + per_item - 1) / per_item;
+  if (items * per_item >= longest) return k;
+  k.len = static_cast<int>(items);
+  // a region per number of places, the longest tiles first as they are launched (documents only shorten tiles)
+  int tiles[kKvMaxRegions] = {};                                // with up to 2^i pieces
+  for (int t = 0; t < n_ktiles; ++t) {
+    const int64_t n = (static_cast<int64_t>(kv_tile_len(p, R, t)) * G + items - 1) / items;
+    int i = 0;
+    while ((1 << i) < n) ++i;
+    ++tiles[i];
+  }
+  int rank = 0, place = 0;
+  for (int i = kKvMaxRegions - 1; i >= 0; --i) {
+    if (tiles[i] == 0) continue;
+    k.first_rank[k.n_regions] = rank;
+    k.first_place[k.n_regions] = place;
+    k.segs[k.n_regions++] = 1 << i;
+    rank += tiles[i];
+    place += tiles[i] << i;
+    if (i > 0) { k.n_ranks = rank; k.n_places = place; }
+  }
+  k.first_rank[k.n_regions] = rank;
+  k.first_place[k.n_regions] = place;
+  return k;
+}
+
 }  // namespace lg
