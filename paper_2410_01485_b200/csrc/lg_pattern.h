@@ -141,7 +141,7 @@ __host__ __device__ __forceinline__ int kv_tile_len(const PatternDev& p, int R, 
 // ceil(n / len) nearly equal pieces, one CTA each, whose partial sums the CTA that finishes last adds in the order
 // of the pieces.  The launch ranks 0, 1, ... (tiles longest first) fall into regions; a rank of region i has places
 // for segs[i] pieces (a power of two; places beyond a tile's pieces stay empty).
-constexpr int kKvMaxRegions = 6, kKvMaxSegs = 32;
+constexpr int kKvMaxRegions = 6, kKvMaxSegs = 32, kKvMaxPlaces = 65535;   // places: a grid's limit in y
 struct KvSplit {
   int len;                        // 0: no tile is cut
   int n_regions;
@@ -199,6 +199,7 @@ inline KvSplit kv_split(const PatternDev& p, int n_ktiles, int G, int64_t nnz, i
   }
   k.first_rank[k.n_regions] = rank;
   k.first_place[k.n_regions] = place;
+  if (place > kKvMaxPlaces) return KvSplit{};                   // (one kv head and more than 8.3 million tokens)
   return k;
 }
 

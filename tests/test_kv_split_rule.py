@@ -129,3 +129,15 @@ def test_places_hold_every_tile_and_the_rule_allocates_nothing(rule):
     assert sum(x[0] > 0 for x in got) > 500            # of 4440: the rule does cut
     assert all(x[2] == 0 for x in got)
     assert [p for p, x in zip(problems, got) if x[3]] == []
+
+
+@pytest.mark.parametrize("mode, a, b, kv", [(1, 1, 2, 1), (1, 1, 1, 2), (2, 4000, 1, 1), (2, 30000, 2, 1)])
+@pytest.mark.parametrize("block", [64, 128])
+def test_places_stay_within_a_grid(rule, block, mode, a, b, kv):
+    """The kv tiles (at most 65535) and the places of cut ones are a grid's y extent: no cut rather than a launch that fails."""
+    problems = [(n * 128 // block, block, mode, a, b, 1, kv, n) for n in [60000, 64000] + list(range(65400, 65536))]
+    got = rule(problems)
+    assert got[0][0] > 0 and got[0][1] > 60000                         # cut well below the limit
+    assert max(places for _, places, _, _ in got) <= 65535
+    assert got[-1][0] == 0                                             # 65535 tiles leave no place to spare
+    assert all(x[3] == 0 for x in got)
