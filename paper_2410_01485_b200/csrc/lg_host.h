@@ -37,7 +37,8 @@ void note_launch();
 constexpr int kMaxDevices = 64;   // devices whose properties are looked up once
 
 // Launch of a kernel that calls pdl_wait() (lg_common.cuh) before it touches global memory: with `overlap` it may
-// start while the kernel before it on the stream drains.
+// start while the kernel before it on the stream drains.  A failed launch is reported by the result alone: it does not
+// stay behind as the runtime's last error, which a later call would take for its own.
 template <typename... Params, typename... Args>
 inline cudaError_t launch_kernel(bool overlap, void (*kern)(Params...), dim3 grid, int block, int smem, cudaStream_t stream, const Args&... args) {
   cudaLaunchAttribute attr;
@@ -49,6 +50,7 @@ inline cudaError_t launch_kernel(bool overlap, void (*kern)(Params...), dim3 gri
   cfg.attrs = &attr; cfg.numAttrs = overlap ? 1 : 0;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
   if (e == cudaSuccess) note_launch();
+  else cudaGetLastError();
   return e;
 }
 
@@ -62,8 +64,8 @@ inline cudaError_t launch_big_smem(bool overlap, std::atomic<bool>* allowed /* [
   if (e != cudaSuccess) return e;
   const bool known = dev < kMaxDevices && allowed[dev].load(std::memory_order_acquire);
   if (known && launch_kernel(overlap, kern, grid, block, smem, stream, args...) == cudaSuccess) return cudaSuccess;
-  if (known) cudaGetLastError();   // (a device that was reset has forgotten it)
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+  // (a device that was reset has forgotten it)
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) { cudaGetLastError(); return e; }
   if (dev < kMaxDevices) allowed[dev].store(true, std::memory_order_release);
   return launch_kernel(overlap, kern, grid, block, smem, stream, args...);
 }
