@@ -86,7 +86,7 @@ constexpr int kDeltaUnroll = 8;
 template <int D> constexpr int kDeltaRowsPerWarp = kDeltaUnroll * 32 / (D / 8);
 __device__ __forceinline__ uint4 ld_once(const void* p) {
   uint4 v;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  asm volatile("ld.global.L1::no_allocate.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }
 template <int D>

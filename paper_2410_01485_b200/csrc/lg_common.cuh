@@ -292,8 +292,9 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 // A kernel launched with `overlap` (launch_kernel, lg_host.h) may start while the kernel before it on the stream drains:
 // its CTAs take the SMs that fall free, and everything up to pdl_wait() -- which returns when that kernel has
 // finished and its writes are visible -- runs beside the other's tail.  Nothing global may be touched before the
-// wait (so such a kernel's parameters are not `const __restrict__`: loads through those may be moved above it), and
-// every thread that goes on to touch something calls it.  pdl_trigger() lets the next kernel start
+// wait, and what it reads may still be written while it already runs: no `const __restrict__` inputs (loads through those
+// may be moved above the wait) and no loads by the non-coherent path, which is for data nobody writes during the kernel's
+// lifetime.  Every thread that goes on to touch something calls the wait.  pdl_trigger() lets the next kernel start
 // once every CTA has called it (or left); without it the next one starts when this one has finished.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

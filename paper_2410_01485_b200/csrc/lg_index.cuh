@@ -194,7 +194,7 @@ __device__ __forceinline__ int merge_cols(const PatternDev& p, int ca, int cb, i
 
 // end (one past the last token) of the document token j belongs to, from doc_start[i] = first token of token i's
 // document (non-decreasing): the first i > j whose document starts after j, found by bisection, or L.
-__device__ __forceinline__ int doc_end_of(const int32_t* __restrict__ ds, int j, int L) {
+__device__ __forceinline__ int doc_end_of(const int32_t* ds, int j, int L) {
   int lo = j, hi = L;            // ds[lo] <= j (its own document); ds[hi] > j, with ds[L] taken as +inf
   while (hi - lo > 1) {
     const int mid = (lo + hi) >> 1;
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kSchedThreads) sched_build_kernel(const SchedA
 }
 
 // rank of tile t by (count descending, tile ascending); one warp
-__device__ __forceinline__ int rank_of(const int32_t* __restrict__ cnt, int n, int t) {
+__device__ __forceinline__ int rank_of(const int32_t* cnt, int n, int t) {
   const int c = cnt[t];
   int rank = 0;
   for (int u = threadIdx.x & 31; u < n; u += 32) {
