@@ -906,7 +906,7 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       const int entry = sEnt[(j & 1) * 2 + (BS == 64 ? col0 / 64 : 0)];
       const int q0 = (entry >> 2) * BS + (BS == 128 ? col0 : col0 % 64);
       const bool on = (entry >> member) & 1;                   // (the same for all rows of a warp)
-      const int xmin = on ? min(max(kj - q0, 0), C) : C;      // columns xmin <= c < xmax are visible
+      const int xmin = min(max(kj - q0, 0), C);                // columns xmin <= c < xmax are visible (of a member that is on)
       const int hi_abs = (a.exact_w > 0 && kb_mine >= a.ns) ? min(dend, kj + a.exact_w) : dend;   // first query that no longer sees me
       const int xmax = min(max(hi_abs - q0, 0), C);
       const uint32_t s_addr = lane_addr + kColS + half * kKvHalf + g * C;
@@ -918,7 +918,8 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       tc_fence_after();
       if (!on) {
         // The tile's other column alone sees these queries (most steps of a sink or comb column whose neighbour is
-        // an ordinary one): P and dS of mine are zero without being computed.
+        // an ordinary one): P and dS of mine are zero without being computed (and a block that is not in the pattern
+        // has no tile to keep).
         const uint32_t zero[C / 2] = {};
         tmem_st16(s_addr, zero);
         ew_publish(bars + B_PF + half);
@@ -1000,15 +1001,12 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // ... and to this half-step's tile in global memory: my C queries are C / 8 16-byte groups of my
         // key.  (Written once, read once by the dQ pass: marked evict-first so that the stream does not
         // push the Q / dO tiles, which every kv tile of a window re-reads, out of the L2.)
-        // (a member the entry does not list has no block, hence no tile: its dS is zero and stays unwritten)
-        if (on) {
-          uint8_t* dst = reinterpret_cast<uint8_t*>(a.ds_buf) + sTile[(j & 1) * 4 + half * 2 + member] * kDsTileBytes<BS> +
-                         (C / 8 * g) * (16 * BS) + (r & (BS - 1)) * 16;
+        uint8_t* dst = reinterpret_cast<uint8_t*>(a.ds_buf) + sTile[(j & 1) * 4 + half * 2 + member] * kDsTileBytes<BS> +
+                       (C / 8 * g) * (16 * BS) + (r & (BS - 1)) * 16;
 #pragma unroll
-          for (int i = 0; i < C / 8; ++i)
-            asm volatile("st.global.L2::cache_hint.v4.b32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(dst + i * (16 * BS)),
-                         "r"(dsreg[4 * i]), "r"(dsreg[4 * i + 1]), "r"(dsreg[4 * i + 2]), "r"(dsreg[4 * i + 3]), "l"(evict_first) : "memory");
-        }
+        for (int i = 0; i < C / 8; ++i)
+          asm volatile("st.global.L2::cache_hint.v4.b32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(dst + i * (16 * BS)),
+                       "r"(dsreg[4 * i]), "r"(dsreg[4 * i + 1]), "r"(dsreg[4 * i + 2]), "r"(dsreg[4 * i + 3]), "l"(evict_first) : "memory");
       }
       ew_publish(bars + B_DSF + half);
       __syncwarp();   // this warp is done with the statistics of step j

@@ -23,10 +23,7 @@
 
 namespace lg {
 
-#ifndef LG_DEC_WARPS
-#define LG_DEC_WARPS 8
-#endif
-constexpr int kDecWarps = LG_DEC_WARPS;   // warps per CTA, each with its own pipeline of tiles
+constexpr int kDecWarps = 8;          // warps per CTA, each with its own pipeline of tiles
 constexpr int kDecThreads = kDecWarps * 32;
 constexpr int kDecStages = 3;
 constexpr int kDecTile = 16;          // tokens per warp tile

@@ -83,16 +83,11 @@ __device__ __forceinline__ void header_begin(WsHeader* h) {
   h->fingerprint = 0;
 }
 
-// oldest block the documents leave to query block qb (see block_active: block kb is dropped when it ends at or
-// before the start of the block's earliest document)
+// Oldest block the documents leave to query block qb.  The first row of a query block belongs to the earliest document
+// of the block, so it sees the most: a key block that ends before that document starts holds nothing any row of the
+// block may see.  (A superset of the blocks that are really needed; what is left over is masked in the kernels.)
 __device__ __forceinline__ int doc_first_block(const PatternDev& p, int qb) {
   return p.doc_start ? max(p.doc_start[qb * p.block], 0) / p.block : 0;
-}
-__device__ __forceinline__ bool pattern_active(const PatternDev& p, int qb, int kb) {
-  if (kb > qb) return false;
-  if (p.mode == 0) return true;
-  if (p.mode == 1) return kb < p.ns || qb - kb < p.nw;
-  return qb - kb < p.nl || kb % p.stride == 0;
 }
 
 // The ascending union of the lists of pattern rows r0 .. r0 + n - 1 (n <= 4) as `kb * mul + member mask`; one warp.
@@ -114,7 +109,7 @@ __device__ __forceinline__ int merge_rows(const PatternDev& p, int r0, int n, in
     if (kb < hi) {
 #pragma unroll
       for (int r = 0; r < 4; ++r)
-        if (kb >= first[r] && pattern_active(p, r0 + r, kb)) mask |= 1 << r;   // (first[r] = INT_MAX: no such row)
+        if (kb >= first[r] && block_active(p, r0 + r, kb)) mask |= 1 << r;   // (first[r] = INT_MAX: no such row)
     }
     const unsigned m = __ballot_sync(0xffffffffu, mask != 0);
     if (mask) out[written + __popc(m & ((1u << lane) - 1))] = kb * mul + mask;
@@ -151,7 +146,7 @@ __device__ __forceinline__ int dq_entries(const PatternDev& p, int R, int n_ktil
 #pragma unroll
         for (int m = 0; m < 2; ++m) {
           const int qb = R * t + m;
-          if (m >= R || c < first[m] || !pattern_active(p, qb, c)) continue;   // (first[m] = INT_MAX: no such row)
+          if (m >= R || c < first[m] || !block_active(p, qb, c)) continue;   // (first[m] = INT_MAX: no such row)
           q[2 * n + m] = col_pos(p, qb, c);
           any = true;
         }
@@ -182,8 +177,8 @@ __device__ __forceinline__ int merge_cols(const PatternDev& p, int ca, int cb, i
     int mask = 0;
     if (qb < hi) {
       const int first = doc_first_block(p, qb);
-      if (ca >= first && pattern_active(p, qb, ca)) mask |= 1;
-      if (cb >= first && cb >= 0 && pattern_active(p, qb, cb)) mask |= 2;
+      if (ca >= first && block_active(p, qb, ca)) mask |= 1;
+      if (cb >= first && cb >= 0 && block_active(p, qb, cb)) mask |= 2;
     }
     const unsigned m = __ballot_sync(0xffffffffu, mask != 0);
     if (mask) out[written + __popc(m & ((1u << lane) - 1))] = qb * 4 + mask;
