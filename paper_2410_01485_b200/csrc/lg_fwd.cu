@@ -4,7 +4,7 @@
 
 namespace lg {
 
-template <int D, int BS>
+template <int D, int BS, int NB>
 static lg_status launch_fwd_t(const Resolved& r, const WsLayout& w, const void* q, const void* k, const void* v,
                               void* o, float* lse, uint8_t* ws, cudaStream_t stream) {
   CUtensorMap tq, tk, tv;
@@ -32,7 +32,7 @@ static lg_status launch_fwd_t(const Resolved& r, const WsLayout& w, const void* 
   a.doc_start = r.doc_start;
   a.scale_log2 = r.scale * 1.4426950408889634f;
   a.head_group = head_group(r, r.B * r.Hq);
-  auto kern = fwd_kernel<D, BS>;
+  auto kern = fwd_kernel<D, BS, NB>;
   constexpr int smem = FwdSmem<D>::kTotal;
   static std::atomic<bool> allowed[kMaxDevices];
   dim3 grid(r.B * r.Hq, r.n_stiles);
@@ -42,10 +42,16 @@ static lg_status launch_fwd_t(const Resolved& r, const WsLayout& w, const void* 
 lg_status launch_fwd(const Resolved& r, const WsLayout& w, const void* q, const void* k, const void* v, void* o,
                      float* lse, uint8_t* ws, cudaStream_t stream) {
   if (r.n_qtiles > 65535) return LG_ERR_UNSUPPORTED;
-  if (r.D == 128 && r.block == 128) return launch_fwd_t<128, 128>(r, w, q, k, v, o, lse, ws, stream);
-  if (r.D == 128 && r.block == 64) return launch_fwd_t<128, 64>(r, w, q, k, v, o, lse, ws, stream);
-  if (r.D == 64 && r.block == 128) return launch_fwd_t<64, 128>(r, w, q, k, v, o, lse, ws, stream);
-  if (r.D == 64 && r.block == 64) return launch_fwd_t<64, 64>(r, w, q, k, v, o, lse, ws, stream);
+  const bool pairs = fwd_two_ctas(r);
+#define LG_FWD_CASE(DD, BB, NN) \
+  if (r.D == DD && r.block == BB && pairs == (NN == 1)) return launch_fwd_t<DD, BB, NN>(r, w, q, k, v, o, lse, ws, stream);
+  LG_FWD_CASE(128, 128, 2)
+  LG_FWD_CASE(128, 64, 2)
+  LG_FWD_CASE(64, 128, 1)
+  LG_FWD_CASE(64, 128, 2)
+  LG_FWD_CASE(64, 64, 1)
+  LG_FWD_CASE(64, 64, 2)
+#undef LG_FWD_CASE
   return LG_ERR_UNSUPPORTED;
 }
 

@@ -17,10 +17,12 @@
 // tensor pipe computes the other, and the second slot fills what is left.
 // D = 64: the products of a half take 320 cycles of the tensor pipe where its exponentials take 512 of
 // the exponential unit, so the element-wise chain sets the pace, and what fills the unit is more rows in
-// work.  Two CTAs share an SM: each has half the tensor memory, one score buffer per slot (S of slot s at
-// 64 s, O at 128 + 64 s; S(0) | PV(0) S(1) | PV(1) S(2) | ...) and 80 registers per thread, hence the half
-// is worked 32 columns at a time (3 x 16 / 4 heads x 6001 tokens, window 1024: 169 -> 150 us).  The online softmax
-// advances half by half.  A row's reference (the maximum its probabilities are expressed relative
+// work.  Grids that fill the chip several times over (fwd_two_ctas, lg_host.h) therefore run two CTAs on an SM (NB = 1):
+// each has half the tensor memory, one score buffer per slot (S of slot s at 64 s, O at 128 + 64 s;
+// S(0) | PV(0) S(1) | PV(1) S(2) | ...) and 80 registers per thread, hence the half is worked 32 columns at a time (3 x 16 /
+// 4 heads x 6001 tokens, window 1024: 164 -> 148 us with 64- and with 128-token blocks, although 13 / 34 registers are
+// spilled there).  Both forms sum in the same order and give the same bits.
+// The online softmax advances half by half.  A row's reference (the maximum its probabilities are expressed relative
 // to) only moves, and O is only rescaled, when a half's probabilities sum to more than 2^8;
 // until then they are relative to the older reference, which fp32 / bf16 hold easily, and the
 // row maximum is not computed at all.
@@ -58,8 +60,7 @@ struct FwdArgs {
 constexpr int kFwdTmaWarp = 8, kFwdMmaWarp0 = 9;
 constexpr int kFwdThreads = 11 * 32;
 constexpr float kFwdMaxProb = 256.0f;   // a half's probabilities may grow to this (relative to the row's reference) before the reference moves
-template <int D> constexpr int kFwdBufs = D == 64 ? 1 : 2;        // score buffers per slot
-template <int D> constexpr int kFwdCtasPerSm = D == 64 ? 2 : 1;
+constexpr int fwd_ctas_per_sm(int bufs) { return bufs == 1 ? 2 : 1; }   // one score buffer per slot: the form of which two share an SM
 template <int D>
 struct FwdSmem {
   static constexpr int kBox = 128 * 128;               // one 64-column box of 128 rows
@@ -72,8 +73,8 @@ struct FwdSmem {
   static constexpr int kTotal = oBar + 256;
 };
 
-template <int D, int BS>
-__global__ void __launch_bounds__(kFwdThreads, kFwdCtasPerSm<D>)
+template <int D, int BS, int NB /* score buffers per slot */>
+__global__ void __launch_bounds__(kFwdThreads, fwd_ctas_per_sm(NB))
 fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
            const __grid_constant__ CUtensorMap tm_v, const FwdArgs a) {
   using SM = FwdSmem<D>;
@@ -81,8 +82,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   constexpr int RS = R4 / 2;                    // pattern rows per slot
   constexpr uint32_t kSlotMask = (1u << RS) - 1u;
   constexpr int kTile = SM::kTile;
-  constexpr int NB = kFwdBufs<D>;
-  constexpr uint32_t kColS = 0, kSlotS = 64 * NB, kColO = 2 * kSlotS, kTmemCols = kColO + 2 * D;
+  constexpr uint32_t kColS = 0, kSlotS = 64 * NB, kColO = 2 * kSlotS, kTmemCols = NB == 1 ? 256 : 512;
   // SF / PF / OD are indexed [slot * 2 + buffer].  A parity wait is only meaningful while the barrier
   // is at most one phase behind the waiter; per half buffer that holds by construction (the S
   // product that re-fills a half is queued behind the P V product that read it), which is why
@@ -93,7 +93,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SM::oBar);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + B_COUNT);
   static_assert(B_COUNT * 8 + 8 <= 256, "barrier area too small");
-  static_assert(kFwdCtasPerSm<D> * (SM::kTotal + 1024) <= 228 * 1024 && kFwdCtasPerSm<D> * kTmemCols <= 512, "does not fit an SM");
+  static_assert(fwd_ctas_per_sm(NB) * (SM::kTotal + 1024) <= 228 * 1024 && kColO + 2 * D <= kTmemCols, "does not fit an SM");
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // same value, known to be warp-uniform
   pdl_trigger();

@@ -135,12 +135,29 @@ int head_group(const Resolved& r, int n_x);
 size_t ds_buffer_bytes(const Resolved& r);
 
 
-// Whether the attention kernels of a problem are launched overlapped: up to two waves of the forward.  Their prologues
+// Whether the attention kernels of a problem are launched overlapped: up to two forward CTAs per SM.  Their prologues
 // and launch latencies then weigh something (2 heads x 512 tokens fwd + bwd 36.9 -> 35.9 us, steps of 40-50 us by
 // 4-18 %).  Large ones gain nothing and lose 1-2 % (full causal, 32 heads x 16K: 8.55 -> 8.63 ms): CTAs that
 // arrive as SMs fall free are spread over the chip in another order than those of an ordinary launch.
 inline bool launch_attn_overlapped(const Resolved& r) {
-  return static_cast<long long>(r.B) * r.Hq * r.n_stiles <= 2 * 148;
+  return static_cast<long long>(r.B) * r.Hq * r.n_stiles <= 2 * kSms;
+}
+
+// Which form of the forward a D = 64 problem takes (lg_fwd.cuh; both give the same bits).  Two CTAs on an SM hide each
+// other's latencies, but one of them alone is 1.3-1.4 times as slow as the form that has the SM to itself, so they need
+// a grid that keeps the pairs together until near its end.  Rounds of one CTA per SM from which the pairs are
+// faster, measured over 230 problems of 8 to 7552 CTAs (time of the single form over that of the pairs):
+//   rows of up to 512 keys on average       1.25   (208 CTAs 1.05-1.08, 128 CTAs 0.80-0.90)
+//   up to 1152                              2      (window 1024: 416-528 CTAs 1.00-1.05, 128 CTAs 0.77-0.82)
+//   longer rows                             4      (windows 2500-4096: 388-592 CTAs 0.91-1.00, 620-2048 CTAs 1.00-1.11)
+//   full causal, lengths from 1 to L / 128  16     (1024 CTAs 0.89-0.95, 2048 CTAs 0.98-1.03, 4096 and more 1.00-1.13)
+// 4 heads x 3318 tokens, full causal, 52 CTAs: 74 us in pairs, 53 us alone; 3 x 16 heads x 6001, window 1024, 1152 CTAs:
+// 148 us in pairs, 164 us alone.
+inline bool fwd_two_ctas(const Resolved& r) {
+  if (r.D != 64) return false;
+  const int64_t ctas = static_cast<int64_t>(r.B) * r.Hq * r.n_stiles, keys = r.nnz * r.block / r.pat.nB;
+  const int quarter_rounds = r.mode == LG_MODE_FULL_CAUSAL ? 64 : keys > 1152 ? 16 : keys > 512 ? 8 : 5;
+  return 4 * ctas > quarter_rounds * static_cast<int64_t>(kSms);
 }
 
 lg_status check_arch();

@@ -6,6 +6,10 @@
 
 namespace lg {
 
+// SMs of a B200, for rules that size a grid.  Fixed and not asked of the device: workspace sizes follow from some of them
+// and must come out the same without a GPU, and so must the bits of a result.
+constexpr int kSms = 148;
+
 struct PatternDev {
   int nB;       // ceil(L / block)
   int mode;     // 0 full causal, 1 sink+window, 2 strided+local
@@ -154,7 +158,7 @@ struct KvSplit {
 // with a sorted copy of the lengths, a backward call over 2 heads x 128K tokens, window 4096, took 75 us of host time; 26).
 inline KvSplit kv_split(const PatternDev& p, int n_ktiles, int G, int64_t nnz, int kv_total) {
   KvSplit k{};
-  constexpr int kSms = 148, kCta = 8, kMinLen = 16;
+  constexpr int kCta = 8, kMinLen = 16;
   const int R = 128 / p.block, per_item = p.block / 64;        // half-steps of an item
   const int64_t per_entry = static_cast<int64_t>(G) * per_item;
   // a bound first, without looking at the tiles: none is longer than twice the rows, and two columns share entries

@@ -43,3 +43,22 @@ def test_rising_scores_and_ragged_lengths(lg, L, block, exact):
     err = np.abs(synth.to_f64(o[0]) - Oo)
     assert (err <= 2.0 ** -8 * (np.abs(Oo) + Av) + 1e-3).all(), err.max()
     assert np.abs(synth.to_f64(lse[0]) - LSE).max() <= TOL_LSE
+
+
+@pytest.mark.parametrize("L", [1, 63, 257, 1000])
+@pytest.mark.parametrize("block,exact", [(64, False), (64, True), (128, False)])
+def test_both_forms_give_the_same_bits(lg, L, block, exact):
+    """A batch of eight runs two CTAs on an SM, one of its sequences has an SM per CTA (fwd_two_ctas, csrc/lg_host.h):
+    groups of a problem's heads or sequences must come out as in the whole."""
+    cfg = replace(synth.CFG1, name="forms", B=8, L=L, D=64, Hq=32, Hkv=8, block=block, sink_tokens=block, window_tokens=2 * block,
+                  window_exact=exact)
+    inp = synth.make_attn_inputs(cfg, "cuda", seed=L)
+    k = inp["k"]
+    for i, at in enumerate((20, 52, 300, 900)):
+        if at < L:
+            k[:, :, at] = inp["q"][:, ::4, min(L - 1, at + 40)] * (1.5 + i)
+    o, lse = lg.lg_sparse_attn_fwd(lg.params_of(cfg), inp["q"], k, inp["v"])
+    one = replace(cfg, B=1)
+    for b in range(cfg.B):
+        ob, lb = lg.lg_sparse_attn_fwd(lg.params_of(one), *(t[b:b + 1] for t in (inp["q"], k, inp["v"])))
+        assert torch.equal(ob[0], o[b]) and torch.equal(lb[0], lse[b])
