@@ -889,6 +889,11 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int dend = (a.doc_end && kb_mine >= 0 && kj < a.L) ? a.doc_end[static_cast<int64_t>(b) * a.L + kj] : a.L;
     const uint32_t lane_addr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
     const uint64_t scale2 = f32x2(a.scale_log2, a.scale_log2);
+    // A half-step whose queries see only the tile's other column is left out where half a step is long enough to be worth
+    // a branch.  Measured, dK/dV pass with and without it: 16 heads x 32K in documents 1055 / 1062 us, 16 / 8 heads x 24K,
+    // stride 8, 765 / 770 us; at D = 64 it costs what it saves and more: 32 / 8 heads x 8K, full causal, 839 / 802 us,
+    // window 3136 209 / 199 us.  (128-token blocks: a tile is one column.)
+    constexpr bool kSkipOff = D == 128 && BS == 64;
     uint64_t evict_first = 0;
     if (kSpill) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(evict_first));
     bool ok = true;
@@ -906,7 +911,7 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       const int entry = sEnt[(j & 1) * 2 + (BS == 64 ? col0 / 64 : 0)];
       const int q0 = (entry >> 2) * BS + (BS == 128 ? col0 : col0 % 64);
       const bool on = (entry >> member) & 1;                   // (the same for all rows of a warp)
-      const int xmin = min(max(kj - q0, 0), C);                // columns xmin <= c < xmax are visible (of a member that is on)
+      const int xmin = on ? min(max(kj - q0, 0), C) : C;      // columns xmin <= c < xmax are visible
       const int hi_abs = (a.exact_w > 0 && kb_mine >= a.ns) ? min(dend, kj + a.exact_w) : dend;   // first query that no longer sees me
       const int xmax = min(max(hi_abs - q0, 0), C);
       const uint32_t s_addr = lane_addr + kColS + half * kKvHalf + g * C;
@@ -916,10 +921,9 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      if (!on) {
+      if (kSkipOff && !on) {
         // The tile's other column alone sees these queries (most steps of a sink or comb column whose neighbour is
-        // an ordinary one): P and dS of mine are zero without being computed (and a block that is not in the pattern
-        // has no tile to keep).
+        // an ordinary one): P and dS of mine are zero without being computed.
         const uint32_t zero[C / 2] = {};
         tmem_st16(s_addr, zero);
         ew_publish(bars + B_PF + half);
@@ -1001,12 +1005,15 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // ... and to this half-step's tile in global memory: my C queries are C / 8 16-byte groups of my
         // key.  (Written once, read once by the dQ pass: marked evict-first so that the stream does not
         // push the Q / dO tiles, which every kv tile of a window re-reads, out of the L2.)
-        uint8_t* dst = reinterpret_cast<uint8_t*>(a.ds_buf) + sTile[(j & 1) * 4 + half * 2 + member] * kDsTileBytes<BS> +
-                       (C / 8 * g) * (16 * BS) + (r & (BS - 1)) * 16;
+        // (a member the entry does not list has no block, hence no tile: its dS is zero and stays unwritten)
+        if (kSkipOff || on) {
+          uint8_t* dst = reinterpret_cast<uint8_t*>(a.ds_buf) + sTile[(j & 1) * 4 + half * 2 + member] * kDsTileBytes<BS> +
+                         (C / 8 * g) * (16 * BS) + (r & (BS - 1)) * 16;
 #pragma unroll
-        for (int i = 0; i < C / 8; ++i)
-          asm volatile("st.global.L2::cache_hint.v4.b32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(dst + i * (16 * BS)),
-                       "r"(dsreg[4 * i]), "r"(dsreg[4 * i + 1]), "r"(dsreg[4 * i + 2]), "r"(dsreg[4 * i + 3]), "l"(evict_first) : "memory");
+          for (int i = 0; i < C / 8; ++i)
+            asm volatile("st.global.L2::cache_hint.v4.b32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(dst + i * (16 * BS)),
+                         "r"(dsreg[4 * i]), "r"(dsreg[4 * i + 1]), "r"(dsreg[4 * i + 2]), "r"(dsreg[4 * i + 3]), "l"(evict_first) : "memory");
+        }
       }
       ew_publish(bars + B_DSF + half);
       __syncwarp();   // this warp is done with the statistics of step j
