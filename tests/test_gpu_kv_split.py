@@ -1,6 +1,7 @@
 """The dK/dV pass with kv tiles cut into pieces (few kv heads, long tiles): both block sizes and head sizes, every
 pattern, ragged lengths, grouped queries, documents (tiles shorter than planned), both backward variants; the host-buffer
-step in head groups gives the same bits as the whole problem."""
+step in head groups gives the same bits as the whole problem.  (test_kv_split_rule.py checks that these problems are cut,
+and that the groups alone would be cut otherwise.)"""
 from dataclasses import replace
 
 import numpy as np
@@ -42,9 +43,7 @@ def _check(got, ref, what):
 @pytest.mark.parametrize("cfg", CASES, ids=lambda c: c.name)
 def test_split_tiles_parity(lg, cfg, docs, variant, monkeypatch):
     monkeypatch.setenv("LG_BWD_VARIANT", variant)
-    if docs and cfg.B > 1:
-        pytest.skip("documents run sequence by sequence")
-    ds = synth.make_doc_start(cfg.L, seed=5, mean_len=500)[None].cuda() if docs else None
+    ds = torch.stack([synth.make_doc_start(cfg.L, seed=5 + b, mean_len=500) for b in range(cfg.B)]).cuda() if docs else None
     p = lg.params_of(cfg, doc_start=ds)
     inp = synth.make_attn_inputs(cfg, "cuda", seed=2, with_do=True)
     ws = lg.attn_workspace(p, True)
@@ -53,18 +52,22 @@ def test_split_tiles_parity(lg, cfg, docs, variant, monkeypatch):
     again = lg.lg_sparse_attn_bwd(p, inp["q"], inp["k"], inp["v"], o, lse, inp["do"], workspace=ws)
     assert lg.lg_last_status(ws) == 0
     assert all(torch.equal(x, y) for x, y in zip(grads, again))         # the pieces are added in a fixed order
-    pat = O.Pattern.of(cfg)
-    if docs:
-        pat = replace(pat, doc_start=ds[0].cpu().numpy())
     for b in range(cfg.B):
+        pat = O.Pattern.of(cfg)
+        if docs:
+            pat = replace(pat, doc_start=ds[b].cpu().numpy())
         q, k, v, do = (synth.to_f64(inp[x][b]) for x in ("q", "k", "v", "do"))
         refs = O.attn_backward(q, k, v, do, pat, 1.0 / np.sqrt(cfg.D), rows_per_slab=cfg.block)[:3]
         for x, ref, what in zip(grads, refs, ("dQ", "dK", "dV")):
             _check(x[b], ref, what)
 
 
+GROUPS = replace(synth.CFG1, name="groups", mode=synth.MODE_FULL_CAUSAL, L=4096, D=64, Hq=8, Hkv=4, block=64)
+DOC_GROUPS = replace(synth.CFG1, name="doc_groups", B=2, L=6000, D=64, Hq=16, Hkv=4, block=64, sink_tokens=64, window_tokens=1024)
+
+
 def test_head_groups_of_the_host_step_split_like_the_whole(lg):
-    cfg = replace(synth.CFG1, name="groups", L=3000, D=64, Hq=8, Hkv=4, block=64, sink_tokens=64, window_tokens=256)
+    cfg = GROUPS
     p = lg.params_of(cfg)
     inp = synth.make_attn_inputs(cfg, "cuda", seed=12, with_do=True)
     o, lse = lg.lg_sparse_attn_fwd(p, inp["q"], inp["k"], inp["v"])
@@ -82,7 +85,7 @@ def test_head_groups_of_the_host_step_split_like_the_whole(lg):
 def test_head_groups_with_documents_in_several_sequences(lg, groups):
     """Documents in a batch of two (run sequence by sequence), 16 / 4 heads: a whole sequence is cut into pieces of 48
     items, two or four kv heads on their own would be cut into 24 or 16."""
-    cfg = replace(synth.CFG1, name="doc_groups", B=2, L=6000, D=64, Hq=16, Hkv=4, block=64, sink_tokens=64, window_tokens=1024)
+    cfg = DOC_GROUPS
     ds = torch.stack([synth.make_doc_start(cfg.L, seed=30 + b, mean_len=5000) for b in range(2)]).cuda()
     p = lg.params_of(cfg, doc_start=ds)
     inp = synth.make_attn_inputs(cfg, "cuda", seed=14, with_do=True)

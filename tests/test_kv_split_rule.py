@@ -8,6 +8,7 @@ import subprocess
 import pytest
 
 from paper_2410_01485_b200 import binding, build
+from tests.test_gpu_kv_split import CASES, DOC_GROUPS, GROUPS
 
 
 @pytest.fixture(scope="module")
@@ -141,3 +142,19 @@ def test_places_stay_within_a_grid(rule, block, mode, a, b, kv):
     assert max(places for _, places, _, _ in got) <= 65535
     assert got[-1][0] == 0                                             # 65535 tiles leave no place to spare
     assert all(x[3] == 0 for x in got)
+
+
+def _problem(cfg, kv_heads):
+    a, b = [(0, 0), (cfg.sink_tokens // cfg.block, cfg.window_tokens // cfg.block + bool(cfg.window_exact)),
+            (cfg.stride_blocks, cfg.local_blocks)][cfg.mode]
+    return -(-cfg.L // cfg.block), cfg.block, cfg.mode, a, b, cfg.Hq // cfg.Hkv, kv_heads, -(-cfg.L // 128)
+
+
+def test_the_gpu_tests_problems_are_cut(rule):
+    """Those of the parity test, whether the whole batch counts or (with documents) a sequence of it; and where groups of
+    heads are compared with the whole, a group by itself would be cut into other pieces."""
+    for cfg in CASES:
+        assert all(x[0] > 0 for x in rule([_problem(cfg, n * cfg.Hkv) for n in {1, cfg.B}])), cfg.name
+    for cfg, groups in ((GROUPS, (2, 4)), (DOC_GROUPS, (2, 4))):
+        whole, *parts = (x[0] for x in rule([_problem(cfg, cfg.Hkv // n) for n in (1, *groups)]))
+        assert whole > 0 and all(0 < x != whole for x in parts), (cfg.name, whole, parts)
