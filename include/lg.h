@@ -194,7 +194,9 @@ lg_status lg_sparse_attn_bwd_marked(const lg_attn_params* p, const void* q, cons
  *                    hand-over between the streams and destroys them before returning.  On
  *                    return everything is enqueued; the host results are complete when
  *                    stream_out is idle (stream_in and stream_compute are then idle too).
- * Results are bit-identical to the two device calls on the whole tensors.  lg_last_status() on
+ * Results are bit-identical to the two device calls on the whole tensors: what those choose by
+ * the problem's size (the backward variant, cut tiles) is chosen here for the whole problem and
+ * holds for every group.  lg_last_status() on
  * dev->workspace reports a device-side failure of any group.
  */
 typedef struct {

@@ -155,9 +155,10 @@ int sm_count() {
 // strided pattern at 128K, 73 GB, still keep dS), 48 GB where no device can be asked.
 // LG_BWD_VARIANT = two_pass | keep_ds overrides the choice (read at every call; it must not change between
 // a size query, a prepare and the calls that use them).
-size_t ds_buffer_bytes(const Resolved& r) {   // 2 bytes per pair of every block of the pattern and query head, plus one tile of zeros at the end
-  return static_cast<size_t>(r.B) * r.Hq * static_cast<size_t>(r.nnz) * r.block * r.block * 2 + 128 * 64 * 2;
+static size_t ds_bytes_of(const Resolved& r, size_t heads) {   // 2 bytes per pair of every block of the pattern and query head, plus one tile of zeros at the end
+  return heads * static_cast<size_t>(r.nnz) * r.block * r.block * 2 + 128 * 64 * 2;
 }
+size_t ds_buffer_bytes(const Resolved& r) { return ds_bytes_of(r, static_cast<size_t>(r.B) * r.Hq); }
 
 // largest dS buffer the default choice accepts, in bytes
 double keep_ds_limit() {
@@ -179,7 +180,8 @@ BwdVariant bwd_variant(const Resolved& r) {
   // (per-sequence lists have no common tile numbering)
   const bool can_keep = !(r.doc_start != nullptr && r.B > 1);
   if (env && strcmp(env, "keep_ds") == 0) return can_keep ? kBwdKeepDs : kBwdTwoPass;
-  return (can_keep && static_cast<double>(ds_buffer_bytes(r)) <= keep_ds_limit()) ? kBwdKeepDs : kBwdTwoPass;
+  // (the buffer of the whole problem: its groups of heads run the same variant, and their buffers exist side by side)
+  return (can_keep && static_cast<double>(ds_bytes_of(r, static_cast<size_t>(r.kv_total) * r.G)) <= keep_ds_limit()) ? kBwdKeepDs : kBwdTwoPass;
 }
 
 WsLayout ws_layout(const Resolved& r, bool want_bwd) {
@@ -399,6 +401,7 @@ __global__ void wait_selftest_kernel(unsigned int* error_word, long long limit_c
 static Resolved one_sequence(const Resolved& r, int b, void* workspace) {
   Resolved r1 = r;
   r1.B = 1;
+  r1.kv_total = r.kv_total / r.B;
   r1.doc_start = r.doc_start + static_cast<int64_t>(b) * r.L;
   r1.error_word = r.error_word ? r.error_word : static_cast<unsigned int*>(workspace);
   return r1;

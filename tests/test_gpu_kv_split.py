@@ -97,3 +97,22 @@ def test_head_groups_with_documents_in_several_sequences(lg, groups):
     torch.cuda.synchronize()
     for name, t in ref.items():
         assert torch.equal(out[name], t.cpu()), (groups, name)
+
+
+def test_head_groups_run_the_backward_of_the_whole(lg, monkeypatch):
+    """A limit on the dS buffer that the whole problem exceeds and a group of its heads does not.  (A strided pattern: its
+    kv tiles hold comb columns first, so the variants sum dQ in different orders.)"""
+    cfg = replace(GROUPS, mode=synth.MODE_STRIDED_LOCAL, stride_blocks=4, local_blocks=2)
+    p = lg.params_of(cfg)
+    ds = cfg.Hq * lg.lg_block_index_nnz(p) * cfg.block * cfg.block * 2
+    monkeypatch.setenv("LG_KEEP_DS_MAX_GB", "%.6f" % (0.5 * ds / 1e9))
+    assert lg.bwd_variant_name(p) == "two_pass"
+    inp = synth.make_attn_inputs(cfg, "cuda", seed=15, with_do=True)
+    o, lse = lg.lg_sparse_attn_fwd(p, inp["q"], inp["k"], inp["v"])
+    ref = dict(zip(("o", "lse", "dq", "dk", "dv"), (o, lse) + lg.lg_sparse_attn_bwd(p, inp["q"], inp["k"], inp["v"], o, lse, inp["do"])))
+    host = {k: v.cpu().pin_memory() for k, v in inp.items()}
+    out = {n: torch.zeros(t.shape, dtype=t.dtype).pin_memory() for n, t in ref.items()}
+    lg.sparse_attn_fwd_bwd_host(lg.params_of(cfg), host, out, head_groups=4)
+    torch.cuda.synchronize()
+    for name, t in ref.items():
+        assert torch.equal(out[name], t.cpu()), name

@@ -158,3 +158,18 @@ def test_the_gpu_tests_problems_are_cut(rule):
     for cfg, groups in ((GROUPS, (2, 4)), (DOC_GROUPS, (2, 4))):
         whole, *parts = (x[0] for x in rule([_problem(cfg, cfg.Hkv // n) for n in (1, *groups)]))
         assert whole > 0 and all(0 < x != whole for x in parts), (cfg.name, whole, parts)
+
+
+@pytest.mark.parametrize("groups", [1, 2, 4])
+def test_groups_of_the_host_step_keep_ds_like_the_whole(lib, groups, monkeypatch):
+    """Which backward runs is decided for the whole problem: its groups' results are bit-identical to it, and the limit
+    on the dS buffer holds for what the groups' workspaces take together."""
+    p = binding.attn_params(1, 16, 4, 8192, 128, 128, binding.MODE_SINK_WINDOW, sink_tokens=128, window_tokens=1024)
+    ds = 16 * binding.lg_block_index_nnz(p) * 128 * 128 * 2
+    monkeypatch.delenv("LG_BWD_VARIANT", raising=False)
+    sizes = []
+    for cap in (0.9 * ds, 1.1 * ds):                       # below the whole's buffer (and above any group's), and above it
+        monkeypatch.setenv("LG_KEEP_DS_MAX_GB", "%.6f" % (cap / 1e9))
+        assert lib.lg_sparse_attn_bwd_variant(C.byref(p)) == (0 if cap < ds else 2)
+        sizes.append(lib.lg_sparse_attn_fwd_bwd_host_workspace_bytes(C.byref(p), groups))
+    assert ds <= sizes[1] - sizes[0] < ds + (1 << 20)
