@@ -150,7 +150,8 @@ lg_status lg_sparse_attn_bwd(const lg_attn_params* p, const void* q, const void*
  * writes dS (bf16, 2 bytes per pair of every block of the pattern and query head) to the workspace and
  * the dQ pass is the single product dQ = dS K.  The second is chosen when that buffer takes at most
  * 40 % of the current device's memory (or LG_KEEP_DS_MAX_GB gigabytes, where the environment sets it;
- * 48 GB where no device can be asked) and the block lists are shared by the batch; the environment
+ * 48 GB where no device can be asked); with doc_start and B > 1, where the call runs sequence by
+ * sequence, that of one sequence counts.  The environment
  * variable LG_BWD_VARIANT = two_pass | keep_ds overrides the choice.  Both give bitwise reproducible
  * results; they differ from one another in the last bits (dS is rounded to bf16 once either way, but the
  * order of the fp32 sums differs).  < 0 = lg_status.  (The paper has no counterpart.)            */

@@ -149,7 +149,7 @@ int sm_count() {
 // Two backward variants compute the same gradients (see BwdVariant).  The two passes run everywhere.
 // Keeping dS trades workspace and HBM traffic (2 bytes per visible pair, written once and read once, on
 // a memory system the attention kernels otherwise leave idle) for the two recomputed products of the dQ
-// pass.  It is the default when the lists are shared by the batch and the dS buffer takes at most
+// pass.  It is the default when the dS buffer (of one sequence, where documents make them run one by one) takes at most
 // LG_KEEP_DS_MAX_GB gigabytes (the buffer holds every block of the pattern in full); without the variable
 // the limit is 40 % of the current device's memory (77 GB of a B200's 192e9 bytes: 64 query heads of the
 // strided pattern at 128K, 73 GB, still keep dS), 48 GB where no device can be asked.
@@ -177,11 +177,9 @@ double keep_ds_limit() {
 BwdVariant bwd_variant(const Resolved& r) {
   const char* env = getenv("LG_BWD_VARIANT");
   if (env && strcmp(env, "two_pass") == 0) return kBwdTwoPass;
-  // (per-sequence lists have no common tile numbering)
-  const bool can_keep = !(r.doc_start != nullptr && r.B > 1);
-  if (env && strcmp(env, "keep_ds") == 0) return can_keep ? kBwdKeepDs : kBwdTwoPass;
+  if (env && strcmp(env, "keep_ds") == 0) return kBwdKeepDs;
   // (the buffer of the whole problem: its groups of heads run the same variant, and their buffers exist side by side)
-  return (can_keep && static_cast<double>(ds_bytes_of(r, static_cast<size_t>(r.kv_total) * r.G)) <= keep_ds_limit()) ? kBwdKeepDs : kBwdTwoPass;
+  return static_cast<double>(ds_bytes_of(r, static_cast<size_t>(r.kv_total) * r.G)) <= keep_ds_limit() ? kBwdKeepDs : kBwdTwoPass;
 }
 
 WsLayout ws_layout(const Resolved& r, bool want_bwd) {
@@ -461,7 +459,8 @@ size_t lg_sparse_attn_workspace_bytes(const lg_attn_params* p, int want_bwd) { r
 int32_t lg_sparse_attn_bwd_variant(const lg_attn_params* p) {
   Resolved r;
   lg_status s = resolve(p, &r);
-  return s == LG_OK ? static_cast<int32_t>(bwd_variant(r)) : static_cast<int32_t>(s);
+  if (s != LG_OK) return static_cast<int32_t>(s);
+  return static_cast<int32_t>(bwd_variant(per_sequence(r) ? one_sequence(r, 0, nullptr) : r));
 }
 
 lg_status lg_sparse_attn_prepare(const lg_attn_params* p, void* workspace, size_t workspace_bytes, int want_bwd,

@@ -173,3 +173,21 @@ def test_groups_of_the_host_step_keep_ds_like_the_whole(lib, groups, monkeypatch
         assert lib.lg_sparse_attn_bwd_variant(C.byref(p)) == (0 if cap < ds else 2)
         sizes.append(lib.lg_sparse_attn_fwd_bwd_host_workspace_bytes(C.byref(p), groups))
     assert ds <= sizes[1] - sizes[0] < ds + (1 << 20)
+
+
+@pytest.mark.parametrize("B", [1, 2])
+def test_the_variant_reported_with_documents_is_the_one_that_runs(lib, B, monkeypatch):
+    """Sequence by sequence: a sequence's own dS buffer decides, and the answer agrees with the workspace."""
+    p = binding.attn_params(B, 16, 4, 8192, 128, 128, binding.MODE_SINK_WINDOW, sink_tokens=128, window_tokens=1024)
+    p.doc_start = 256                                      # (only its presence is looked at)
+    ds = 16 * binding.lg_block_index_nnz(p) * 128 * 128 * 2
+    sizes = {}
+    for variant in ("two_pass", "keep_ds"):
+        monkeypatch.setenv("LG_BWD_VARIANT", variant)
+        sizes[variant] = lib.lg_sparse_attn_workspace_bytes(C.byref(p), 1)
+    assert B * ds <= sizes["keep_ds"] - sizes["two_pass"] < B * (ds + (1 << 20))
+    monkeypatch.delenv("LG_BWD_VARIANT")
+    for cap, want in ((0.9 * ds, "two_pass"), (1.1 * ds, "keep_ds")):
+        monkeypatch.setenv("LG_KEEP_DS_MAX_GB", "%.6f" % (cap / 1e9))
+        assert binding.bwd_variant_name(p) == want
+        assert lib.lg_sparse_attn_workspace_bytes(C.byref(p), 1) == sizes[want]
