@@ -48,6 +48,9 @@ __device__ __forceinline__ void cp_async16(uint32_t smem_addr, const void* gptr,
   const int sz = valid ? 16 : 0;
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr), "l"(gptr), "r"(sz) : "memory");
 }
+__device__ __forceinline__ void prefetch_l2(const void* gptr, uint32_t bytes) {   // 16-byte aligned, a multiple of 16 bytes
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gptr), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
@@ -103,7 +106,7 @@ __device__ __forceinline__ void decode_run_segment(const DecodeArgs& a, uint8_t*
   int ex0 = 0, ex_cnt = 0;
   const int ring_w = a.C - a.sink;
   if (a.block_tokens > 0) {
-    const int64_t n = a.n_tokens[b];
+    const int64_t n = __ldcg(reinterpret_cast<const long long*>(a.n_tokens) + b);
     if (n > a.C) {                                  // before the ring has wrapped nothing is left out
       const int64_t first_held = n - ring_w;        // oldest window token in the ring (>= sink here)
       const int64_t first_kept = ((n - 1) / a.block_tokens - ring_w / a.block_tokens + 1) * a.block_tokens;
@@ -255,29 +258,39 @@ __device__ __forceinline__ void decode_run_segment(const DecodeArgs& a, uint8_t*
     }
   }
   __syncthreads();
-  for (int idx = threadIdx.x; idx < kDecHeads * D; idx += blockDim.x) {
-    const int head = idx / D, d = idx % D;
-    float m = -INFINITY;
+  {   // a warp per head: its weights once per thread, then D / 32 neighbouring values of a lane
+    static_assert(kDecWarps == kDecHeads && (D / 32) % 2 == 0, "a warp per head");
+    constexpr int V = D / 32;
+    const int head = warp, d = lane * V;
+    const float* mine = red + head * kRec;               // the head's row of warp 0's record
+    float f[kDecWarps], m = -INFINITY, l = 0.f, acc[V] = {};
 #pragma unroll
-    for (int w = 0; w < kDecWarps; ++w) m = fmaxf(m, red[(w * kDecHeads + head) * kRec + D]);
+    for (int w = 0; w < kDecWarps; ++w) { f[w] = mine[w * kDecHeads * kRec + D]; m = fmaxf(m, f[w]); }
     const float mu = m == -INFINITY ? 0.f : m;
-    float acc = 0.f, l = 0.f;
 #pragma unroll
     for (int w = 0; w < kDecWarps; ++w) {
-      const float f = fast_exp2(red[(w * kDecHeads + head) * kRec + D] - mu);
-      acc += f * red[(w * kDecHeads + head) * kRec + d];
-      l += f * red[(w * kDecHeads + head) * kRec + D + 1];
+      f[w] = fast_exp2(f[w] - mu);
+      l += f[w] * mine[w * kDecHeads * kRec + D + 1];
+#pragma unroll
+      for (int x = 0; x < V; x += 2) {
+        const float2 o2 = *reinterpret_cast<const float2*>(mine + w * kDecHeads * kRec + d + x);
+        acc[x] += f[w] * o2.x;
+        acc[x + 1] += f[w] * o2.y;
+      }
     }
     if (direct) {
       const int gh = hg * kDecHeads + head;
       if (gh < a.G) {
         const int64_t qh = static_cast<int64_t>(b) * a.Hq + kvh * a.G + gh;
-        a.o[qh * D + d] = __float2bfloat16(l > 0.f ? acc / l : 0.f);
-        if (d == 0 && a.lse) a.lse[qh] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+#pragma unroll
+        for (int x = 0; x < V; x += 2)
+          *reinterpret_cast<uint32_t*>(a.o + qh * D + d + x) = l > 0.f ? pack_bf16(acc[x] / l, acc[x + 1] / l) : 0u;
+        if (lane == 0 && a.lse) a.lse[qh] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
       }
     } else {
-      out[idx] = acc;
-      if (d == 0) { out[kDecHeads * D + 2 * head] = m; out[kDecHeads * D + 2 * head + 1] = l; }
+#pragma unroll
+      for (int x = 0; x < V; x += 2) *reinterpret_cast<float2*>(out + head * D + d + x) = make_float2(acc[x], acc[x + 1]);
+      if (lane == 0) { out[kDecHeads * D + 2 * head] = m; out[kDecHeads * D + 2 * head + 1] = l; }
     }
   }
 }
@@ -307,21 +320,25 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_split_kernel(const Deco
 // record of (CTA c, unit u) lives at index c + u, which grows strictly along the sequence.
 constexpr int kDecFlatMaxB = 2048;      // sequences the flattened path supports (prefix array in shared memory)
 constexpr int kDecFlatMaxCtas = 320;    // upper bound of its grid (two CTAs per SM)
+constexpr int kDecHintTiles = 3;        // tiles a warp asks for before the wait of an overlapped launch
 
+// (n_tokens is read through the L2: it is looked at once before the wait of an overlapped launch and again after it)
+__device__ __forceinline__ int decode_valid_of(const DecodeArgs& a, int b) {
+  const int64_t n = __ldcg(reinterpret_cast<const long long*>(a.n_tokens) + b);
+  return static_cast<int>(n < a.C ? (n < 0 ? 0 : n) : a.C);
+}
 __device__ __forceinline__ int decode_tiles_of(const DecodeArgs& a, int b) {
-  const int64_t n = a.n_tokens[b];
-  const int nvalid = static_cast<int>(n < a.C ? (n < 0 ? 0 : n) : a.C);
-  return (nvalid + kDecTile - 1) / kDecTile;
+  return (decode_valid_of(a, b) + kDecTile - 1) / kDecTile;
 }
 
 // cum[b] = tiles of the sequences before b, b = 0 .. B (block of kDecThreads threads; ends with a barrier).
-// Returns whether some sequence holds no token.
-__device__ __forceinline__ bool decode_build_cum(const DecodeArgs& a, int* cum) {
+// Returns whether some sequence holds no token; first: tiles of the thread's first sequence.
+__device__ __forceinline__ bool decode_build_cum(const DecodeArgs& a, int* cum, int& first) {
   __shared__ int warp_sum[kDecWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ipt = (a.B + kDecThreads - 1) / kDecThreads;
   const int b0 = tid * ipt;
-  const int first = b0 < a.B ? decode_tiles_of(a, b0) : 0;   // usually all of the thread's sequences
+  first = b0 < a.B ? decode_tiles_of(a, b0) : 0;             // usually all of the thread's sequences
   int local = first;
   bool empty = b0 < a.B && first == 0;
   for (int i = 1; i < ipt; ++i)
@@ -421,11 +438,43 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
   constexpr int kRec = D + 2;
   int* cum = reinterpret_cast<int*>(dsmem + kPipeBytes);
   // overlapped with the kernel before (an append, or the decode of the step before): append + decode of 16 sequences
-  // over 4224 slots, 64 / 8 heads, 53.7 -> 49.3 us a step, of one sequence 28.7 -> 13.7 us with the merge below
+  // over 4224 slots, 64 / 8 heads, 53.7 -> 49.3 us a step, of one sequence 28.7 -> 13.7 us with the merge below (then the hint)
   pdl_trigger();
-  pdl_wait();
-  const bool any_empty = decode_build_cum(a, cum);
   const int ups = a.Hkv * a.HG;
+  // Before the wait: a guess at my slice, from token counts that the kernel before may still be changing, and the first
+  // tiles of its warps asked into the L2, so that the HBM starts while the kernel before (an append, or the last merges of a
+  // decode) ends.  A hint only: nothing read here is used for more than addresses inside the caches, the L2 sees
+  // whatever is still written to the lines, and the counts are read again after the wait.  With one round trip less in the
+  // append and one fence a CTA instead of one a thread: append + decode of 16 sequences over 4224 slots, 64 / 8 heads,
+  // 49.2 -> 47.6 us, of one sequence 13.7 -> 12.8 us, of 4 linear caches of 9000 to 32768 tokens, 32 heads, 208.9 -> 206.4 us.
+  int tiles;
+  bool any_empty = decode_build_cum(a, cum, tiles);
+  {
+    const int64_t total = static_cast<int64_t>(cum[a.B]) * ups;
+    const int64_t f0 = total * blockIdx.x / gridDim.x, f1 = total * (blockIdx.x + 1) / gridDim.x;
+    if (f0 < f1 && (threadIdx.x & 31) < 2) {
+      int lo = 0, hi = a.B;
+      while (hi - lo > 1) {
+        const int mid = (lo + hi) >> 1;
+        if (static_cast<int64_t>(cum[mid]) * ups <= f0) lo = mid; else hi = mid;
+      }
+      const int nt = cum[lo + 1] - cum[lo];
+      const int64_t rel = f0 - static_cast<int64_t>(cum[lo]) * ups;
+      const int k = static_cast<int>(rel / nt), t0 = static_cast<int>(rel - static_cast<int64_t>(k) * nt);
+      const int n = static_cast<int>(min(static_cast<int64_t>(nt - t0), f1 - f0)), w = threadIdx.x >> 5;
+      const int tb = t0 + static_cast<int>(static_cast<int64_t>(n) * w / kDecWarps);
+      const int te = min(t0 + static_cast<int>(static_cast<int64_t>(n) * (w + 1) / kDecWarps), tb + kDecHintTiles);
+      const int slot0 = tb * kDecTile, rows = min(te * kDecTile, a.C) - slot0;
+      if (rows > 0) {
+        const __nv_bfloat16* base = (threadIdx.x & 1) ? a.v_cache : a.k_cache;
+        prefetch_l2(base + ((static_cast<int64_t>(lo) * a.Hkv + k / a.HG) * a.C + slot0) * D, rows * D * 2);
+      }
+    }
+  }
+  pdl_wait();
+  // (with more sequences than threads they are simply counted again)
+  const bool changed = a.B > kDecThreads || (threadIdx.x < a.B && decode_tiles_of(a, threadIdx.x) != tiles);
+  if (__syncthreads_or(changed)) any_empty = decode_build_cum(a, cum, tiles);
   const int64_t total = static_cast<int64_t>(cum[a.B]) * ups;
   __shared__ int s_merge[3];
   auto start_of = [&](int64_t c) { return total * c / gridDim.x; };
@@ -459,8 +508,7 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
     const int64_t rel = pos - static_cast<int64_t>(cum[b]) * ups;
     const int k = static_cast<int>(rel / nt), t0 = static_cast<int>(rel - static_cast<int64_t>(k) * nt);
     const int n = static_cast<int>(min(static_cast<int64_t>(nt - t0), f1 - pos));
-    const int64_t nn = a.n_tokens[b];
-    const int nvalid = static_cast<int>(nn < a.C ? (nn < 0 ? 0 : nn) : a.C);
+    const int nvalid = decode_valid_of(a, b);
     const int tb = t0 + static_cast<int>(static_cast<int64_t>(n) * warp / kDecWarps);
     const int te = t0 + static_cast<int>(static_cast<int64_t>(n) * (warp + 1) / kDecWarps);
     const int64_t u = static_cast<int64_t>(b) * ups + k;
@@ -472,9 +520,9 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
     if (direct) continue;
     // The CTA that delivers the last record of a unit merges it (records are read in index
     // order, so the result does not depend on which CTA that is) and re-arms the counter.
-    __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
+      __threadfence();   // (the CTA's stores, ordered before by the barrier)
       const int64_t first = static_cast<int64_t>(cum[b]) * ups + static_cast<int64_t>(k) * nt;
       const int c_lo = (t0 == 0) ? static_cast<int>(blockIdx.x) : cta_of(first);
       const int c_hi = (t0 + n == nt) ? static_cast<int>(blockIdx.x) : cta_of(first + nt - 1);
@@ -540,18 +588,19 @@ __global__ void ring_append_kernel(__nv_bfloat16* k_cache, __nv_bfloat16* v_cach
   const int64_t bh = row_id / T;
   const int b = static_cast<int>(bh / Hkv);
   pdl_wait();
+  // the row travels with the count: one round trip before the stores
+  const uint4 kv = *(reinterpret_cast<const uint4*>(k_new + row_id * D) + ch);
+  const uint4 vv = *(reinterpret_cast<const uint4*>(v_new + row_id * D) + ch);
   const int64_t n0 = n_before[b];
   if (n0 < 0) return;                                  // a negative count addresses nothing: the sequence is skipped
   const int64_t j = n0 + t, last = n0 + T - 1;
   if (j >= sink && j + window <= last) return;       // overwritten later in this call
   const int64_t slot = j < sink ? j : sink + (j - sink) % window;
   const int64_t C = static_cast<int64_t>(sink) + window;
-  const uint4* ks = reinterpret_cast<const uint4*>(k_new + row_id * D) + ch;
-  const uint4* vs = reinterpret_cast<const uint4*>(v_new + row_id * D) + ch;
   uint4* kd = reinterpret_cast<uint4*>(k_cache + (bh * C + slot) * D) + ch;
   uint4* vd = reinterpret_cast<uint4*>(v_cache + (bh * C + slot) * D) + ch;
-  *kd = *ks;
-  *vd = *vs;
+  *kd = kv;
+  *vd = vv;
 }
 
 static lg_status check_decode(const lg_decode_params* p) {
