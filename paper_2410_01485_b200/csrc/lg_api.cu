@@ -118,8 +118,10 @@ lg_status resolve(const lg_attn_params* p, Resolved* r, bool want_bwd, int kv_to
   r->nnz = nnz;
   r->kv_total = kv_total > 0 ? kv_total : p->B * p->Hkv;
   if (nnz > 0x3fffffff || pt.nB > (1 << 20)) return LG_ERR_UNSUPPORTED;
-  // (documents in several sequences: the pass runs once per sequence)
-  r->split = want_bwd ? kv_split(pt, r->n_ktiles, r->G, nnz, per_sequence(*r) ? r->kv_total / r->B : r->kv_total) : KvSplit{};
+  // (documents in several sequences: the passes run once per sequence)
+  const int kv_alone = per_sequence(*r) ? r->kv_total / r->B : r->kv_total;
+  r->fsplit = fwd_split_of(*r, static_cast<int64_t>(kv_alone) * r->G);
+  r->split = want_bwd ? kv_split(pt, r->n_ktiles, r->G, nnz, kv_alone) : KvSplit{};
   return LG_OK;
 }
 
@@ -195,6 +197,16 @@ WsLayout ws_layout(const Resolved& r, bool want_bwd) {
   w.sq_cnt = take(r.n_stiles * 4);
   w.sq_ent = take(nnz * 4);
   w.sq_order = take(r.n_stiles * 4);
+  size_t fwd_end = 0;
+  if (r.fsplit.len > 0) {
+    // The pieces' sums lie behind all lists, the backward's too (at most so long), whatever the head counts: one workspace
+    // serves both directions.  They are scratch of the forward, what a backward keeps there is scratch of its own.
+    const size_t lists = align_up(nnz * kDqEntInts * 4, 256) + align_up(nnz * 4, 256) + 8 * align_up(static_cast<size_t>(r.n_qtiles) * 4, 256);
+    const size_t pieces = static_cast<size_t>(r.B) * r.Hq * r.fsplit.n_cut * r.fsplit.places;
+    w.fwd_ml = off + lists;
+    w.fwd_part = w.fwd_ml + pieces * 256 * 8;
+    fwd_end = w.fwd_part + pieces * 256 * r.D * 4;
+  }
   if (want_bwd) {
     const bool keep = bwd_variant(r) == kBwdKeepDs;
     w.qt_off = take(static_cast<size_t>(r.n_qtiles) * 4);
@@ -216,7 +228,7 @@ WsLayout ws_layout(const Resolved& r, bool want_bwd) {
       w.kv_ticket = take(heads * split.n_ranks * 4);
     }
   }
-  w.total = off;
+  w.total = off > fwd_end ? off : fwd_end;
   return w;
 }
 
@@ -376,6 +388,7 @@ static lg_status plan_chunk(const lg_decode_params* p, int32_t T, int64_t n_befo
   // window, which contains it.
   c->r.win_block = p->block_tokens;
   c->r.win_phase = p->block_tokens > 0 ? static_cast<int>((n_before - kept) % p->block_tokens) : 0;
+  c->r.fsplit = fwd_split_of(c->r, static_cast<int64_t>(p->B) * p->Hq);
   c->w = ws_layout(c->r, false);
   c->lin_bytes = align_up(static_cast<size_t>(p->B) * p->Hkv * ap.L * p->D * sizeof(__nv_bfloat16), 256);
   c->o_k = align_up(c->w.total, 256);
@@ -482,9 +495,9 @@ lg_status lg_sparse_attn_prepare(const lg_attn_params* p, void* workspace, size_
 
 namespace lg {
 lg_status attn_fwd_entry(const lg_attn_params* p, const void* q, const void* k, const void* v, void* o, float* lse,
-                         void* workspace, size_t workspace_bytes, void* stream, unsigned int* status_word) {
+                         void* workspace, size_t workspace_bytes, void* stream, unsigned int* status_word, int kv_total) {
   Resolved r;
-  lg_status s = resolve(p, &r);
+  lg_status s = resolve(p, &r, false, kv_total);
   if (s != LG_OK) return s;
   r.error_word = status_word;
   if (!q || !k || !v || !o || !lse || !workspace) return LG_ERR_INVALID_ARG;

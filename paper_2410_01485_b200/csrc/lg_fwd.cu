@@ -4,7 +4,7 @@
 
 namespace lg {
 
-template <int D, int BS, int NB>
+template <int D, int BS, int NB, bool kSplit>
 static lg_status launch_fwd_t(const Resolved& r, const WsLayout& w, const void* q, const void* k, const void* v,
                               void* o, float* lse, uint8_t* ws, cudaStream_t stream) {
   CUtensorMap tq, tk, tv;
@@ -32,11 +32,16 @@ static lg_status launch_fwd_t(const Resolved& r, const WsLayout& w, const void* 
   a.doc_start = r.doc_start;
   a.scale_log2 = r.scale * 1.4426950408889634f;
   a.head_group = head_group(r, r.B * r.Hq);
-  auto kern = fwd_kernel<D, BS, NB>;
+  a.split = r.fsplit;
+  a.part = reinterpret_cast<float4*>(ws + w.fwd_part);
+  a.part_ml = reinterpret_cast<float2*>(ws + w.fwd_ml);
+  auto kern = fwd_kernel<D, BS, NB, kSplit>;
   constexpr int smem = FwdSmem<D>::kTotal;
   static std::atomic<bool> allowed[kMaxDevices];
-  dim3 grid(r.B * r.Hq, r.n_stiles);
-  return launch_big_smem(launch_attn_overlapped(r), allowed, kern, grid, kFwdThreads, smem, stream, tq, tk, tv, a) == cudaSuccess ? LG_OK : LG_ERR_CUDA;
+  dim3 grid(r.B * r.Hq, r.n_stiles + (kSplit ? r.fsplit.n_cut * (r.fsplit.places - 1) : 0));
+  if (launch_big_smem(launch_attn_overlapped(r), allowed, kern, grid, kFwdThreads, smem, stream, tq, tk, tv, a) != cudaSuccess) return LG_ERR_CUDA;
+  if (kSplit && launch_kernel(true, fwd_add_kernel<D, BS>, dim3(r.B * r.Hq, r.fsplit.n_cut, 256 / 32), kFwdAddThreads, 0, stream, a) != cudaSuccess) return LG_ERR_CUDA;
+  return LG_OK;
 }
 
 lg_status launch_fwd(const Resolved& r, const WsLayout& w, const void* q, const void* k, const void* v, void* o,
@@ -44,7 +49,14 @@ lg_status launch_fwd(const Resolved& r, const WsLayout& w, const void* q, const 
   if (r.n_qtiles > 65535) return LG_ERR_UNSUPPORTED;
   const bool pairs = fwd_two_ctas(r);
 #define LG_FWD_CASE(DD, BB, NN) \
-  if (r.D == DD && r.block == BB && pairs == (NN == 1)) return launch_fwd_t<DD, BB, NN>(r, w, q, k, v, o, lse, ws, stream);
+  if (r.D == DD && r.block == BB && pairs == (NN == 1)) return launch_fwd_t<DD, BB, NN, false>(r, w, q, k, v, o, lse, ws, stream);
+#define LG_FWD_CUT_CASE(DD, BB) \
+  if (r.fsplit.len > 0 && r.D == DD && r.block == BB) return launch_fwd_t<DD, BB, 2, true>(r, w, q, k, v, o, lse, ws, stream);
+  LG_FWD_CUT_CASE(128, 128)
+  LG_FWD_CUT_CASE(128, 64)
+  LG_FWD_CUT_CASE(64, 128)
+  LG_FWD_CUT_CASE(64, 64)
+#undef LG_FWD_CUT_CASE
   LG_FWD_CASE(128, 128, 2)
   LG_FWD_CASE(128, 64, 2)
   LG_FWD_CASE(64, 128, 1)

@@ -29,6 +29,7 @@
 #pragma once
 #include <cuda.h>
 #include "lg_common.cuh"
+#include "lg_pattern.h"
 
 namespace lg {
 
@@ -55,6 +56,9 @@ struct FwdArgs {
   const int32_t* doc_start;  // [B, L] first position of each query's document, or null
   float scale_log2;          // scale * log2(e)
   int head_group;            // heads whose CTAs run side by side (cta_coords); >= gridDim.x: all of them
+  FwdSplit split;            // tiles cut along their keys
+  float4* part;              // pieces' sums as they stand, [cut tile, head][place][D / 4][256 rows]
+  float2* part_ml;           // (reference, sum of probabilities) of their rows, [cut tile, head][place][256 rows]
 };
 
 constexpr int kFwdTmaWarp = 8, kFwdMmaWarp0 = 9;
@@ -73,7 +77,74 @@ struct FwdSmem {
   static constexpr int kTotal = oBar + 256;
 };
 
-template <int D, int BS, int NB /* score buffers per slot */>
+// Pieces of a tile that walks n_steps steps and is one of the ranks that are cut.
+__device__ __forceinline__ int fwd_pieces(const FwdSplit& k, int n_steps) { return n_steps > k.len ? min((n_steps + k.len - 1) / k.len, k.places) : 1; }
+
+// Adds the pieces of the cut tiles, in their order, and writes O and LSE.  grid = (heads, cut ranks, 8): 32 rows of a tile,
+// their sums read 512 contiguous bytes at a time from the L2, all pieces' on their way together, the rows written whole through
+// shared memory.  (Added by the CTA that delivers a tile's last piece, behind a ticket, a tile's 0.4-0.8 MB took one SM 15 us.)
+constexpr int kFwdAddThreads = 256;
+template <int D, int BS>
+__global__ void __launch_bounds__(kFwdAddThreads) fwd_add_kernel(const FwdArgs a) {
+  pdl_trigger();
+  pdl_wait();
+  if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 1u)) return;
+  if (__syncthreads_or(*reinterpret_cast<volatile unsigned int*>(a.error_word) != 0)) return;   // a piece was given up
+  const int tile = checked(a.order[blockIdx.y], 0, a.n_tiles - 1, a.error_word, 103);
+  const int n_ent = checked(a.tile_cnt[tile], 0, a.n_list, a.error_word, 104);
+  const int n_segs = fwd_pieces(a.split, (BS == 128) ? n_ent : (n_ent + 1) / 2);
+  if (n_segs == 1) return;                                        // written by its CTA
+  const int64_t unit = static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x;
+  const int b = blockIdx.x / a.Hq, h = blockIdx.x % a.Hq, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int r0 = blockIdx.z * 32, row = a.row_origin + tile * 256 + r0 + lane;   // a lane per row
+  const float2* ml = a.part_ml + unit * a.split.places * 256 + r0 + lane;
+  float w[kFwdMaxPieces], m = -INFINITY, l = 0.f;
+  float2 pair[kFwdMaxPieces];
+#pragma unroll
+  for (int i = 0; i < kFwdMaxPieces; ++i) {
+    pair[i] = i < n_segs ? __ldcg(ml + i * 256) : make_float2(-INFINITY, 0.f);
+    m = fmaxf(m, pair[i].x);
+  }
+  const float mu = m == -INFINITY ? 0.f : m;
+#pragma unroll
+  for (int i = 0; i < kFwdMaxPieces; ++i) {
+    w[i] = fast_exp2(pair[i].x - mu);                             // (a piece no key of which the row sees: 0)
+    if (i < n_segs) l += w[i] * pair[i].y;
+  }
+  const float inv = l > 0.f ? 1.f / l : l;                        // 0 where the row sees nothing, NaN stays NaN
+  __shared__ __align__(16) uint8_t stage[32 * (D * 2 + 16)];      // rows, 16 bytes apart from a multiple of the banks
+  const float4* part = a.part + unit * a.split.places * (D / 4 * 256) + r0 + lane;
+  constexpr int kCols = D / 4 / (kFwdAddThreads / 32);            // groups of four columns of a warp
+  float4 v[kCols][kFwdMaxPieces];
+#pragma unroll
+  for (int c = 0; c < kCols; ++c)
+#pragma unroll
+    for (int i = 0; i < kFwdMaxPieces; ++i)
+      if (i < n_segs) v[c][i] = __ldcg(part + (static_cast<int64_t>(i) * (D / 4) + warp * kCols + c) * 256);
+#pragma unroll
+  for (int c = 0; c < kCols; ++c) {
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < kFwdMaxPieces; ++i)
+      if (i < n_segs && w[i] != 0.f) {                            // (otherwise its sums may never have been written)
+        acc.x += w[i] * v[c][i].x; acc.y += w[i] * v[c][i].y; acc.z += w[i] * v[c][i].z; acc.w += w[i] * v[c][i].w;
+      }
+    *reinterpret_cast<uint2*>(stage + lane * (D * 2 + 16) + (warp * kCols + c) * 8) =
+        make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
+  }
+  if (warp == 0 && row < a.L && row >= a.q_start)
+    a.lse[(static_cast<int64_t>(b) * a.Hq + h) * a.Lq + row - a.q_start] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+  __syncthreads();
+  constexpr int kChunks = D / 8;                                  // 16-byte chunks of a row
+  for (int u = threadIdx.x; u < 32 * kChunks; u += kFwdAddThreads) {
+    const int r = u / kChunks, c = u % kChunks, q = row - lane + r;
+    if (q < a.L && q >= a.q_start)
+      *reinterpret_cast<uint4*>(a.o + b * a.o_strides[0] + h * a.o_strides[1] + static_cast<int64_t>(q - a.q_start) * a.o_strides[2] + c * 8) =
+          *reinterpret_cast<const uint4*>(stage + r * (D * 2 + 16) + c * 16);
+  }
+}
+
+template <int D, int BS, int NB /* score buffers per slot */, bool kSplit>
 __global__ void __launch_bounds__(kFwdThreads, fwd_ctas_per_sm(NB))
 fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
            const __grid_constant__ CUtensorMap tm_v, const FwdArgs a) {
@@ -111,14 +182,34 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   unsigned int abort_word = 0;
   if (tid == 0) abort_word = *reinterpret_cast<volatile unsigned int*>(a.error_word);
   int cta_x, cta_y;   // (batch, query head) and launch rank of this CTA's super-tile
-  cta_coords(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, cta_x, cta_y);
+  int seg = 0;        // which piece of the tile
+  bool cut = false;   // one of the ranks that are cut
+  if constexpr (kSplit) {
+    // the pieces of the ranks that are cut in turn, the tiles side by side
+    cta_x = static_cast<int>(blockIdx.x);
+    const int y = static_cast<int>(blockIdx.y), n_cut = a.split.n_cut;
+    cut = y < n_cut * a.split.places;
+    seg = cut ? y / n_cut : 0;
+    cta_y = cut ? y % n_cut : y - n_cut * (a.split.places - 1);
+  } else {
+    cta_coords(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, cta_x, cta_y);
+  }
   const int tile = checked(a.order[cta_y], 0, a.n_tiles - 1, a.error_word, 100);
   const int b = cta_x / a.Hq, h = cta_x % a.Hq, hk = h / a.G;
   const int ent_off = checked(a.tile_off[tile], 0, a.n_list, a.error_word, 101);
-  const int n_ent = checked(a.tile_cnt[tile], 0, a.n_list - ent_off, a.error_word, 102);
+  int n_ent = checked(a.tile_cnt[tile], 0, a.n_list - ent_off, a.error_word, 102);
   const int32_t* ent = a.tile_ent + ent_off;
   const int row0 = a.row_origin + tile * 256;
-  const int n_steps = (BS == 128) ? n_ent : (n_ent + 1) / 2;
+  int n_steps = (BS == 128) ? n_ent : (n_ent + 1) / 2;
+  const int n_segs = kSplit && cut ? fwd_pieces(a.split, n_steps) : 1;
+  if (kSplit && seg >= n_segs) return;                     // an empty place (uniform over the CTA)
+  if (kSplit && n_segs > 1) {
+    const int first = n_steps * seg / n_segs, end = n_steps * (seg + 1) / n_segs;
+    ent += (128 / BS) * first;
+    n_ent = min(n_ent - (128 / BS) * first, (128 / BS) * (end - first));
+    n_steps = end - first;
+  }
+  const int64_t unit = kSplit ? static_cast<int64_t>(cta_y) * gridDim.x + cta_x : 0;   // of a cut tile
 
   // entries of the two halves of step j (0: nobody's member, also past the end)
   auto load_ent = [&](int j, int& e0, int& e1) {
@@ -416,6 +507,29 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     }
     // ---- epilogue: O / l -> bf16, LSE ------------------------------------------------------
     if (ok) ok = wait_o(14);
+    if (kSplit && n_segs > 1) {
+      // a piece of a cut tile: the sums as they stand, 512 contiguous bytes per store instruction of a warp
+      if (ok) {
+        const int64_t at = unit * a.split.places + seg;
+        const int row = s * 128 + r;
+        if (p0 + p1 > 0) {
+          tc_fence_after();
+          float4* part = a.part + at * (D / 4 * 256) + row;
+#pragma unroll
+          for (int c = 0; c < D; c += 32) {
+            uint32_t reg[32];
+            tmem_ld32(my_o + c, reg);
+            tmem_ld_wait();
+#pragma unroll
+            for (int x = 0; x < 32; x += 4)
+              part[((c + x) / 4) * 256] = make_float4(__uint_as_float(reg[x]), __uint_as_float(reg[x + 1]),
+                                                      __uint_as_float(reg[x + 2]), __uint_as_float(reg[x + 3]));
+          }
+        }
+        a.part_ml[at * 256 + row] = make_float2(l_run == 0.f ? -INFINITY : m_ref, l_run);
+      }
+      ok = false;   // (the rows are not mine to write)
+    }
     // warp-uniform condition (the tensor-memory loads below need the whole warp): some row of the warp
     // is a real query; rows past L or before q_start load with the others and store nothing
     if (ok && p0 + p1 > 0 && qi - lane < a.L && qi - lane + 32 > a.q_start) {

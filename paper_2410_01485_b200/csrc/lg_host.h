@@ -87,6 +87,7 @@ struct Resolved {          // validated, defaulted copy of lg_attn_params
   int64_t nnz;
   int kv_total;              // kv heads (times batch) of the whole problem: B * Hkv, more when the call works a group of its heads
   KvSplit split;             // how the dK/dV pass cuts its kv tiles (calls with a backward; see kv_split)
+  FwdSplit fsplit;           // which super-tiles the forward cuts (see fwd_split)
 };
 
 // want_bwd: the call runs, prepares or sizes a backward; kv_total: kv heads of the whole problem when `p` is a group of
@@ -97,6 +98,7 @@ lg_status resolve(const lg_attn_params* p, Resolved* r, bool want_bwd = false, i
 struct WsLayout {
   // per schedule: start of each tile's entries, their number, the entries, launch rank -> tile
   size_t sq_off, sq_cnt, sq_ent, sq_order;       // super-tiles (forward)
+  size_t fwd_ml, fwd_part;                       // forward with cut tiles: the pieces' sums
   size_t qt_off, qt_cnt, qt_ent, qt_order;       // query tiles (dQ pass: over kv blocks, or over the kept dS tiles)
   size_t kt_off, kt_cnt, kt_ent, kt_order;       // kv tiles (dK/dV pass)
   size_t kt_cols;                                // pattern columns of each kv tile
@@ -160,6 +162,16 @@ inline bool fwd_two_ctas(const Resolved& r) {
   return 4 * ctas > quarter_rounds * static_cast<int64_t>(kSms);
 }
 
+// Which tiles the forward of `r` cuts when the whole problem has `heads` query heads (times batch).  (Two CTAs on an SM: a
+// grid of many rounds.  Documents: how long the tiles are is not known here, and pieces planned for tiles that are shorter
+// cost more than they give: 4 heads x 8000 tokens in documents of 3000, full causal, 52 -> 60 us.)
+inline FwdSplit fwd_split_of(const Resolved& r, int64_t heads) {
+  Resolved whole = r;
+  whole.B = 1;
+  whole.Hq = static_cast<int>(heads);
+  return r.doc_start || fwd_two_ctas(whole) ? FwdSplit{} : fwd_split(r.pat, r.D, r.st_row0, r.n_stiles, heads);
+}
+
 lg_status check_arch();
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
@@ -172,11 +184,12 @@ lg_status launch_bwd(const Resolved& r, const WsLayout& w, const void* q, const 
 // The forward / backward entry points with the status word of the call redirected (null: the start
 // of `workspace`): a step that runs several calls on slices of one workspace reports through one word.
 lg_status attn_fwd_entry(const lg_attn_params* p, const void* q, const void* k, const void* v, void* o, float* lse,
-                         void* workspace, size_t workspace_bytes, void* stream, unsigned int* status_word);
+                         void* workspace, size_t workspace_bytes, void* stream, unsigned int* status_word,
+                         int kv_total = 0 /* kv heads of the whole problem when this is a group of them */);
 lg_status attn_bwd_entry(const lg_attn_params* p, const void* q, const void* k, const void* v, const void* o,
                          const float* lse, const void* d_o, void* dq, void* dk, void* dv, void* workspace,
                          size_t workspace_bytes, void* stream, cudaEvent_t* marks, unsigned int* status_word,
-                         int kv_total = 0 /* kv heads of the whole problem when this is a group of them */);
+                         int kv_total = 0 /* the same */);
 size_t attn_workspace_bytes(const lg_attn_params* p, int want_bwd, int kv_total);
 
 }  // namespace lg

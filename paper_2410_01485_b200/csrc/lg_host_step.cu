@@ -115,7 +115,7 @@ lg_status lg_sparse_attn_fwd_bwd_host(const lg_attn_params* p, const void* q_hos
       // every group reports through the first word of the caller's workspace (group 0's own header):
       // a failure of any group shows in lg_last_status(dev->workspace), and later groups then do nothing
       unsigned int* status = grp == 0 ? nullptr : reinterpret_cast<unsigned int*>(ws);
-      result = attn_fwd_entry(&g.pg, qd, kd, vd, od, lsed, wsg, g.ws_per, s_cmp, status);
+      result = attn_fwd_entry(&g.pg, qd, kd, vd, od, lsed, wsg, g.ws_per, s_cmp, status, g.kv_total);
       if (result == LG_OK)
         result = attn_bwd_entry(&g.pg, qd, kd, vd, od, lsed, dod, off(dev->dq, q0, head_bytes),
                                 off(dev->dk, kv0, head_bytes), off(dev->dv, kv0, head_bytes), wsg, g.ws_per, s_cmp,

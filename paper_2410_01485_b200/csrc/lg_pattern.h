@@ -124,6 +124,69 @@ __host__ __device__ __forceinline__ int kv_start(const PatternDev& p, int R, int
   return static_cast<int>(m * p.nB - p.stride * (m * (m - 1) / 2) + short_cols_sum(p, k - m));
 }
 
+// Steps (128 keys) that the forward walks for the super-tile of n pattern rows from r0 on: the union of the rows' lists.
+__host__ __device__ __forceinline__ int fwd_tile_steps(const PatternDev& p, int r0, int n) {
+  const int end = r0 + n < p.nB ? r0 + n : p.nB;               // one past the youngest row's diagonal
+  int blocks = end;
+  if (p.mode != 0) {
+    const int w = p.mode == 1 ? p.nw : p.nl;
+    const int lo = r0 - w + 1 > 0 ? r0 - w + 1 : 0;            // oldest block of the oldest row's run
+    blocks = end - lo + (p.mode == 1 ? (p.ns < lo ? p.ns : lo) : (lo + p.stride - 1) / p.stride);
+  }
+  return (blocks * p.block + 127) / 128;
+}
+
+// Super-tiles of the forward that are cut along their keys, a CTA per piece: the tiles of the first n_cut launch ranks (the
+// longest) into ceil(steps / len) nearly equal pieces (at most `places`); a kernel of its own adds the pieces of a tile in their order.
+constexpr int kFwdMaxCutTiles = 4 * kSms, kFwdMaxPieces = 8, kFwdMaxPlaces = 1024;
+struct FwdSplit {
+  int len;                        // 0: no tile is cut
+  int n_cut, places;
+};
+
+// Cut the longest super-tiles?  In units of steps (1.7 us): a CTA costs about 3 besides its own (launch, first loads, epilogue), the
+// second kernel about 3, and a piece's sums (128 KB at D = 128, written and read back) a 32nd.  An SM's share of the pass is
+// (all + 3 per CTA) / SMs.  Where the longest tile alone takes longer (few heads, long rows) the number of pieces is the one with
+// the smallest estimate: one round of CTAs ends with its longest, several with an SM's share and half a piece that
+// sticks out.  Tiles are cut where that is less than 7 / 8 of the longest tile.  Measured, forward: 4 heads x 3318
+// tokens, full causal, D = 128 / 64: 58 -> 36 / 56 -> 31 us; 2 x 6000: 93 -> 42 us; 4 x 5000, window 4096: 74 -> 54 us; 8 x 2000: 41 -> 34 us.
+// heads: query heads times batch of the whole problem, so that a step worked in groups of heads gives the same bits.
+inline FwdSplit fwd_split(const PatternDev& p, int D, int st_row0, int n_tiles, int64_t heads) {
+  FwdSplit k{};
+  constexpr int kCta = 3, kCut = 3, kMinLen = 3, kScale = 32;   // (estimates in 32nds)
+  const int rows = 256 / p.block;
+  if (heads * n_tiles > kFwdMaxCutTiles) return k;             // (an SM's share then holds several tiles)
+  int64_t all = 0;
+  int longest = 0;
+  for (int t = 0; t < n_tiles; ++t) {
+    const int n = fwd_tile_steps(p, st_row0 + rows * t, rows);
+    all += n;
+    if (n > longest) longest = n;
+  }
+  if (longest < 8 || (all + kCta * n_tiles) * heads >= static_cast<int64_t>(longest + kCta) * kSms) return k;
+  int64_t best = static_cast<int64_t>(longest + kCta) * kScale * 7 / 8;
+  for (int pieces = 2; pieces <= kFwdMaxPieces; ++pieces) {
+    const int len = (longest + pieces - 1) / pieces;
+    if (len < kMinLen) break;
+    int64_t ctas = 0, n_cut = 0, cut = 0;
+    for (int t = 0; t < n_tiles; ++t) {
+      const int n = fwd_tile_steps(p, st_row0 + rows * t, rows), segs = (n + len - 1) / len;
+      ctas += segs;
+      if (segs > 1) { ++n_cut; cut += segs; }
+    }
+    if (heads * n_cut * pieces > kFwdMaxPlaces) continue;
+    int64_t then = ctas * heads <= kSms ? static_cast<int64_t>(len + kCta) * kScale
+                                        : (all + kCta * ctas) * heads * kScale / kSms + (len + kCta) * kScale / 2;
+    then += kCut * kScale + cut * heads * D / 128 * kScale / 32;
+    if (then >= best) continue;
+    best = then;
+    k.len = len;
+    k.n_cut = static_cast<int>(n_cut);
+    k.places = pieces;
+  }
+  return k;
+}
+
 // Query blocks that see a kv tile, i.e. the union of its columns' runs.
 __host__ __device__ __forceinline__ int kv_tile_len(const PatternDev& p, int R, int t) {
   const int a = kv_col(p, R, R * t), na = col_len(p, a);

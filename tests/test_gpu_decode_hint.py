@@ -37,7 +37,7 @@ def test_counts_of_the_kernel_before(lg, B, Hq, Hkv, D, sink, W, bt):
     def steps(wait):
         out = []
         for t in range(20):
-            n.copy_(counts[t])                     # a kernel on the same stream, just ahead
+            torch.add(counts[t], 0, out=n)         # a kernel on the same stream, just ahead
             out.append(lg.lg_sparse_decode(p, q, kc, vc, n, workspace=ws))
             out.append(lg.lg_sparse_decode(p, q, kc, vc, n, workspace=ws))
             if wait:
