@@ -196,12 +196,12 @@ WsLayout ws_layout(const Resolved& r, bool want_bwd) {
   w.sq_off = take(r.n_stiles * 4);
   w.sq_cnt = take(r.n_stiles * 4);
   w.sq_ent = take(nnz * 4);
-  w.sq_order = take(r.n_stiles * 4);
+  w.sq_order = take(r.n_stiles * sizeof(TileRec));
   size_t fwd_end = 0;
   if (r.fsplit.len > 0) {
     // The pieces' sums lie behind all lists, the backward's too (at most so long), whatever the head counts: one workspace
     // serves both directions.  They are scratch of the forward, what a backward keeps there is scratch of its own.
-    const size_t lists = align_up(nnz * kDqEntInts * 4, 256) + align_up(nnz * 4, 256) + 8 * align_up(static_cast<size_t>(r.n_qtiles) * 4, 256);
+    const size_t lists = align_up(nnz * kDqEntInts * 4, 256) + align_up(nnz * 4, 256) + 14 * align_up(static_cast<size_t>(r.n_qtiles) * 4, 256);
     const size_t pieces = static_cast<size_t>(r.B) * r.Hq * r.fsplit.n_cut * r.fsplit.places;
     w.fwd_ml = off + lists;
     w.fwd_part = w.fwd_ml + pieces * 256 * 8;
@@ -212,11 +212,11 @@ WsLayout ws_layout(const Resolved& r, bool want_bwd) {
     w.qt_off = take(static_cast<size_t>(r.n_qtiles) * 4);
     w.qt_cnt = take(static_cast<size_t>(r.n_qtiles) * 4);
     w.qt_ent = take(nnz * (keep ? kDqEntInts : 1) * 4);
-    w.qt_order = take(static_cast<size_t>(r.n_qtiles) * 4);
+    w.qt_order = take(static_cast<size_t>(r.n_qtiles) * sizeof(TileRec));
     w.kt_off = take(static_cast<size_t>(r.n_ktiles) * 4);
     w.kt_cnt = take(static_cast<size_t>(r.n_ktiles) * 4);
     w.kt_ent = take(nnz * 4);
-    w.kt_order = take(static_cast<size_t>(r.n_ktiles) * 4);
+    w.kt_order = take(static_cast<size_t>(r.n_ktiles) * sizeof(TileRec));
     w.kt_cols = take(static_cast<size_t>(r.n_ktiles) * 2 * 4);
     if (r.doc_start) w.doc_end = take(static_cast<size_t>(r.B) * r.L * 4);
     w.delta = take(static_cast<size_t>(r.B) * r.Hq * align_up(r.L, 128) * 8);   // rows padded to whole tiles   // two planes: -LSE * log2 e and -delta per query row
@@ -262,6 +262,7 @@ lg_status prepare_workspace(const Resolved& r, const WsLayout& w, uint8_t* ws, i
                             unsigned long long fp, cudaStream_t stream, const RingCopy* copy) {
   const bool want_fwd = (what & 1) != 0, want_bwd = (what & 2) != 0;
   auto i32 = [&](size_t off) { return reinterpret_cast<int32_t*>(ws + off); };
+  auto recs = [&](size_t off) { return reinterpret_cast<TileRec*>(ws + off); };
   SchedArgs a{};
   a.p = r.pat;
   // The lists are shared by all sequences of the batch, so documents can only prune them when there
@@ -273,13 +274,13 @@ lg_status prepare_workspace(const Resolved& r, const WsLayout& w, uint8_t* ws, i
   a.L = r.L;
   if (want_fwd) {   // the forward walks super-tiles of 256 rows; the backward passes have their own schedules
     a.n_stiles = r.n_stiles; a.st_row0 = r.st_row0;
-    a.sq_off = i32(w.sq_off); a.sq_cnt = i32(w.sq_cnt); a.sq_ent = i32(w.sq_ent); a.sq_order = i32(w.sq_order);
+    a.sq_off = i32(w.sq_off); a.sq_cnt = i32(w.sq_cnt); a.sq_ent = i32(w.sq_ent); a.sq_order = recs(w.sq_order);
   }
   if (want_bwd) {
     a.n_qtiles = r.n_qtiles; a.n_ktiles = r.n_ktiles;
     a.keep_ds = bwd_variant(r) == kBwdKeepDs;
-    a.qt_off = i32(w.qt_off); a.qt_cnt = i32(w.qt_cnt); a.qt_ent = i32(w.qt_ent); a.qt_order = i32(w.qt_order);
-    a.kt_off = i32(w.kt_off); a.kt_cnt = i32(w.kt_cnt); a.kt_ent = i32(w.kt_ent); a.kt_order = i32(w.kt_order);
+    a.qt_off = i32(w.qt_off); a.qt_cnt = i32(w.qt_cnt); a.qt_ent = i32(w.qt_ent); a.qt_order = recs(w.qt_order);
+    a.kt_off = i32(w.kt_off); a.kt_cnt = i32(w.kt_cnt); a.kt_ent = i32(w.kt_ent); a.kt_order = recs(w.kt_order);
     a.kt_cols = i32(w.kt_cols);
     if (r.doc_start) {
       a.doc_start = r.doc_start;

@@ -54,11 +54,9 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
     if ((s = make_tmap(&tdo, d_o, r.B, r.Hq, r.L, D, r.os, BS)) != LG_OK) return s;
     if ((s = make_tmap(&tk, k, r.B, r.Hkv, r.L, D, r.ks, BS)) != LG_OK) return s;
     if ((s = make_tmap(&tv, v, r.B, r.Hkv, r.L, D, r.vs, BS)) != LG_OK) return s;
-    a.tile_off = reinterpret_cast<const int32_t*>(ws + w.kt_off);
     a.tile_cols = reinterpret_cast<const int32_t*>(ws + w.kt_cols);
-    a.tile_cnt = reinterpret_cast<const int32_t*>(ws + w.kt_cnt);
     a.tile_ent = reinterpret_cast<const int32_t*>(ws + w.kt_ent);
-    a.order = reinterpret_cast<const int32_t*>(ws + w.kt_order);
+    a.order = reinterpret_cast<const TileRec*>(ws + w.kt_order);
     a.out0 = static_cast<__nv_bfloat16*>(dk);
     a.out1 = static_cast<__nv_bfloat16*>(dv);
     for (int i = 0; i < 3; ++i) { a.s0[i] = r.ks[i]; a.s1[i] = r.vs[i]; }
@@ -105,11 +103,9 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
     // ---- dQ = scale * dS K from the kept tiles --------------------------------------------
     CUtensorMap tk;
     if ((s = make_tmap(&tk, k, r.B, r.Hkv, r.L, D, r.ks, BS)) != LG_OK) return s;
-    a.tile_off = reinterpret_cast<const int32_t*>(ws + w.qt_off);
     a.tile_ent = reinterpret_cast<const int32_t*>(ws + w.qt_ent);
     a.tile_cols = reinterpret_cast<const int32_t*>(ws + w.kt_cols);
-    a.tile_cnt = reinterpret_cast<const int32_t*>(ws + w.qt_cnt);
-    a.order = reinterpret_cast<const int32_t*>(ws + w.qt_order);
+    a.order = reinterpret_cast<const TileRec*>(ws + w.qt_order);
     a.out0 = static_cast<__nv_bfloat16*>(dq);
     a.out1 = nullptr;
     for (int i = 0; i < 3; ++i) { a.s0[i] = r.qs[i]; a.s1[i] = 0; }
@@ -131,11 +127,9 @@ static lg_status launch_bwd_t(const Resolved& r, const WsLayout& w, const void* 
     if ((s = make_tmap(&tdo, d_o, r.B, r.Hq, r.L, D, r.os, 128)) != LG_OK) return s;
     if ((s = make_tmap(&tk, k, r.B, r.Hkv, r.L, D, r.ks, BS)) != LG_OK) return s;
     if ((s = make_tmap(&tv, v, r.B, r.Hkv, r.L, D, r.vs, BS)) != LG_OK) return s;
-    a.tile_off = reinterpret_cast<const int32_t*>(ws + w.qt_off);
     a.tile_cols = nullptr;
-    a.tile_cnt = reinterpret_cast<const int32_t*>(ws + w.qt_cnt);
     a.tile_ent = reinterpret_cast<const int32_t*>(ws + w.qt_ent);
-    a.order = reinterpret_cast<const int32_t*>(ws + w.qt_order);
+    a.order = reinterpret_cast<const TileRec*>(ws + w.qt_order);
     a.out0 = static_cast<__nv_bfloat16*>(dq);
     a.out1 = nullptr;
     for (int i = 0; i < 3; ++i) { a.s0[i] = r.qs[i]; a.s1[i] = 0; }

@@ -34,11 +34,9 @@
 namespace lg {
 
 struct BwdArgs {
-  const int32_t* tile_off;   // where a tile's entries start
-  const int32_t* tile_cols;  // dK/dV pass: pattern column of each member of a kv tile (-1: none)
-  const int32_t* tile_cnt;
+  const TileRec* order;      // tiles by launch rank
   const int32_t* tile_ent;   // idx * 4 + member mask
-  const int32_t* order;
+  const int32_t* tile_cols;  // dQ pass that reads dS back: pattern column of each member of a kv tile (-1: none)
   const float* stat;         // two planes of [B, Hq, Lp] floats: -LSE * log2(e), then -delta; Lp = L rounded up
                              // to 128 (rows past L hold zeros, so that whole-tile copies stay inside a head)
   int64_t stat_plane;        // floats per plane
@@ -220,7 +218,6 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
     if (tid == 0) atomicCAS(a.error_word, 0u, (2u << 24) | 20u);
     return;
   }
-  if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 20u)) return;
   uint8_t* sQ = smem + SM::oFix0;
   uint8_t* sDO = smem + SM::oFix1;
   uint8_t* sK = smem + SM::oA;
@@ -231,10 +228,12 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
   if (tid == 0) abort_word = *reinterpret_cast<volatile unsigned int*>(a.error_word);
   int cta_x, cta_y;   // (batch, query head) and launch rank of this CTA's query tile
   cta_coords(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, cta_x, cta_y);
-  const int tile = checked(a.order[cta_y], 0, a.n_tiles - 1, a.error_word, 110);
+  const TileRec rec = load_rec(a.order + cta_y);
+  if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 20u)) return;
+  const int tile = checked(rec.a, 0, a.n_tiles - 1, a.error_word, 110);
   const int b = cta_x / a.Hq, h = cta_x % a.Hq, hk = h / a.G;
-  const int ent_off = checked(a.tile_off[tile], 0, a.n_list, a.error_word, 111);
-  const int n_ent = checked(a.tile_cnt[tile], 0, a.n_list - ent_off, a.error_word, 112);
+  const int ent_off = checked(rec.off, 0, a.n_list, a.error_word, 111);
+  const int n_ent = checked(rec.cnt, 0, a.n_list - ent_off, a.error_word, 112);
   const int32_t* ent = a.tile_ent + ent_off;
   const int row0 = tile * 128;
   const int n_steps = (BS == 128) ? n_ent : (n_ent + 1) / 2;
@@ -575,7 +574,6 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     if (tid == 0) atomicCAS(a.error_word, 0u, (2u << 24) | 10u);
     return;
   }
-  if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 10u)) return;
   uint8_t* sK = smem + SM::oFix0;
   uint8_t* sV = smem + SM::oFix1;
   uint8_t* sQ = smem + SM::oA;     // [3]
@@ -599,14 +597,15 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
   } else {
     cta_coords2(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.long_group, a.n_long, a.head_group, cta_x, cta_y);
   }
-  const int tile = checked(a.order[cta_y], 0, a.n_tiles - 1, a.error_word, 120);
+  const TileRec rec = load_rec(a.order + cta_y);
+  if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 10u)) return;
   const int b = cta_x / a.Hkv, hk = cta_x % a.Hkv;
-  const int ent_off = checked(a.tile_off[tile], 0, a.n_list, a.error_word, 121);
-  const int n_ent = checked(a.tile_cnt[tile], 0, a.n_list - ent_off, a.error_word, 122);
+  const int ent_off = checked(rec.off, 0, a.n_list, a.error_word, 121);
+  const int n_ent = checked(rec.cnt, 0, a.n_list - ent_off, a.error_word, 122);
   const int32_t* ent = a.tile_ent + ent_off;
   // key blocks of the tile's members (with 64-token blocks the two members need not be neighbours)
-  const int kb_a = checked(a.tile_cols[R * tile], 0, a.nB - 1, a.error_word, 123);
-  const int kb_b = (R == 2) ? checked(a.tile_cols[R * tile + 1], -1, a.nB - 1, a.error_word, 124) : -1;
+  const int kb_a = checked(rec.a, 0, a.nB - 1, a.error_word, 123);
+  const int kb_b = (R == 2) ? checked(rec.b, -1, a.nB - 1, a.error_word, 124) : -1;
   const int all_items = n_ent * a.G;
   const int n_segs = (kSplit && all_items > a.split.len) ? (all_items + a.split.len - 1) / a.split.len : 1;
   if (seg >= n_segs) return;                               // an empty place (uniform over the CTA)
@@ -705,11 +704,11 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         if (w >= static_cast<int64_t>(gridDim.x) * gridDim.y) return;
         int x2, y2;
         cta_coords2(w, gridDim.x, gridDim.y, a.long_group, a.n_long, a.head_group, x2, y2);
-        const int t2 = checked(a.order[y2], 0, a.n_tiles - 1, a.error_word, 126);
+        const TileRec r2 = load_rec(a.order + y2);
         const int b2 = x2 / a.Hkv, hk2 = x2 % a.Hkv;
 #pragma unroll
         for (int m = 0; m < R; ++m) {
-          const int kb2 = checked(a.tile_cols[R * t2 + m], -1, a.nB - 1, a.error_word, 127);
+          const int kb2 = checked(m == 0 ? r2.a : r2.b, -1, a.nB - 1, a.error_word, 127);
           if (kb2 < 0) continue;
 #pragma unroll
           for (int x = 0; x < D / 64; ++x) {
@@ -1161,9 +1160,10 @@ bwd_dq_from_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const BwdArgs a,
     Item it;
     const int x = static_cast<int>(w % n_heads), y = static_cast<int>(w / n_heads);
     it.b = x / a.Hq; it.h = x % a.Hq;
-    it.t = checked(a.order[y], 0, a.n_tiles - 1, a.error_word, 130);   // query tile (128 rows)
-    const int ent_off = checked(a.tile_off[it.t], 0, a.n_list, a.error_word, 131);
-    it.n_ent = checked(a.tile_cnt[it.t], 0, a.n_list - ent_off, a.error_word, 132);
+    const TileRec rec = load_rec(a.order + y);
+    it.t = checked(rec.a, 0, a.n_tiles - 1, a.error_word, 130);   // query tile (128 rows)
+    const int ent_off = checked(rec.off, 0, a.n_list, a.error_word, 131);
+    it.n_ent = checked(rec.cnt, 0, a.n_list - ent_off, a.error_word, 132);
     it.ent = a.tile_ent + kDqEntInts * static_cast<int64_t>(ent_off);   // (kv tile, dS tiles of its quarters)
     return it;
   };

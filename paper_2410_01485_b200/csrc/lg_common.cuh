@@ -17,6 +17,11 @@ struct WsHeader {
   unsigned long long fingerprint;  // which pattern the lists and schedules below were built for (0: none)
   unsigned int pad[58];
 };
+// What a CTA needs to know about its tile, in launch order: one load at the head of every CTA instead of a chain of them.
+struct __align__(16) TileRec {
+  int off, cnt;   // where the tile's entries start, and their number
+  int a, b;       // super-tiles and query tiles: the tile; kv tiles: the pattern columns of its members (b: -1 without a second)
+};
 constexpr int kDqEntInts = 5;   // ints per entry of the schedule of the dQ pass that reads dS back (dq_entries)
 constexpr unsigned long long kWsMagic = 0x4c47575348445231ull;   // "LGWSHDR1"
 static_assert(sizeof(WsHeader) == 256, "header size");
@@ -30,6 +35,13 @@ __device__ __forceinline__ bool lists_match(unsigned int* error_word, unsigned l
   if (have == fp || have == fp2) return true;
   if (threadIdx.x == 0) atomicCAS(error_word, 0u, (3u << 24) | site);
   return false;
+}
+
+// (volatile: issued where it stands, before the checks of the header that it travels with)
+__device__ __forceinline__ TileRec load_rec(const TileRec* p) {
+  TileRec r;
+  asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r.off), "=r"(r.cnt), "=r"(r.a), "=r"(r.b) : "l"(p) : "memory");
+  return r;
 }
 
 // Checked builds (-DLG_DEBUG): every value read from a schedule or list that is later used as an index, an

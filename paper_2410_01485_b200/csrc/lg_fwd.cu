@@ -13,10 +13,8 @@ static lg_status launch_fwd_t(const Resolved& r, const WsLayout& w, const void* 
   if ((s = make_tmap(&tk, k, r.B, r.Hkv, r.L, D, r.ks, BS)) != LG_OK) return s;
   if ((s = make_tmap(&tv, v, r.B, r.Hkv, r.L, D, r.vs, BS)) != LG_OK) return s;
   FwdArgs a;
-  a.tile_off = reinterpret_cast<const int32_t*>(ws + w.sq_off);
-  a.tile_cnt = reinterpret_cast<const int32_t*>(ws + w.sq_cnt);
   a.tile_ent = reinterpret_cast<const int32_t*>(ws + w.sq_ent);
-  a.order = reinterpret_cast<const int32_t*>(ws + w.sq_order);
+  a.order = reinterpret_cast<const TileRec*>(ws + w.sq_order);
   a.o = static_cast<__nv_bfloat16*>(o);
   a.lse = lse;
   a.error_word = r.error_word ? r.error_word : reinterpret_cast<unsigned int*>(ws);

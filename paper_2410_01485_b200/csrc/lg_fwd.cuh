@@ -34,10 +34,8 @@
 namespace lg {
 
 struct FwdArgs {
-  const int32_t* tile_off;   // [n_super_tiles] where a super-tile's entries start
-  const int32_t* tile_cnt;   // [n_super_tiles]
   const int32_t* tile_ent;   // kb * 16 + member mask (bit r: pattern row r of the super-tile has the block)
-  const int32_t* order;      // [n_super_tiles] launch rank -> super-tile
+  const TileRec* order;      // [n_super_tiles] by launch rank
   __nv_bfloat16* o;
   float* lse;                // [B, Hq, L]
   unsigned int* error_word;  // first word of the workspace header
@@ -90,8 +88,9 @@ __global__ void __launch_bounds__(kFwdAddThreads) fwd_add_kernel(const FwdArgs a
   pdl_wait();
   if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 1u)) return;
   if (__syncthreads_or(*reinterpret_cast<volatile unsigned int*>(a.error_word) != 0)) return;   // a piece was given up
-  const int tile = checked(a.order[blockIdx.y], 0, a.n_tiles - 1, a.error_word, 103);
-  const int n_ent = checked(a.tile_cnt[tile], 0, a.n_list, a.error_word, 104);
+  const TileRec rec = load_rec(a.order + blockIdx.y);
+  const int tile = checked(rec.a, 0, a.n_tiles - 1, a.error_word, 103);
+  const int n_ent = checked(rec.cnt, 0, a.n_list, a.error_word, 104);
   const int n_segs = fwd_pieces(a.split, (BS == 128) ? n_ent : (n_ent + 1) / 2);
   if (n_segs == 1) return;                                        // written by its CTA
   const int64_t unit = static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x;
@@ -173,12 +172,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     if (tid == 0) atomicCAS(a.error_word, 0u, (2u << 24) | 1u);
     return;
   }
-  if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 1u)) return;
-  uint8_t* sQ = smem + SM::oQ;
-  uint8_t* sK = smem + SM::oK;
-  uint8_t* sV = smem + SM::oV;
-
-  // has a wait already given up in this call?  (read now, so that it travels with the schedule loads below)
+  // has a wait already given up in this call?  (read now, so that it travels with the loads below)
   unsigned int abort_word = 0;
   if (tid == 0) abort_word = *reinterpret_cast<volatile unsigned int*>(a.error_word);
   int cta_x, cta_y;   // (batch, query head) and launch rank of this CTA's super-tile
@@ -194,10 +188,16 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   } else {
     cta_coords(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, cta_x, cta_y);
   }
-  const int tile = checked(a.order[cta_y], 0, a.n_tiles - 1, a.error_word, 100);
+  const TileRec rec = load_rec(a.order + cta_y);
+  if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 1u)) return;
+  uint8_t* sQ = smem + SM::oQ;
+  uint8_t* sK = smem + SM::oK;
+  uint8_t* sV = smem + SM::oV;
+
+  const int tile = checked(rec.a, 0, a.n_tiles - 1, a.error_word, 100);
   const int b = cta_x / a.Hq, h = cta_x % a.Hq, hk = h / a.G;
-  const int ent_off = checked(a.tile_off[tile], 0, a.n_list, a.error_word, 101);
-  int n_ent = checked(a.tile_cnt[tile], 0, a.n_list - ent_off, a.error_word, 102);
+  const int ent_off = checked(rec.off, 0, a.n_list, a.error_word, 101);
+  int n_ent = checked(rec.cnt, 0, a.n_list - ent_off, a.error_word, 102);
   const int32_t* ent = a.tile_ent + ent_off;
   const int row0 = a.row_origin + tile * 256;
   int n_steps = (BS == 128) ? n_ent : (n_ent + 1) / 2;

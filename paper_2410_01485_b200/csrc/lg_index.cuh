@@ -63,9 +63,10 @@ struct SchedArgs {
   int n_stiles, st_row0;     // super-tiles, and the pattern row the first one starts at
   int n_qtiles, n_ktiles;    // 0: no schedule of that kind
   int keep_ds;               // query tiles: the schedule over the kept dS instead of the recomputing pass's
-  int32_t *sq_off, *sq_cnt, *sq_ent, *sq_order;
-  int32_t *qt_off, *qt_cnt, *qt_ent, *qt_order;
-  int32_t *kt_off, *kt_cnt, *kt_ent, *kt_order, *kt_cols;
+  int32_t *sq_off, *sq_cnt, *sq_ent;
+  int32_t *qt_off, *qt_cnt, *qt_ent;
+  int32_t *kt_off, *kt_cnt, *kt_ent, *kt_cols;
+  TileRec *sq_order, *qt_order, *kt_order;
   const int32_t* doc_start;  // with documents and a backward: doc_end[i] is derived for n_doc tokens, L per sequence
   int32_t* doc_end;
   int64_t n_doc;
@@ -275,7 +276,7 @@ __device__ __forceinline__ int rank_of(const int32_t* cnt, int n, int t) {
   return __reduce_add_sync(0xffffffffu, rank);
 }
 
-// Launch order: tiles with more work first (order[rank] = tile).  The last launch of a build: the header gets the
+// Launch order: tiles with more work first (order[rank] = what a CTA needs to know of the tile).  The last launch of a build: the header gets the
 // fingerprint the lists are known by (0: none).
 __global__ void __launch_bounds__(kSchedThreads) sched_order_kernel(const SchedArgs a, unsigned long long fp) {
   pdl_trigger();
@@ -283,13 +284,18 @@ __global__ void __launch_bounds__(kSchedThreads) sched_order_kernel(const SchedA
   if (blockIdx.x == 0 && threadIdx.x == 0 && fp != 0) a.header->fingerprint = fp;
   int w = blockIdx.x * (kSchedThreads / 32) + (threadIdx.x >> 5);
   const int32_t* cnt[3] = {a.sq_cnt, a.qt_cnt, a.kt_cnt};
-  int32_t* order[3] = {a.sq_order, a.qt_order, a.kt_order};
+  const int32_t* off[3] = {a.sq_off, a.qt_off, a.kt_off};
+  TileRec* order[3] = {a.sq_order, a.qt_order, a.kt_order};
   const int n[3] = {a.n_stiles, a.n_qtiles, a.n_ktiles};
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     if (w < n[i]) {
       const int rank = rank_of(cnt[i], n[i], w);
-      if ((threadIdx.x & 31) == 0) order[i][rank] = w;
+      if ((threadIdx.x & 31) == 0) {
+        TileRec r{off[i][w], cnt[i][w], w, -1};
+        if (i == 2) { r.a = a.kt_cols[a.R * w]; r.b = a.R == 2 ? a.kt_cols[2 * w + 1] : -1; }
+        order[i][rank] = r;
+      }
       return;
     }
     w -= n[i];
