@@ -31,6 +31,8 @@
 #include "lg_common.cuh"
 #include "lg_pattern.h"
 
+#include <type_traits>
+
 namespace lg {
 
 struct BwdArgs {
@@ -943,28 +945,31 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const bool masked = __any_sync(0xffffffffu, xmin > 0 || xmax < C);
         static_assert(C == 32, "one mask word");
         const uint32_t seen = bit_range(xmin, xmax);
+        auto probabilities = [&](auto with_mask) {   // (a loop of its own for the half-steps of which a key sees all)
 #pragma unroll
-        for (int c = 0; c < C; c += 4) {
-          const float4 l4 = st_l[c >> 2];
-          float x0, x1, x2, x3;
-          f32x2_split(fma_f32x2(f32x2(__uint_as_float(sreg[c]), __uint_as_float(sreg[c + 1])), scale2,
-                                f32x2(l4.x, l4.y)), x0, x1);
-          f32x2_split(fma_f32x2(f32x2(__uint_as_float(sreg[c + 2]), __uint_as_float(sreg[c + 3])), scale2,
-                                f32x2(l4.z, l4.w)), x2, x3);
-          // (all on the exponential unit: with the two teams the element-wise warps have slack, and under
-          // the power cap the instructions of a polynomial on the FMA pipe cost more than the unit's cycles)
-          float v0 = fast_exp2(x0), v1 = fast_exp2(x1), v2 = fast_exp2(x2), v3 = fast_exp2(x3);
-          if (masked) {
-            v0 = (seen >> c) & 1 ? v0 : 0.f;
-            v1 = (seen >> (c + 1)) & 1 ? v1 : 0.f;
-            v2 = (seen >> (c + 2)) & 1 ? v2 : 0.f;
-            v3 = (seen >> (c + 3)) & 1 ? v3 : 0.f;
+          for (int c = 0; c < C; c += 4) {
+            const float4 l4 = st_l[c >> 2];
+            float x0, x1, x2, x3;
+            f32x2_split(fma_f32x2(f32x2(__uint_as_float(sreg[c]), __uint_as_float(sreg[c + 1])), scale2,
+                                  f32x2(l4.x, l4.y)), x0, x1);
+            f32x2_split(fma_f32x2(f32x2(__uint_as_float(sreg[c + 2]), __uint_as_float(sreg[c + 3])), scale2,
+                                  f32x2(l4.z, l4.w)), x2, x3);
+            // (all on the exponential unit: with the two teams the element-wise warps have slack, and under
+            // the power cap the instructions of a polynomial on the FMA pipe cost more than the unit's cycles)
+            float v0 = fast_exp2(x0), v1 = fast_exp2(x1), v2 = fast_exp2(x2), v3 = fast_exp2(x3);
+            if constexpr (decltype(with_mask)::value) {
+              v0 = (seen >> c) & 1 ? v0 : 0.f;
+              v1 = (seen >> (c + 1)) & 1 ? v1 : 0.f;
+              v2 = (seen >> (c + 2)) & 1 ? v2 : 0.f;
+              v3 = (seen >> (c + 3)) & 1 ? v3 : 0.f;
+            }
+            p[c] = v0;
+            p[c + 1] = v1;
+            p[c + 2] = v2;
+            p[c + 3] = v3;
           }
-          p[c] = v0;
-          p[c + 1] = v1;
-          p[c + 2] = v2;
-          p[c + 3] = v3;
-        }
+        };
+        if (masked) probabilities(std::true_type{}); else probabilities(std::false_type{});
         uint32_t preg[C / 2];
 #pragma unroll
         for (int c = 0; c < C; c += 2) preg[c >> 1] = pack_bf16(p[c], p[c + 1]);
