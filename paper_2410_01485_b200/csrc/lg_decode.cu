@@ -51,6 +51,11 @@ __device__ __forceinline__ void cp_async16(uint32_t smem_addr, const void* gptr,
 __device__ __forceinline__ void prefetch_l2(const void* gptr, uint32_t bytes) {   // 16-byte aligned, a multiple of 16 bytes
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(gptr), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ unsigned ticket_add(unsigned int* p) {
+  unsigned old;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
+  return old;
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() {
@@ -173,7 +178,7 @@ __device__ __forceinline__ void decode_run_segment(const DecodeArgs& a, uint8_t*
     const uint32_t sk = wsm_u32 + stage * 2 * kTileBytes, sv = sk + kTileBytes;
 
     // ---- S^T[16 tokens, 8 heads] = K Q^T ------------------------------------------------
-    float sacc[4] = {0.f, 0.f, 0.f, 0.f};
+    float sacc[4] = {0.f, 0.f, 0.f, 0.f}, sodd[4] = {0.f, 0.f, 0.f, 0.f};   // two chains of products: half the latency
     {
       const int row = ((lane >> 3) & 1) * 8 + (lane & 7);
 #pragma unroll
@@ -181,8 +186,10 @@ __device__ __forceinline__ void decode_run_segment(const DecodeArgs& a, uint8_t*
         const int cc = 2 * k + (lane >> 4);
         uint32_t a0, a1, a2, a3;
         ldsm_x4(sk + row * kRowBytes + ((cc ^ (row & 7)) * 16), a0, a1, a2, a3);
-        mma16816(sacc, a0, a1, a2, a3, qf[k][0], qf[k][1]);
+        mma16816(k & 1 ? sodd : sacc, a0, a1, a2, a3, qf[k][0], qf[k][1]);
       }
+#pragma unroll
+      for (int x = 0; x < 4; ++x) sacc[x] += sodd[x];
     }
     // sacc[0,1]: token r, heads 2c, 2c+1;  sacc[2,3]: token r + 8
     const int tok0 = t * kDecTile + r;
@@ -379,6 +386,18 @@ __device__ __forceinline__ void decode_merge_unit(const DecodeArgs& a, float* sc
   const bool sparse_slices = total < n_cta;
   auto absent = [&](int c) { return sparse_slices && total * c / n_cta == total * (c + 1) / n_cta; };
   float2* ml = reinterpret_cast<float2*>(scratch);           // [n_rec][8]: (max, sum), then x becomes the record's weight
+  // the first records' values travel together with the pairs (four values of one head a thread)
+  constexpr int kBatch = 8;
+  const int idx = tid * 4;
+  float4 v[kBatch];
+  auto load_batch = [&](int i0) {
+#pragma unroll
+    for (int x = 0; x < kBatch; ++x)
+      v[x] = (idx < kDecHeads * D && i0 + x < n_rec && !absent(first_cta + i0 + x))
+                 ? __ldcg(reinterpret_cast<const float4*>(recs + static_cast<int64_t>(i0 + x) * (kDecHeads * kRec) + idx))
+                 : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  load_batch(0);
   __syncthreads();                                           // scratch: whoever used this shared memory is done
   for (int e = tid; e < n_rec * kDecHeads; e += kDecThreads) {
     const int i = e / kDecHeads;
@@ -404,30 +423,29 @@ __device__ __forceinline__ void decode_merge_unit(const DecodeArgs& a, float* sc
     if (lane == 0) ml[n_rec * kDecHeads + head] = make_float2(m, l);
   }
   __syncthreads();
-  for (int idx = tid * 4; idx < kDecHeads * D; idx += kDecThreads * 4) {   // four values of one head
+  static_assert(kDecHeads * 128 <= kDecThreads * 4, "one piece of a head per thread");
+  if (idx < kDecHeads * D) {
     const int head = idx / D, gh = hg * kDecHeads + head;
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int i0 = 0; i0 < n_rec; i0 += 8) {
-      float4 r[8];
+    for (int i0 = 0;;) {
 #pragma unroll
-      for (int x = 0; x < 8; ++x)
-        r[x] = (i0 + x < n_rec && !absent(first_cta + i0 + x))
-                   ? __ldcg(reinterpret_cast<const float4*>(recs + static_cast<int64_t>(i0 + x) * (kDecHeads * kRec) + idx))
-                   : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-      for (int x = 0; x < 8; ++x) {
+      for (int x = 0; x < kBatch; ++x) {
         const float f = i0 + x < n_rec ? ml[(i0 + x) * kDecHeads + head].x : 0.f;
-        acc.x += f * r[x].x; acc.y += f * r[x].y; acc.z += f * r[x].z; acc.w += f * r[x].w;
+        acc.x += f * v[x].x; acc.y += f * v[x].y; acc.z += f * v[x].z; acc.w += f * v[x].w;
       }
+      i0 += kBatch;
+      if (i0 >= n_rec) break;
+      load_batch(i0);
     }
-    if (gh >= a.G) continue;
-    const float m = ml[n_rec * kDecHeads + head].x, l = ml[n_rec * kDecHeads + head].y;
-    const int64_t qh = static_cast<int64_t>(b) * a.Hq + kvh * a.G + gh;
-    uint2 out;
-    out.x = l > 0.f ? pack_bf16(acc.x / l, acc.y / l) : 0u;
-    out.y = l > 0.f ? pack_bf16(acc.z / l, acc.w / l) : 0u;
-    *reinterpret_cast<uint2*>(a.o + qh * D + idx % D) = out;
-    if (idx % D == 0 && a.lse) a.lse[qh] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+    if (gh < a.G) {
+      const float m = ml[n_rec * kDecHeads + head].x, l = ml[n_rec * kDecHeads + head].y;
+      const int64_t qh = static_cast<int64_t>(b) * a.Hq + kvh * a.G + gh;
+      uint2 out;
+      out.x = l > 0.f ? pack_bf16(acc.x / l, acc.y / l) : 0u;
+      out.y = l > 0.f ? pack_bf16(acc.z / l, acc.w / l) : 0u;
+      *reinterpret_cast<uint2*>(a.o + qh * D + idx % D) = out;
+      if (idx % D == 0 && a.lse) a.lse[qh] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+    }
   }
 }
 
@@ -438,77 +456,94 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
   constexpr int kRec = D + 2;
   int* cum = reinterpret_cast<int*>(dsmem + kPipeBytes);
   // overlapped with the kernel before (an append, or the decode of the step before): append + decode of 16 sequences
-  // over 4224 slots, 64 / 8 heads, 53.7 -> 49.3 us a step, of one sequence 28.7 -> 13.7 us with the merge below (then the hint)
+  // over 4224 slots, 64 / 8 heads, 53.7 -> 49.3 us a step, of one sequence 28.7 -> 13.7 us with the merge below
   pdl_trigger();
   const int ups = a.Hkv * a.HG;
-  // Before the wait: a guess at my slice, from token counts that the kernel before may still be changing, and the first
-  // tiles of its warps asked into the L2, so that the HBM starts while the kernel before (an append, or the last merges of a
-  // decode) ends.  A hint only: nothing read here is used for more than addresses inside the caches, the L2 sees
-  // whatever is still written to the lines, and the counts are read again after the wait.  With one round trip less in the
-  // append and one fence a CTA instead of one a thread: append + decode of 16 sequences over 4224 slots, 64 / 8 heads,
-  // 49.2 -> 47.6 us, of one sequence 13.7 -> 12.8 us, of 4 linear caches of 9000 to 32768 tokens, 32 heads, 208.9 -> 206.4 us.
+  bool any_empty;
   int tiles;
-  bool any_empty = decode_build_cum(a, cum, tiles);
-  {
-    const int64_t total = static_cast<int64_t>(cum[a.B]) * ups;
-    const int64_t f0 = total * blockIdx.x / gridDim.x, f1 = total * (blockIdx.x + 1) / gridDim.x;
-    if (f0 < f1 && (threadIdx.x & 31) < 2) {
-      int lo = 0, hi = a.B;
-      while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (static_cast<int64_t>(cum[mid]) * ups <= f0) lo = mid; else hi = mid;
-      }
-      const int nt = cum[lo + 1] - cum[lo];
-      const int64_t rel = f0 - static_cast<int64_t>(cum[lo]) * ups;
-      const int k = static_cast<int>(rel / nt), t0 = static_cast<int>(rel - static_cast<int64_t>(k) * nt);
-      const int n = static_cast<int>(min(static_cast<int64_t>(nt - t0), f1 - f0)), w = threadIdx.x >> 5;
-      const int tb = t0 + static_cast<int>(static_cast<int64_t>(n) * w / kDecWarps);
-      const int te = min(t0 + static_cast<int>(static_cast<int64_t>(n) * (w + 1) / kDecWarps), tb + kDecHintTiles);
-      const int slot0 = tb * kDecTile, rows = min(te * kDecTile, a.C) - slot0;
-      if (rows > 0) {
-        const __nv_bfloat16* base = (threadIdx.x & 1) ? a.v_cache : a.k_cache;
-        prefetch_l2(base + ((static_cast<int64_t>(lo) * a.Hkv + k / a.HG) * a.C + slot0) * D, rows * D * 2);
-      }
-    }
-  }
-  pdl_wait();
-  // (with more sequences than threads they are simply counted again)
-  const bool changed = a.B > kDecThreads || (threadIdx.x < a.B && decode_tiles_of(a, threadIdx.x) != tiles);
-  if (__syncthreads_or(changed)) any_empty = decode_build_cum(a, cum, tiles);
-  const int64_t total = static_cast<int64_t>(cum[a.B]) * ups;
-  __shared__ int s_merge[3];
-  auto start_of = [&](int64_t c) { return total * c / gridDim.x; };
+  int64_t total, f0, f1;
+  bool narrow;                             // the slices' arithmetic fits 32 bits (64-bit divisions take 200 cycles each)
+  auto start_of = [&](int64_t c) -> int64_t {
+    return narrow ? static_cast<uint32_t>(total) * static_cast<uint32_t>(c) / gridDim.x : total * c / gridDim.x;
+  };
   auto cta_of = [&](int64_t f) {           // the CTA whose slice holds tile f
-    int64_t c = f * gridDim.x / total;
+    int64_t c = narrow ? static_cast<uint32_t>(f) * gridDim.x / static_cast<uint32_t>(total) : f * gridDim.x / total;
     while (c + 1 < gridDim.x && start_of(c + 1) <= f) ++c;
     while (c > 0 && start_of(c) > f) --c;
     return static_cast<int>(c);
   };
+  // the segment of my slice that starts at tile pos: n tiles from tile t0 on of unit (b, k), which CTAs c_lo .. c_hi share,
+  // `pieces` of them with a record
+  int b = 0, k = 0, t0 = 0, n = 0, nt = 0, c_lo = 0, c_hi = 0, pieces = 0;
+  auto segment = [&](int64_t pos) {
+    while (static_cast<int64_t>(cum[b + 1]) * ups <= pos) ++b;          // skip finished / empty sequences
+    nt = cum[b + 1] - cum[b];
+    const int64_t before = static_cast<int64_t>(cum[b]) * ups, rel = pos - before;
+    k = narrow ? static_cast<int>(static_cast<uint32_t>(rel) / static_cast<uint32_t>(nt)) : static_cast<int>(rel / nt);
+    t0 = static_cast<int>(rel - static_cast<int64_t>(k) * nt);
+    n = static_cast<int>(min(static_cast<int64_t>(nt - t0), f1 - pos));
+    const int64_t first = before + static_cast<int64_t>(k) * nt;
+    c_lo = (t0 == 0) ? static_cast<int>(blockIdx.x) : cta_of(first);
+    c_hi = (t0 + n == nt) ? static_cast<int>(blockIdx.x) : cta_of(first + nt - 1);
+    pieces = c_hi - c_lo + 1;
+    if (total < gridDim.x)
+      for (int c = c_lo; c <= c_hi; ++c) pieces -= (start_of(c) == start_of(c + 1)) ? 1 : 0;
+  };
+  auto plan = [&]() {                      // cum, my slice and its first segment
+    any_empty = decode_build_cum(a, cum, tiles);
+    total = static_cast<int64_t>(cum[a.B]) * ups;
+    narrow = total * gridDim.x <= 0xffffffffll;
+    f0 = start_of(blockIdx.x);
+    f1 = start_of(blockIdx.x + 1);
+    if (f0 >= f1) return;
+    int lo = 0, hi = a.B;                  // cum[lo] * ups <= f0 < cum[hi] * ups
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) >> 1;
+      if (static_cast<int64_t>(cum[mid]) * ups <= f0) lo = mid; else hi = mid;
+    }
+    b = lo;
+    segment(f0);
+  };
+  const int warp = threadIdx.x >> 5;
+  // Before the wait: the plan from token counts that the kernel before may still be changing, and the first
+  // tiles of my warps asked into the L2, so that the HBM starts while the kernel before (an append, or the last merges of a
+  // decode) ends.  Nothing read here is used for more than addresses inside the caches until the counts have been read again
+  // after the wait and are the same, and the L2 sees whatever is still written to the lines.  The plan's 64-bit
+  // divisions and the chain of loads were 1.5 us behind the wait, two fences (fence.sc) of 1.3 us each went with the acquiring and
+  // releasing ticket: append + decode of one sequence over 4224 slots, 64 / 8 heads,
+  // 12.7 -> 11.6 us, of 16 sequences 47.2 -> 46.2 us (13.7 and 49.2 us before the hint).
+  plan();
+  if (f0 < f1 && (threadIdx.x & 31) < 2) {
+    const int tb = t0 + static_cast<int>(static_cast<int64_t>(n) * warp / kDecWarps);
+    const int te = min(t0 + static_cast<int>(static_cast<int64_t>(n) * (warp + 1) / kDecWarps), tb + kDecHintTiles);
+    const int slot0 = tb * kDecTile, rows = min(te * kDecTile, a.C) - slot0;
+    if (rows > 0) {
+      const __nv_bfloat16* base = (threadIdx.x & 1) ? a.v_cache : a.k_cache;
+      prefetch_l2(base + ((static_cast<int64_t>(b) * a.Hkv + k / a.HG) * a.C + slot0) * D, rows * D * 2);
+    }
+  }
+  pdl_wait();
+  // (with more sequences than threads they are simply counted again)
+  int nvalid = f0 < f1 ? decode_valid_of(a, b) : 0;        // (travels with the counts)
+  const bool changed = a.B > kDecThreads || (threadIdx.x < a.B && decode_tiles_of(a, threadIdx.x) != tiles);
+  if (__syncthreads_or(changed)) {
+    plan();
+    if (f0 < f1) nvalid = decode_valid_of(a, b);
+  }
+  __shared__ int s_last;
   // units of sequences without tokens get their (empty) result here, spread over the CTAs
   for (int e = 0; any_empty && e < a.B; ++e) {
     if (cum[e + 1] != cum[e]) continue;
-    for (int k = 0; k < ups; ++k) {
-      const int64_t u = static_cast<int64_t>(e) * ups + k;
-      if (u % gridDim.x == blockIdx.x) decode_merge_unit<D>(a, reinterpret_cast<float*>(dsmem), e, k, u, 0, 0, total, gridDim.x);
+    for (int x = 0; x < ups; ++x) {
+      const int64_t u = static_cast<int64_t>(e) * ups + x;
+      if (u % gridDim.x == blockIdx.x) decode_merge_unit<D>(a, reinterpret_cast<float*>(dsmem), e, x, u, 0, 0, total, gridDim.x);
     }
   }
-  const int64_t f0 = start_of(blockIdx.x), f1 = start_of(blockIdx.x + 1);
-  if (f0 >= f1) return;
-  int lo = 0, hi = a.B;   // cum[lo] * ups <= f0 < cum[hi] * ups
-  while (hi - lo > 1) {
-    const int mid = (lo + hi) >> 1;
-    if (static_cast<int64_t>(cum[mid]) * ups <= f0) lo = mid; else hi = mid;
-  }
-  int b = lo;
-  const int warp = threadIdx.x >> 5;
-  int64_t pos = f0;
-  while (pos < f1) {
-    while (static_cast<int64_t>(cum[b + 1]) * ups <= pos) ++b;          // skip finished / empty sequences
-    const int nt = cum[b + 1] - cum[b];
-    const int64_t rel = pos - static_cast<int64_t>(cum[b]) * ups;
-    const int k = static_cast<int>(rel / nt), t0 = static_cast<int>(rel - static_cast<int64_t>(k) * nt);
-    const int n = static_cast<int>(min(static_cast<int64_t>(nt - t0), f1 - pos));
-    const int nvalid = decode_valid_of(a, b);
+  for (int64_t pos = f0; pos < f1;) {
+    if (pos != f0) {
+      segment(pos);
+      nvalid = decode_valid_of(a, b);
+    }
     const int tb = t0 + static_cast<int>(static_cast<int64_t>(n) * warp / kDecWarps);
     const int te = t0 + static_cast<int>(static_cast<int64_t>(n) * (warp + 1) / kDecWarps);
     const int64_t u = static_cast<int64_t>(b) * ups + k;
@@ -519,27 +554,17 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
     pos += n;
     if (direct) continue;
     // The CTA that delivers the last record of a unit merges it (records are read in index
-    // order, so the result does not depend on which CTA that is) and re-arms the counter.
+    // order, so the result does not depend on which CTA that is) and re-arms the counter.  The ticket releases the CTA's
+    // record (its stores are ordered before by the barrier) and acquires the others'.
     __syncthreads();
     if (threadIdx.x == 0) {
-      __threadfence();   // (the CTA's stores, ordered before by the barrier)
-      const int64_t first = static_cast<int64_t>(cum[b]) * ups + static_cast<int64_t>(k) * nt;
-      const int c_lo = (t0 == 0) ? static_cast<int>(blockIdx.x) : cta_of(first);
-      const int c_hi = (t0 + n == nt) ? static_cast<int>(blockIdx.x) : cta_of(first + nt - 1);
-      int pieces = c_hi - c_lo + 1;
-      if (total < gridDim.x)
-        for (int c = c_lo; c <= c_hi; ++c) pieces -= (start_of(c) == start_of(c + 1)) ? 1 : 0;
-      const unsigned ticket = atomicAdd(a.unit_count + u, 1u);
-      s_merge[0] = (ticket + 1u == static_cast<unsigned>(pieces)) ? 1 : 0;
-      s_merge[1] = c_lo;
-      s_merge[2] = c_hi - c_lo + 1;
+      const unsigned ticket = ticket_add(a.unit_count + u);
+      const bool last = ticket + 1u == static_cast<unsigned>(pieces);
+      s_last = last;
+      if (last) a.unit_count[u] = 0u;
     }
     __syncthreads();
-    if (s_merge[0]) {
-      __threadfence();
-      decode_merge_unit<D>(a, reinterpret_cast<float*>(dsmem), b, k, u, s_merge[1], s_merge[2], total, gridDim.x);
-      if (threadIdx.x == 0) a.unit_count[u] = 0u;
-    }
+    if (s_last) decode_merge_unit<D>(a, reinterpret_cast<float*>(dsmem), b, k, u, c_lo, c_hi - c_lo + 1, total, gridDim.x);
   }
 }
 
