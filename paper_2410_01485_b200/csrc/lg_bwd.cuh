@@ -229,7 +229,7 @@ bwd_dq_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ 
   unsigned int abort_word = 0;
   if (tid == 0) abort_word = *reinterpret_cast<volatile unsigned int*>(a.error_word);
   int cta_x, cta_y;   // (batch, query head) and launch rank of this CTA's query tile
-  cta_coords(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, cta_x, cta_y);
+  cta_coords(blockIdx.y * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, cta_x, cta_y);
   const TileRec rec = load_rec(a.order + cta_y);
   if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 20u)) return;
   const int tile = checked(rec.a, 0, a.n_tiles - 1, a.error_word, 110);
@@ -597,7 +597,7 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     seg = (place - a.split.first_place[reg]) / seg_stride;
     cta_y = a.split.first_rank[reg] + (place - a.split.first_place[reg]) % seg_stride;
   } else {
-    cta_coords2(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.long_group, a.n_long, a.head_group, cta_x, cta_y);
+    cta_coords2(blockIdx.y * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.long_group, a.n_long, a.head_group, cta_x, cta_y);
   }
   const TileRec rec = load_rec(a.order + cta_y);
   if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 10u)) return;
@@ -702,8 +702,8 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
       // A hint only: nothing waits for it and a wrong guess costs two tile reads.
       auto prefetch_successor = [&]() {
         if (kSplit || a.ahead <= 0) return;
-        const int64_t w = static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x + a.ahead;
-        if (w >= static_cast<int64_t>(gridDim.x) * gridDim.y) return;
+        const uint32_t w = blockIdx.y * gridDim.x + blockIdx.x + a.ahead;
+        if (w >= gridDim.x * gridDim.y) return;
         int x2, y2;
         cta_coords2(w, gridDim.x, gridDim.y, a.long_group, a.n_long, a.head_group, x2, y2);
         const TileRec r2 = load_rec(a.order + y2);
@@ -1138,7 +1138,7 @@ bwd_dq_from_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const BwdArgs a,
   if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 80u)) return;
   unsigned int abort_word = 0;
   if (tid == 0) abort_word = *reinterpret_cast<volatile unsigned int*>(a.error_word);
-  const long long n_items = static_cast<long long>(n_heads) * n_ranks;
+  const uint32_t n_items = static_cast<uint32_t>(n_heads) * n_ranks;   // (32 bits: see cta_coords)
   if (tid == 0) {
     for (int i = 0; i < kAS; ++i) { mbar_init(bars + B_AF + i, 1); mbar_init(bars + B_AE + i, 1); }
     for (int i = 0; i < kKS; ++i) { mbar_init(bars + B_KF + i, 1); mbar_init(bars + B_KE + i, 1); }
@@ -1161,7 +1161,7 @@ bwd_dq_from_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const BwdArgs a,
   }
   // item w of the launch order: (batch entry, head), query tile and its schedule entries
   struct Item { int b, h, t, n_ent; const int32_t* ent; };
-  auto item_of = [&](long long w) {
+  auto item_of = [&](uint32_t w) {
     Item it;
     const int x = static_cast<int>(w % n_heads), y = static_cast<int>(w / n_heads);
     it.b = x / a.Hq; it.h = x % a.Hq;
@@ -1182,7 +1182,7 @@ bwd_dq_from_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const BwdArgs a,
       const int64_t zero_tile = static_cast<int64_t>(n_heads) * a.ds_nnz * (BS / 64);                // the tile after the last head's
       bool ok = true;
       int g = 0;   // steps loaded so far, over all items: ring slots and barrier phases follow it
-      for (long long w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
+      for (uint32_t w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
         const Item it = item_of(w);
         const int hk = it.h / a.G;
         const int64_t head_base = (static_cast<int64_t>(it.b) * a.Hq + it.h) * a.ds_nnz * (BS / 64);
@@ -1243,7 +1243,7 @@ bwd_dq_from_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const BwdArgs a,
     bool ok = true;
     int g = 0, n_acc = 0;   // steps consumed and accumulators filled so far, over all items
 #pragma unroll 1
-    for (long long w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
+    for (uint32_t w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
       const Item it = item_of(w);
       if (it.n_ent == 0) continue;
       const uint32_t acc = tmem + (n_acc & 1) * D;
@@ -1274,7 +1274,7 @@ bwd_dq_from_ds_kernel(const __grid_constant__ CUtensorMap tm_k, const BwdArgs a,
     // ------------------------------ epilogue: dQ * scale -> bf16 ----------------------------
     bool ok = true;
     int n_acc = 0;
-    for (long long w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
+    for (uint32_t w = blockIdx.x; w < n_items && ok; w += gridDim.x) {
       const Item it = item_of(w);
       const int qi = it.t * 128 + warp * 32 + lane;
       __nv_bfloat16* base = a.out0 + it.b * a.s0[0] + it.h * a.s0[1];

@@ -322,8 +322,9 @@ constexpr int kHeadGroup = 4;
 constexpr int kHeadGroupCombs = 2;     // strided pattern, dK/dV pass: the comb tiles of this many kv heads at a time
 constexpr int kHeadGroupCombsGqa = 4;  // the same with grouped queries
 constexpr int kHeadGroupFull = 2;   // full causal attention: every tile of a head streams the same rows from the same end
-__device__ __forceinline__ void cta_coords(long long w, int n_x, int n_y, int group, int& x, int& y) {
-  const long long per_group = static_cast<long long>(group) * n_y;
+// (32 bits: a grid holds fewer than 2^32 CTAs, each of which owns at least 16 KB of a tensor; a 64-bit division takes 200 cycles)
+__device__ __forceinline__ void cta_coords(uint32_t w, int n_x, int n_y, int group, int& x, int& y) {
+  const uint32_t per_group = static_cast<uint32_t>(group) * n_y;
   const int grp = static_cast<int>(w / per_group);
   const int rem = static_cast<int>(w - grp * per_group);
   const int size = min(group, n_x - grp * group);   // the last group may be smaller
@@ -338,8 +339,8 @@ __device__ __forceinline__ void cta_coords(long long w, int n_x, int n_y, int gr
 //     groups.  Inside a group alone the longest-first order does not hold over the grid: the last group's sink tiles
 //     started when most of the work was done, and the pass waited for them (3 x 4 kv heads, 6001 tokens, window
 //     1024: SMs busy for 52 % of the pass).
-__device__ __forceinline__ void cta_coords2(long long w, int n_x, int n_y, int long_group, int n_long, int group, int& x, int& y) {
-  const long long first = static_cast<long long>(n_x) * n_long;
+__device__ __forceinline__ void cta_coords2(uint32_t w, int n_x, int n_y, int long_group, int n_long, int group, int& x, int& y) {
+  const uint32_t first = static_cast<uint32_t>(n_x) * n_long;
   if (w < first) { cta_coords(w, n_x, n_long, long_group, x, y); return; }
   cta_coords(w - first, n_x, n_y - n_long, group, x, y);
   y += n_long;

@@ -186,7 +186,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     seg = cut ? y / n_cut : 0;
     cta_y = cut ? y % n_cut : y - n_cut * (a.split.places - 1);
   } else {
-    cta_coords(static_cast<long long>(blockIdx.y) * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, cta_x, cta_y);
+    cta_coords(blockIdx.y * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, cta_x, cta_y);
   }
   const TileRec rec = load_rec(a.order + cta_y);
   if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 1u)) return;
