@@ -945,7 +945,9 @@ bwd_dkdv_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const bool masked = __any_sync(0xffffffffu, xmin > 0 || xmax < C);
         static_assert(C == 32, "one mask word");
         const uint32_t seen = bit_range(xmin, xmax);
-        auto probabilities = [&](auto with_mask) {   // (a loop of its own for the half-steps of which a key sees all)
+        // A loop of its own for the half-steps of which every key sees all, most of them: the mask bits took 12 % of the
+        // instructions (D = 64, 3 x 16 / 4 heads x 6001: pass 244 -> 235 us; D = 128, 32 / 8 heads x 8192 full causal: 1035 -> 1012 us).
+        auto probabilities = [&](auto with_mask) {
 #pragma unroll
           for (int c = 0; c < C; c += 4) {
             const float4 l4 = st_l[c >> 2];

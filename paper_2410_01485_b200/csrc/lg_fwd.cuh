@@ -22,6 +22,7 @@
 // S(0) | PV(0) S(1) | PV(1) S(2) | ...) and 80 registers per thread, hence the half is worked 32 columns at a time (3 x 16 /
 // 4 heads x 6001 tokens, window 1024: 164 -> 148 us with 64- and with 128-token blocks, although 13 / 34 registers are
 // spilled there).  Both forms sum in the same order and give the same bits.
+// Grids of few heads cut long super-tiles along their keys (fwd_split, lg_pattern.h): a CTA per piece, kSplit; fwd_add_kernel adds them.
 // The online softmax advances half by half.  A row's reference (the maximum its probabilities are expressed relative
 // to) only moves, and O is only rescaled, when a half's probabilities sum to more than 2^8;
 // until then they are relative to the older reference, which fp32 / bf16 hold easily, and the
