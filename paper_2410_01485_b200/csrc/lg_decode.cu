@@ -178,7 +178,7 @@ __device__ __forceinline__ void decode_run_segment(const DecodeArgs& a, uint8_t*
     const uint32_t sk = wsm_u32 + stage * 2 * kTileBytes, sv = sk + kTileBytes;
 
     // ---- S^T[16 tokens, 8 heads] = K Q^T ------------------------------------------------
-    float sacc[4] = {0.f, 0.f, 0.f, 0.f}, sodd[4] = {0.f, 0.f, 0.f, 0.f};   // two chains of products: half the latency
+    float sacc[4] = {0.f, 0.f, 0.f, 0.f};   // one chain, in the order of the head dimension
     {
       const int row = ((lane >> 3) & 1) * 8 + (lane & 7);
 #pragma unroll
@@ -186,10 +186,8 @@ __device__ __forceinline__ void decode_run_segment(const DecodeArgs& a, uint8_t*
         const int cc = 2 * k + (lane >> 4);
         uint32_t a0, a1, a2, a3;
         ldsm_x4(sk + row * kRowBytes + ((cc ^ (row & 7)) * 16), a0, a1, a2, a3);
-        mma16816(k & 1 ? sodd : sacc, a0, a1, a2, a3, qf[k][0], qf[k][1]);
+        mma16816(sacc, a0, a1, a2, a3, qf[k][0], qf[k][1]);
       }
-#pragma unroll
-      for (int x = 0; x < 4; ++x) sacc[x] += sodd[x];
     }
     // sacc[0,1]: token r, heads 2c, 2c+1;  sacc[2,3]: token r + 8
     const int tok0 = t * kDecTile + r;
