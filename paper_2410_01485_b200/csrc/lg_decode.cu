@@ -599,6 +599,13 @@ __global__ void __launch_bounds__(128) decode_merge_kernel(const DecodeArgs a) {
 // slot(j) = j < sink ? j : sink + (j - sink) % window.  One group of D/8 threads copies one
 // K row and one V row (16 bytes per thread per row).  A token that a later token of the same
 // call would overwrite is skipped, so the outcome equals appending one at a time.
+// kEarly: the row travels with the count, one round trip before the stores (one token: 1.65 -> 1.19 us).  A call longer than the
+// ring drops most rows, and in one of many rounds of blocks what is worked out for them first costs more than the round
+// trip: 8 heads into 4224 slots, late / early: 8192 tokens 7.06 / 6.72 us, 12288 9.07 / 9.11, 32768 20.0 / 21.1, 131072
+// 71.8 / 78.6; into 640 slots 4096 tokens 3.55 / 3.38, 8192 5.77 / 5.69.  Hence the line at four rounds (ring_append_early).
+constexpr int64_t kAppendEarlyBlocks = 4 * kSms * (2048 / 256);
+static bool ring_append_early(int T, int window, int64_t blocks) { return T <= window || blocks <= kAppendEarlyBlocks; }
+template <bool kEarly>
 __global__ void ring_append_kernel(__nv_bfloat16* k_cache, __nv_bfloat16* v_cache, const __nv_bfloat16* k_new,
                                    const __nv_bfloat16* v_new, const int64_t* n_before, int B, int Hkv, int D, int T,
                                    int sink, int window) {
@@ -613,9 +620,11 @@ __global__ void ring_append_kernel(__nv_bfloat16* k_cache, __nv_bfloat16* v_cach
   const int64_t bh = row_id / T;
   const int b = static_cast<int>(bh / Hkv);
   pdl_wait();
-  // the row travels with the count: one round trip before the stores
-  const uint4 kv = *(reinterpret_cast<const uint4*>(k_new + row_id * D) + ch);
-  const uint4 vv = *(reinterpret_cast<const uint4*>(v_new + row_id * D) + ch);
+  uint4 kv, vv;
+  if (kEarly) {
+    kv = *(reinterpret_cast<const uint4*>(k_new + row_id * D) + ch);
+    vv = *(reinterpret_cast<const uint4*>(v_new + row_id * D) + ch);
+  }
   const int64_t n0 = n_before[b];
   if (n0 < 0) return;                                  // a negative count addresses nothing: the sequence is skipped
   const int64_t j = n0 + t, last = n0 + T - 1;
@@ -624,8 +633,8 @@ __global__ void ring_append_kernel(__nv_bfloat16* k_cache, __nv_bfloat16* v_cach
   const int64_t C = static_cast<int64_t>(sink) + window;
   uint4* kd = reinterpret_cast<uint4*>(k_cache + (bh * C + slot) * D) + ch;
   uint4* vd = reinterpret_cast<uint4*>(v_cache + (bh * C + slot) * D) + ch;
-  *kd = kv;
-  *vd = vv;
+  *kd = kEarly ? kv : *(reinterpret_cast<const uint4*>(k_new + row_id * D) + ch);
+  *vd = kEarly ? vv : *(reinterpret_cast<const uint4*>(v_new + row_id * D) + ch);
 }
 
 static lg_status check_decode(const lg_decode_params* p) {
@@ -720,7 +729,8 @@ lg_status lg_kv_ring_append(const lg_decode_params* p, void* k_cache, void* v_ca
   const int64_t threads = static_cast<int64_t>(p->B) * p->Hkv * T_new * (p->D / 8);
   const int64_t blocks = (threads + 255) / 256;
   if (blocks > 0x7fffffff) return LG_ERR_UNSUPPORTED;
-  return launch_kernel(true, ring_append_kernel, dim3(static_cast<unsigned>(blocks)), 256, 0, static_cast<cudaStream_t>(stream),
+  return launch_kernel(true, ring_append_early(T_new, p->window_tokens, blocks) ? ring_append_kernel<true> : ring_append_kernel<false>,
+                       dim3(static_cast<unsigned>(blocks)), 256, 0, static_cast<cudaStream_t>(stream),
                            static_cast<__nv_bfloat16*>(k_cache), static_cast<__nv_bfloat16*>(v_cache),
                            static_cast<const __nv_bfloat16*>(k_new), static_cast<const __nv_bfloat16*>(v_new), n_tokens_before,
                            p->B, p->Hkv, p->D, T_new, p->sink_tokens, p->window_tokens) == cudaSuccess ? LG_OK : LG_ERR_CUDA;
