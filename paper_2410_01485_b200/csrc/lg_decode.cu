@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
   const int ups = a.Hkv * a.HG;
   bool any_empty;
   int tiles;
-  int64_t total, f0, f1;
+  int64_t total, f0 = 0, f1 = 0;
   bool narrow;                             // the slices' arithmetic fits 32 bits (64-bit divisions take 200 cycles each)
   auto start_of = [&](int64_t c) -> int64_t {
     return narrow ? static_cast<uint32_t>(total) * static_cast<uint32_t>(c) / gridDim.x : total * c / gridDim.x;
@@ -512,7 +512,8 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
   // divisions and the chain of loads were 1.5 us behind the wait, two fences (fence.sc) of 1.3 us each went with the acquiring and
   // releasing ticket: append + decode of one sequence over 4224 slots, 64 / 8 heads,
   // 12.7 -> 11.6 us, of 16 sequences 47.2 -> 46.2 us (13.7 and 49.2 us before the hint).
-  plan();
+  // With more sequences than threads a count would be read twice and the readings could differ: no plan and no hint.
+  if (a.B <= kDecThreads) plan();
   if (f0 < f1 && (threadIdx.x & 31) < 2) {
     const int tb = t0 + static_cast<int>(static_cast<int64_t>(n) * warp / kDecWarps);
     const int te = min(t0 + static_cast<int>(static_cast<int64_t>(n) * (warp + 1) / kDecWarps), tb + kDecHintTiles);
@@ -523,7 +524,6 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
     }
   }
   pdl_wait();
-  // (with more sequences than threads they are simply counted again)
   int nvalid = f0 < f1 ? decode_valid_of(a, b) : 0;        // (travels with the counts)
   const bool changed = a.B > kDecThreads || (threadIdx.x < a.B && decode_tiles_of(a, threadIdx.x) != tiles);
   if (__syncthreads_or(changed)) {
