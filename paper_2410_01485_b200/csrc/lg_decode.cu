@@ -111,7 +111,7 @@ __device__ __forceinline__ void decode_run_segment(const DecodeArgs& a, uint8_t*
   int ex0 = 0, ex_cnt = 0;
   const int ring_w = a.C - a.sink;
   if (a.block_tokens > 0) {
-    const int64_t n = __ldcg(reinterpret_cast<const long long*>(a.n_tokens) + b);
+    const int64_t n = a.n_tokens[b];
     if (n > a.C) {                                  // before the ring has wrapped nothing is left out
       const int64_t first_held = n - ring_w;        // oldest window token in the ring (>= sink here)
       const int64_t first_kept = ((n - 1) / a.block_tokens - ring_w / a.block_tokens + 1) * a.block_tokens;
@@ -263,10 +263,10 @@ __device__ __forceinline__ void decode_run_segment(const DecodeArgs& a, uint8_t*
     }
   }
   __syncthreads();
-  {   // a warp per head: its weights once per thread, then D / 32 neighbouring values of a lane
+  {   // a warp per head: its weights once per thread, then D / 32 values of a lane, two neighbours at a time (four: two-way conflicts)
     static_assert(kDecWarps == kDecHeads && (D / 32) % 2 == 0, "a warp per head");
     constexpr int V = D / 32;
-    const int head = warp, d = lane * V;
+    const int head = warp, d = lane * 2;                 // values d, d + 1, and every 64 on
     const float* mine = red + head * kRec;               // the head's row of warp 0's record
     float f[kDecWarps], m = -INFINITY, l = 0.f, acc[V] = {};
 #pragma unroll
@@ -278,7 +278,7 @@ __device__ __forceinline__ void decode_run_segment(const DecodeArgs& a, uint8_t*
       l += f[w] * mine[w * kDecHeads * kRec + D + 1];
 #pragma unroll
       for (int x = 0; x < V; x += 2) {
-        const float2 o2 = *reinterpret_cast<const float2*>(mine + w * kDecHeads * kRec + d + x);
+        const float2 o2 = *reinterpret_cast<const float2*>(mine + w * kDecHeads * kRec + d + 32 * x);
         acc[x] += f[w] * o2.x;
         acc[x + 1] += f[w] * o2.y;
       }
@@ -289,12 +289,12 @@ __device__ __forceinline__ void decode_run_segment(const DecodeArgs& a, uint8_t*
         const int64_t qh = static_cast<int64_t>(b) * a.Hq + kvh * a.G + gh;
 #pragma unroll
         for (int x = 0; x < V; x += 2)
-          *reinterpret_cast<uint32_t*>(a.o + qh * D + d + x) = l > 0.f ? pack_bf16(acc[x] / l, acc[x + 1] / l) : 0u;
+          *reinterpret_cast<uint32_t*>(a.o + qh * D + d + 32 * x) = l > 0.f ? pack_bf16(acc[x] / l, acc[x + 1] / l) : 0u;
         if (lane == 0 && a.lse) a.lse[qh] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
       }
     } else {
 #pragma unroll
-      for (int x = 0; x < V; x += 2) *reinterpret_cast<float2*>(out + head * D + d + x) = make_float2(acc[x], acc[x + 1]);
+      for (int x = 0; x < V; x += 2) *reinterpret_cast<float2*>(out + head * D + d + 32 * x) = make_float2(acc[x], acc[x + 1]);
       if (lane == 0) { out[kDecHeads * D + 2 * head] = m; out[kDecHeads * D + 2 * head + 1] = l; }
     }
   }
@@ -329,10 +329,12 @@ constexpr int kDecFlatMaxCtas = 320;    // upper bound of its grid (two CTAs per
 // 0.996x for short caches, 5 are 0.988x and 1.000x (what is asked for competes with the tail of the step before).
 constexpr int kDecHintTiles = 3;
 
-// (n_tokens is read through the L2: it is looked at once before the wait of an overlapped launch and again after it)
+// (n_tokens is read through the L2 where it may be looked at before the wait of an overlapped launch, and when it is looked at again
+// behind it; the later segments read it the ordinary way: a trip to the L2 for each of a CTA's 10-20 units was 2-5 % of decodes
+// of many short sequences, 2048 x 8 heads over 128 slots 195 -> 185 us)
+__device__ __forceinline__ int decode_clamped(const DecodeArgs& a, int64_t n) { return static_cast<int>(n < a.C ? (n < 0 ? 0 : n) : a.C); }
 __device__ __forceinline__ int decode_valid_of(const DecodeArgs& a, int b) {
-  const int64_t n = __ldcg(reinterpret_cast<const long long*>(a.n_tokens) + b);
-  return static_cast<int>(n < a.C ? (n < 0 ? 0 : n) : a.C);
+  return decode_clamped(a, __ldcg(reinterpret_cast<const long long*>(a.n_tokens) + b));
 }
 __device__ __forceinline__ int decode_tiles_of(const DecodeArgs& a, int b) {
   return (decode_valid_of(a, b) + kDecTile - 1) / kDecTile;
@@ -542,7 +544,7 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
   for (int64_t pos = f0; pos < f1;) {
     if (pos != f0) {
       segment(pos);
-      nvalid = decode_valid_of(a, b);
+      nvalid = decode_clamped(a, a.n_tokens[b]);
     }
     const int tb = t0 + static_cast<int>(static_cast<int64_t>(n) * warp / kDecWarps);
     const int te = t0 + static_cast<int>(static_cast<int64_t>(n) * (warp + 1) / kDecWarps);
