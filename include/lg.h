@@ -118,8 +118,7 @@ size_t lg_sparse_attn_workspace_bytes(const lg_attn_params* p, int want_bwd);
  * lg_sparse_attn_fwd (and, with want_bwd != 0, lg_sparse_attn_bwd) called with the same
  * workspace, the same pattern (L, block, mode, sink / window / stride / local counts,
  * window_exact, doc_start pointer) and lists_prepared = 1 launch their attention kernels only:
- * one kernel for the forward (two where few long rows are cut along their keys), three for the
- * backward.  The lists do not depend on the head
+ * one kernel for the forward, three for the backward.  The lists do not depend on the head
  * counts, on D or on the strides.  With doc_start the lists also depend on the CONTENTS of that
  * array: prepare again whenever they change.  The workspace keeps a fingerprint of what it was
  * prepared for; a call with lists_prepared = 1 whose pattern does not match it launches kernels

@@ -197,16 +197,6 @@ WsLayout ws_layout(const Resolved& r, bool want_bwd) {
   w.sq_cnt = take(r.n_stiles * 4);
   w.sq_ent = take(nnz * 4);
   w.sq_order = take(r.n_stiles * sizeof(TileRec));
-  size_t fwd_end = 0;
-  if (r.fsplit.len > 0) {
-    // The pieces' sums lie behind all lists, the backward's too (at most so long), whatever the head counts: one workspace
-    // serves both directions.  They are scratch of the forward, what a backward keeps there is scratch of its own.
-    const size_t lists = align_up(nnz * kDqEntInts * 4, 256) + align_up(nnz * 4, 256) + 14 * align_up(static_cast<size_t>(r.n_qtiles) * 4, 256);
-    const size_t pieces = static_cast<size_t>(r.B) * r.Hq * r.fsplit.n_cut * r.fsplit.places;
-    w.fwd_ml = off + lists;
-    w.fwd_part = w.fwd_ml + pieces * 256 * 8;
-    fwd_end = w.fwd_part + pieces * 256 * r.D * 4;
-  }
   if (want_bwd) {
     const bool keep = bwd_variant(r) == kBwdKeepDs;
     w.qt_off = take(static_cast<size_t>(r.n_qtiles) * 4);
@@ -228,7 +218,7 @@ WsLayout ws_layout(const Resolved& r, bool want_bwd) {
       w.kv_ticket = take(heads * split.n_ranks * 4);
     }
   }
-  w.total = off > fwd_end ? off : fwd_end;
+  w.total = off;
   return w;
 }
 

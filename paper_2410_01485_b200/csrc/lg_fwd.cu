@@ -31,15 +31,14 @@ static lg_status launch_fwd_t(const Resolved& r, const WsLayout& w, const void* 
   a.scale_log2 = r.scale * 1.4426950408889634f;
   a.head_group = head_group(r, r.B * r.Hq);
   a.split = r.fsplit;
-  a.part = reinterpret_cast<float4*>(ws + w.fwd_part);
-  a.part_ml = reinterpret_cast<float2*>(ws + w.fwd_ml);
   auto kern = fwd_kernel<D, BS, NB, kSplit>;
   constexpr int smem = FwdSmem<D>::kTotal;
   static std::atomic<bool> allowed[kMaxDevices];
-  dim3 grid(r.B * r.Hq, r.n_stiles + (kSplit ? r.fsplit.n_cut * (r.fsplit.places - 1) : 0));
-  if (launch_big_smem(launch_attn_overlapped(r), allowed, kern, grid, kFwdThreads, smem, stream, tq, tk, tv, a) != cudaSuccess) return LG_ERR_CUDA;
-  if (kSplit && launch_kernel(true, fwd_add_kernel<D, BS>, dim3(r.B * r.Hq, r.fsplit.n_cut, 256 / 32), kFwdAddThreads, 0, stream, a) != cudaSuccess) return LG_ERR_CUDA;
-  return LG_OK;
+  // cut tiles: clusters of as many CTAs as a tile has places; the last cluster is filled up
+  const int cluster = kSplit ? r.fsplit.places : 1;
+  const int n_y = r.n_stiles + (kSplit ? r.fsplit.n_cut * (cluster - 1) : 0);
+  const dim3 grid(r.B * r.Hq, (n_y + cluster - 1) / cluster * cluster);
+  return launch_big_smem_clusters(launch_attn_overlapped(r), cluster, allowed, kern, grid, kFwdThreads, smem, stream, tq, tk, tv, a) == cudaSuccess ? LG_OK : LG_ERR_CUDA;
 }
 
 lg_status launch_fwd(const Resolved& r, const WsLayout& w, const void* q, const void* k, const void* v, void* o,

@@ -22,7 +22,8 @@
 // S(0) | PV(0) S(1) | PV(1) S(2) | ...) and 80 registers per thread, hence the half is worked 32 columns at a time (3 x 16 /
 // 4 heads x 6001 tokens, window 1024: 164 -> 148 us with 64- and with 128-token blocks, although 13 / 34 registers are
 // spilled there).  Both forms sum in the same order and give the same bits.
-// Grids of few heads cut long super-tiles along their keys (fwd_split, lg_pattern.h): a CTA per piece, kSplit; fwd_add_kernel adds them.
+// Grids of few heads cut long super-tiles along their keys (fwd_split, lg_pattern.h): kSplit, a CTA per piece, a tile's in one
+// cluster, which adds them (fwd_join).
 // The online softmax advances half by half.  A row's reference (the maximum its probabilities are expressed relative
 // to) only moves, and O is only rescaled, when a half's probabilities sum to more than 2^8;
 // until then they are relative to the older reference, which fp32 / bf16 hold easily, and the
@@ -56,8 +57,6 @@ struct FwdArgs {
   float scale_log2;          // scale * log2(e)
   int head_group;            // heads whose CTAs run side by side (cta_coords); >= gridDim.x: all of them
   FwdSplit split;            // tiles cut along their keys
-  float4* part;              // pieces' sums as they stand, [cut tile, head][place][D / 4][256 rows]
-  float2* part_ml;           // (reference, sum of probabilities) of their rows, [cut tile, head][place][256 rows]
 };
 
 constexpr int kFwdTmaWarp = 8, kFwdMmaWarp0 = 9;
@@ -79,69 +78,69 @@ struct FwdSmem {
 // Pieces of a tile that walks n_steps steps and is one of the ranks that are cut.
 __device__ __forceinline__ int fwd_pieces(const FwdSplit& k, int n_steps) { return n_steps > k.len ? min((n_steps + k.len - 1) / k.len, k.places) : 1; }
 
-// Adds the pieces of the cut tiles, in their order, and writes O and LSE.  grid = (heads, cut ranks, 8): 32 rows of a tile,
-// their sums read 512 contiguous bytes at a time from the L2, all pieces' on their way together, the rows written whole through
-// shared memory.  (Added by the CTA that delivers a tile's last piece, behind a ticket, a tile's 0.4-0.8 MB took one SM 15 us.)
-constexpr int kFwdAddThreads = 256;
-template <int D, int BS>
-__global__ void __launch_bounds__(kFwdAddThreads) fwd_add_kernel(const FwdArgs a) {
-  pdl_trigger();
-  pdl_wait();
-  if (!lists_match(a.error_word, a.expect_fp, a.expect_fp2, 1u)) return;
-  if (__syncthreads_or(*reinterpret_cast<volatile unsigned int*>(a.error_word) != 0)) return;   // a piece was given up
-  const TileRec rec = load_rec(a.order + blockIdx.y);
-  const int tile = checked(rec.a, 0, a.n_tiles - 1, a.error_word, 103);
-  const int n_ent = checked(rec.cnt, 0, a.n_list, a.error_word, 104);
-  const int n_segs = fwd_pieces(a.split, (BS == 128) ? n_ent : (n_ent + 1) / 2);
-  if (n_segs == 1) return;                                        // written by its CTA
-  const int64_t unit = static_cast<int64_t>(blockIdx.y) * gridDim.x + blockIdx.x;
-  const int b = blockIdx.x / a.Hq, h = blockIdx.x % a.Hq, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r0 = blockIdx.z * 32, row = a.row_origin + tile * 256 + r0 + lane;   // a lane per row
-  const float2* ml = a.part_ml + unit * a.split.places * 256 + r0 + lane;
-  float w[kFwdMaxPieces], m = -INFINITY, l = 0.f;
-  float2 pair[kFwdMaxPieces];
+// Joins the pieces of a cut tile inside its cluster.  Every CTA has laid its sums as they stand into its own shared memory, a row
+// of D + 4 floats each (writes of a lane per row and reads along a row both without bank conflicts), and the rows'
+// (reference, sum of probabilities) behind them; the CTA of piece `seg` adds its share of the 256 rows over all pieces, in
+// their order, and writes O and LSE.  Nothing of it lies in global memory: calls that share a workspace share lists only.
+template <int D>
+struct FwdJoin {
+  static constexpr int kRow = (D + 4) * 4, oMl = 256 * kRow, kBytes = oMl + 256 * 8;
+};
+// Rows r0, r0 + step, .. below `end` of a tile of up to N pieces, kBatch of them at a time: a load from another SM takes 1000
+// cycles, so that one row after the other the share of a CTA took 6-8 us (4 heads x 3318 tokens, full causal, D = 128, two
+// pieces a tile: 45.1 us, in batches 41.1).
+template <int D, int N, int kBatch>
+__device__ __forceinline__ void fwd_join_rows(const FwdArgs& a, uint32_t base, int n_segs, int b, int h, int row0, int r0, int end, int step, int c) {
+  for (; r0 < end; r0 += kBatch * step) {
+    float2 pair[kBatch][N];
+    float4 v[kBatch][N];
 #pragma unroll
-  for (int i = 0; i < kFwdMaxPieces; ++i) {
-    pair[i] = i < n_segs ? __ldcg(ml + i * 256) : make_float2(-INFINITY, 0.f);
-    m = fmaxf(m, pair[i].x);
-  }
-  const float mu = m == -INFINITY ? 0.f : m;
+    for (int x = 0; x < kBatch; ++x)
 #pragma unroll
-  for (int i = 0; i < kFwdMaxPieces; ++i) {
-    w[i] = fast_exp2(pair[i].x - mu);                             // (a piece no key of which the row sees: 0)
-    if (i < n_segs) l += w[i] * pair[i].y;
-  }
-  const float inv = l > 0.f ? 1.f / l : l;                        // 0 where the row sees nothing, NaN stays NaN
-  __shared__ __align__(16) uint8_t stage[32 * (D * 2 + 16)];      // rows, 16 bytes apart from a multiple of the banks
-  const float4* part = a.part + unit * a.split.places * (D / 4 * 256) + r0 + lane;
-  constexpr int kCols = D / 4 / (kFwdAddThreads / 32);            // groups of four columns of a warp
-  float4 v[kCols][kFwdMaxPieces];
-#pragma unroll
-  for (int c = 0; c < kCols; ++c)
-#pragma unroll
-    for (int i = 0; i < kFwdMaxPieces; ++i)
-      if (i < n_segs) v[c][i] = __ldcg(part + (static_cast<int64_t>(i) * (D / 4) + warp * kCols + c) * 256);
-#pragma unroll
-  for (int c = 0; c < kCols; ++c) {
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-    for (int i = 0; i < kFwdMaxPieces; ++i)
-      if (i < n_segs && w[i] != 0.f) {                            // (otherwise its sums may never have been written)
-        acc.x += w[i] * v[c][i].x; acc.y += w[i] * v[c][i].y; acc.z += w[i] * v[c][i].z; acc.w += w[i] * v[c][i].w;
+      for (int i = 0; i < N; ++i) {
+        const int r = r0 + x * step;
+        pair[x][i] = make_float2(-INFINITY, 0.f);
+        if (i < n_segs && r < end) {
+          const uint32_t peer = cluster_addr(base, i);
+          pair[x][i] = cluster_ld64(peer + FwdJoin<D>::oMl + r * 8);
+          v[x][i] = cluster_ld128(peer + r * FwdJoin<D>::kRow + c * 16);
+        }
       }
-    *reinterpret_cast<uint2*>(stage + lane * (D * 2 + 16) + (warp * kCols + c) * 8) =
-        make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
+#pragma unroll
+    for (int x = 0; x < kBatch; ++x) {
+      float m = -INFINITY, l = 0.f;
+#pragma unroll
+      for (int i = 0; i < N; ++i) m = fmaxf(m, pair[x][i].x);
+      const float mu = m == -INFINITY ? 0.f : m;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        const float w = fast_exp2(pair[x][i].x - mu);             // (0 for a piece no key of which the row sees,
+        l += w * pair[x][i].y;
+        if (pair[x][i].x == -INFINITY) continue;                  // which may not have written its sums)
+        acc.x += w * v[x][i].x; acc.y += w * v[x][i].y; acc.z += w * v[x][i].z; acc.w += w * v[x][i].w;
+      }
+      const float inv = l > 0.f ? 1.f / l : l;                    // 0 where the row sees nothing, NaN stays NaN
+      const int r = r0 + x * step, q = row0 + r;
+      if (r < end && q < a.L && q >= a.q_start) {
+        *reinterpret_cast<uint2*>(a.o + b * a.o_strides[0] + h * a.o_strides[1] + static_cast<int64_t>(q - a.q_start) * a.o_strides[2] + c * 4) =
+            make_uint2(pack_bf16(acc.x * inv, acc.y * inv), pack_bf16(acc.z * inv, acc.w * inv));
+        if (c == 0) a.lse[(static_cast<int64_t>(b) * a.Hq + h) * a.Lq + q - a.q_start] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
+      }
+    }
   }
-  if (warp == 0 && row < a.L && row >= a.q_start)
-    a.lse[(static_cast<int64_t>(b) * a.Hq + h) * a.Lq + row - a.q_start] = l > 0.f ? (m + log2f(l)) * 0.6931471805599453f : -INFINITY;
-  __syncthreads();
-  constexpr int kChunks = D / 8;                                  // 16-byte chunks of a row
-  for (int u = threadIdx.x; u < 32 * kChunks; u += kFwdAddThreads) {
-    const int r = u / kChunks, c = u % kChunks, q = row - lane + r;
-    if (q < a.L && q >= a.q_start)
-      *reinterpret_cast<uint4*>(a.o + b * a.o_strides[0] + h * a.o_strides[1] + static_cast<int64_t>(q - a.q_start) * a.o_strides[2] + c * 8) =
-          *reinterpret_cast<const uint4*>(stage + r * (D * 2 + 16) + c * 16);
-  }
+}
+template <int D>
+__device__ __forceinline__ void fwd_join(const FwdArgs& a, uint32_t base, uint32_t failed_flag, int seg, int n_segs, int b, int h, int row0) {
+  constexpr int kLanes = D / 4, kRows = 32 / kLanes;              // lanes of a row (four columns each), rows of a warp
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = lane % kLanes;
+  uint32_t failed = 0;
+  for (int i = 0; i < n_segs; ++i) failed |= cluster_ld32(cluster_addr(failed_flag, i));
+  if (failed) return;                                             // a piece was given up: the status word says so
+  const int first = 256 * seg / n_segs + warp * kRows + lane / kLanes, end = 256 * (seg + 1) / n_segs, step = kFwdThreads / 32 * kRows;
+  if (n_segs <= 2) fwd_join_rows<D, 2, 6>(a, base, n_segs, b, h, row0, first, end, step, c);
+  else if (n_segs <= 4) fwd_join_rows<D, 4, 4>(a, base, n_segs, b, h, row0, first, end, step, c);
+  else fwd_join_rows<D, 8, 2>(a, base, n_segs, b, h, row0, first, end, step, c);
 }
 
 template <int D, int BS, int NB /* score buffers per slot */, bool kSplit>
@@ -162,8 +161,8 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
 
   extern __shared__ __align__(1024) uint8_t smem[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SM::oBar);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + B_COUNT);
-  static_assert(B_COUNT * 8 + 8 <= 256, "barrier area too small");
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + B_COUNT);   // address, an earlier failure, a failure of this CTA's piece
+  static_assert(B_COUNT * 8 + 12 <= 256, "barrier area too small");
   static_assert(fwd_ctas_per_sm(NB) * (SM::kTotal + 1024) <= 228 * 1024 && kColO + 2 * D <= kTmemCols, "does not fit an SM");
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // same value, known to be warp-uniform
@@ -180,12 +179,13 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   int seg = 0;        // which piece of the tile
   bool cut = false;   // one of the ranks that are cut
   if constexpr (kSplit) {
-    // the pieces of the ranks that are cut in turn, the tiles side by side
+    // a cluster of `places` CTAs per cut tile, then the other tiles one by one (and what fills up their last cluster)
     cta_x = static_cast<int>(blockIdx.x);
     const int y = static_cast<int>(blockIdx.y), n_cut = a.split.n_cut;
     cut = y < n_cut * a.split.places;
-    seg = cut ? y / n_cut : 0;
-    cta_y = cut ? y % n_cut : y - n_cut * (a.split.places - 1);
+    seg = cut ? y % a.split.places : 0;
+    cta_y = cut ? y / a.split.places : y - n_cut * (a.split.places - 1);
+    if (cta_y >= a.n_tiles) return;
   } else {
     cta_coords(blockIdx.y * gridDim.x + blockIdx.x, gridDim.x, gridDim.y, a.head_group, cta_x, cta_y);
   }
@@ -203,14 +203,14 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   const int row0 = a.row_origin + tile * 256;
   int n_steps = (BS == 128) ? n_ent : (n_ent + 1) / 2;
   const int n_segs = kSplit && cut ? fwd_pieces(a.split, n_steps) : 1;
-  if (kSplit && seg >= n_segs) return;                     // an empty place (uniform over the CTA)
-  if (kSplit && n_segs > 1) {
+  if (kSplit && seg >= n_segs) return;                     // an empty place (uniform over the CTA; the cluster's barriers count who is left)
+  const bool joint = kSplit && n_segs > 1;                 // the same in all CTAs of the cluster that are left
+  if (joint) {
     const int first = n_steps * seg / n_segs, end = n_steps * (seg + 1) / n_segs;
     ent += (128 / BS) * first;
     n_ent = min(n_ent - (128 / BS) * first, (128 / BS) * (end - first));
     n_steps = end - first;
   }
-  const int64_t unit = kSplit ? static_cast<int64_t>(cta_y) * gridDim.x + cta_x : 0;   // of a cut tile
 
   // entries of the two halves of step j (0: nobody's member, also past the end)
   auto load_ent = [&](int j, int& e0, int& e1) {
@@ -229,7 +229,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     }
     for (int i = 0; i < 4; ++i) { mbar_init(bars + B_SF + i, 1); mbar_init(bars + B_PF + i, 4); mbar_init(bars + B_OD + i, 1); }
     mbar_fence_init();
-    tmem_slot[1] = abort_word;
+    tmem_slot[1] = tmem_slot[2] = abort_word;
   }
   if (warp == kFwdMmaWarp0) {
     tmem_alloc(tmem_slot, kTmemCols);
@@ -240,10 +240,17 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   if (tmem_slot[1] != 0) {   // after a failed wait the rest of the grid does nothing: the call ends in seconds, not minutes
-    if (warp == kFwdMmaWarp0) tmem_dealloc(tmem, kTmemCols);
-    return;
+    if (!joint) {
+      if (warp == kFwdMmaWarp0) tmem_dealloc(tmem, kTmemCols);
+      return;
+    }
+    n_steps = n_ent = 0;                                   // (others of the cluster may be waiting for me)
   }
 
+  // of a softmax thread's row:
+  float m_ref = -INFINITY;   // reference maximum (scaled, log2 domain) the probabilities are relative to
+  float l_run = 0.f;
+  int p0 = 0, p1 = 0;        // P tiles published per score buffer (barrier phases)
   if (warp == kFwdTmaWarp) {
     // ------------------------------ TMA producer ------------------------------------------
     if (lane == 0) {
@@ -284,6 +291,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
         load_step(sV + sv * kTile, &tm_v, bars + B_VF + sv, kb0, kb1);
         nv = j + 1;
       }
+      if (kSplit && !ok) tmem_slot[2] = 1;
       // every copy this thread started has landed before the CTA may exit
       mbar_wait(bars + B_Q, 0, a.error_word, 4);
       for (int j = max(nk - 3, 0); j < nk; ++j) mbar_wait(bars + B_KF + j % 3, (j / 3) & 1, a.error_word, 5);
@@ -364,6 +372,7 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
       ne0 = nn0; ne1 = nn1;
       load_ent(j + 3, nn0, nn1);   // read ahead: off the critical path
     }
+    if (kSplit && !ok) tmem_slot[2] = 1;
     if (lead) mma_commit(bars + B_DRAIN + s);
     mbar_wait(bars + B_DRAIN + s, 0, a.error_word, 11);   // nothing of ours is still running at exit
   } else {
@@ -381,9 +390,6 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     const int win_lo = a.win_block > 0
                            ? ((qi + a.win_phase) / a.win_block - a.exact_w / a.win_block + 1) * a.win_block - a.win_phase
                            : qi - a.exact_w + 1;
-    float m_ref = -INFINITY;   // reference maximum (scaled, log2 domain) the probabilities are relative to
-    float l_run = 0.f;
-    int p0 = 0, p1 = 0;        // P tiles published per score buffer (barrier phases)
     // every P V product issued so far has completed (at most one per buffer can still be running)
     auto wait_o = [&](uint32_t site) {
       bool w = true;
@@ -508,28 +514,9 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
     }
     // ---- epilogue: O / l -> bf16, LSE ------------------------------------------------------
     if (ok) ok = wait_o(14);
-    if (kSplit && n_segs > 1) {
-      // a piece of a cut tile: the sums as they stand, 512 contiguous bytes per store instruction of a warp
-      if (ok) {
-        const int64_t at = unit * a.split.places + seg;
-        const int row = s * 128 + r;
-        if (p0 + p1 > 0) {
-          tc_fence_after();
-          float4* part = a.part + at * (D / 4 * 256) + row;
-#pragma unroll
-          for (int c = 0; c < D; c += 32) {
-            uint32_t reg[32];
-            tmem_ld32(my_o + c, reg);
-            tmem_ld_wait();
-#pragma unroll
-            for (int x = 0; x < 32; x += 4)
-              part[((c + x) / 4) * 256] = make_float4(__uint_as_float(reg[x]), __uint_as_float(reg[x + 1]),
-                                                      __uint_as_float(reg[x + 2]), __uint_as_float(reg[x + 3]));
-          }
-        }
-        a.part_ml[at * 256 + row] = make_float2(l_run == 0.f ? -INFINITY : m_ref, l_run);
-      }
-      ok = false;   // (the rows are not mine to write)
+    if (joint) {                                             // a piece's sums stay as they are until both slots are done
+      if (!ok) tmem_slot[2] = 1;
+      ok = false;                                            // (the rows are not mine to write)
     }
     // warp-uniform condition (the tensor-memory loads below need the whole warp): some row of the warp
     // is a real query; rows past L or before q_start load with the others and store nothing
@@ -555,6 +542,33 @@ fwd_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUt
   }
   tc_fence_before();
   __syncthreads();
+  if constexpr (kSplit) {
+    if (joint) {
+      // all copies have landed and all products are done: the operand buffers hold the sums from here on
+      static_assert(FwdJoin<D>::kBytes <= SM::oBar, "the sums fit where the operands were");
+      tc_fence_after();
+      if (warp < kFwdTmaWarp) {
+        const int row = warp * 32 + lane;                  // slot, row of the slot
+        if (p0 + p1 > 0) {                                 // (uniform over the slot)
+          const uint32_t my_o = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + kColO + (warp >> 2) * D;
+#pragma unroll
+          for (int c = 0; c < D; c += 32) {
+            uint32_t reg[32];
+            tmem_ld32(my_o + c, reg);
+            tmem_ld_wait();
+#pragma unroll
+            for (int x = 0; x < 32; x += 4)
+              *reinterpret_cast<uint4*>(smem + row * FwdJoin<D>::kRow + (c + x) * 4) = make_uint4(reg[x], reg[x + 1], reg[x + 2], reg[x + 3]);
+          }
+        }
+        *reinterpret_cast<float2*>(smem + FwdJoin<D>::oMl + row * 8) = make_float2(l_run == 0.f ? -INFINITY : m_ref, l_run);
+        tc_fence_before();
+      }
+      cluster_sync();                                      // (threads of CTAs that have left are not waited for)
+      fwd_join<D>(a, smem_u32(smem), smem_u32(tmem_slot + 2), seg, n_segs, b, h, row0);
+      cluster_sync();                                      // nobody leaves while its sums are being read
+    }
+  }
   if (warp == kFwdMmaWarp0) tmem_dealloc(tmem, kTmemCols);
 }
 

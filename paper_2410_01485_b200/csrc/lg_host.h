@@ -40,34 +40,53 @@ constexpr int kMaxDevices = 64;   // devices whose properties are looked up once
 // start while the kernel before it on the stream drains.  A failed launch is reported by the result alone: it does not
 // stay behind as the runtime's last error, which a later call would take for its own.
 template <typename... Params, typename... Args>
-inline cudaError_t launch_kernel(bool overlap, void (*kern)(Params...), dim3 grid, int block, int smem, cudaStream_t stream, const Args&... args) {
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+inline cudaError_t launch_clusters(bool overlap, int cluster_y, void (*kern)(Params...), dim3 grid, int block, int smem, cudaStream_t stream,
+                                   const Args&... args) {
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (overlap) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster_y > 1) {   // clusters of 1 x cluster_y CTAs
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = attr[n].val.clusterDim.z = 1;
+    attr[n++].val.clusterDim.y = static_cast<unsigned>(cluster_y);
+  }
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid; cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = smem; cfg.stream = stream;
-  cfg.attrs = &attr; cfg.numAttrs = overlap ? 1 : 0;
+  cfg.attrs = attr; cfg.numAttrs = n;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...);
   if (e == cudaSuccess) note_launch();
   else cudaGetLastError();
   return e;
 }
 
+template <typename... Params, typename... Args>
+inline cudaError_t launch_kernel(bool overlap, void (*kern)(Params...), dim3 grid, int block, int smem, cudaStream_t stream, const Args&... args) {
+  return launch_clusters(overlap, 1, kern, grid, block, smem, stream, args...);
+}
+
 // The same for a kernel that needs more dynamic shared memory than a launch may ask for by default (allowed once per
 // device; a call on every launch cost the host a microsecond).
 template <typename... Params, typename... Args>
-inline cudaError_t launch_big_smem(bool overlap, std::atomic<bool>* allowed /* [kMaxDevices] of this kernel */, void (*kern)(Params...), dim3 grid,
+inline cudaError_t launch_big_smem_clusters(bool overlap, int cluster_y, std::atomic<bool>* allowed /* [kMaxDevices] of this kernel */, void (*kern)(Params...), dim3 grid,
                                    int block, int smem, cudaStream_t stream, const Args&... args) {
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   const bool known = dev < kMaxDevices && allowed[dev].load(std::memory_order_acquire);
-  if (known && launch_kernel(overlap, kern, grid, block, smem, stream, args...) == cudaSuccess) return cudaSuccess;
+  if (known && launch_clusters(overlap, cluster_y, kern, grid, block, smem, stream, args...) == cudaSuccess) return cudaSuccess;
   // (a device that was reset has forgotten it)
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) { cudaGetLastError(); return e; }
   if (dev < kMaxDevices) allowed[dev].store(true, std::memory_order_release);
-  return launch_kernel(overlap, kern, grid, block, smem, stream, args...);
+  return launch_clusters(overlap, cluster_y, kern, grid, block, smem, stream, args...);
+}
+template <typename... Params, typename... Args>
+inline cudaError_t launch_big_smem(bool overlap, std::atomic<bool>* allowed, void (*kern)(Params...), dim3 grid, int block, int smem, cudaStream_t stream,
+                                   const Args&... args) {
+  return launch_big_smem_clusters(overlap, 1, allowed, kern, grid, block, smem, stream, args...);
 }
 
 struct Resolved {          // validated, defaulted copy of lg_attn_params
@@ -98,7 +117,6 @@ lg_status resolve(const lg_attn_params* p, Resolved* r, bool want_bwd = false, i
 struct WsLayout {
   // per schedule: start of each tile's entries, their number, the entries, launch rank -> tile
   size_t sq_off, sq_cnt, sq_ent, sq_order;       // super-tiles (forward)
-  size_t fwd_ml, fwd_part;                       // forward with cut tiles: the pieces' sums
   size_t qt_off, qt_cnt, qt_ent, qt_order;       // query tiles (dQ pass: over kv blocks, or over the kept dS tiles)
   size_t kt_off, kt_cnt, kt_ent, kt_order;       // kv tiles (dK/dV pass)
   size_t kt_cols;                                // pattern columns of each kv tile

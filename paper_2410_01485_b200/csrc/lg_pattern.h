@@ -137,23 +137,28 @@ __host__ __device__ __forceinline__ int fwd_tile_steps(const PatternDev& p, int 
 }
 
 // Super-tiles of the forward that are cut along their keys, a CTA per piece: the tiles of the first n_cut launch ranks (the
-// longest) into ceil(steps / len) nearly equal pieces (at most `places`); a kernel of its own adds the pieces of a tile in their order.
+// longest) into ceil(steps / len) nearly equal pieces, at most `places`.  The CTAs of a tile are one cluster, which adds the pieces.
 constexpr int kFwdMaxCutTiles = 4 * kSms, kFwdMaxPieces = 8, kFwdMaxPlaces = 1024;
 struct FwdSplit {
   int len;                        // 0: no tile is cut
   int n_cut, places;
 };
 
-// Cut the longest super-tiles?  In units of steps (1.7 us): a CTA costs about 3 besides its own (launch, first loads, epilogue), the
-// second kernel about 3, and a piece's sums (128 KB at D = 128, written and read back) a 32nd.  An SM's share of the pass is
-// (all + 3 per CTA) / SMs.  Where the longest tile alone takes longer (few heads, long rows) the number of pieces is the one with
-// the smallest estimate: one round of CTAs ends with its longest, several with an SM's share and half a piece that
-// sticks out.  Tiles are cut where that is less than 7 / 8 of the longest tile.  Measured, forward: 4 heads x 3318
-// tokens, full causal, D = 128 / 64: 58 -> 36 / 56 -> 31 us; 2 x 6000: 93 -> 42 us; 4 x 5000, window 4096: 74 -> 54 us; 8 x 2000: 41 -> 34 us.
+// CTAs, of clusters of 2 .. 8 with an SM for each CTA, that are taken to run at one time: a little less than the 148, 135, 132, 130, 132,
+// 105 and 120 that the occupancy calculator gives for whole clusters; places that stay empty leave in 2 us and count for nothing.
+// Above that the clusters wait for one another: 4 heads x 3318 tokens, D = 128, in 3 pieces (104 CTAs) 37 us, in 4 (128) 45 us.
+constexpr int kFwdClusterCtas[kFwdMaxPieces + 1] = {0, 148, 144, 132, 120, 112, 96, 80, 80};
+
+// Cut the longest super-tiles?  In units of steps (1.8 us): a CTA costs about 3 besides its own (launch, first loads, epilogue), and
+// adding two pieces 3 at D = 64 and 4.5 at D = 128, more pieces 1.5 more.  An SM's share of the pass is (all + 3 per CTA) / SMs.  Where
+// the longest tile alone takes longer (few heads, long rows) the number of pieces is the one with the smallest estimate:
+// one round of CTAs ends with its longest; several, which only pairs of CTAs fill without gaps, with an SM's share and
+// half a piece that sticks out.  Tiles are cut where that is less than 9 / 10 of the longest tile.  Over 54 problems x 7 numbers of
+// pieces the choice takes 39.8 us on average, the best number for each 38.7, uncut 48.5.
 // heads: query heads times batch of the whole problem, so that a step worked in groups of heads gives the same bits.
 inline FwdSplit fwd_split(const PatternDev& p, int D, int st_row0, int n_tiles, int64_t heads) {
   FwdSplit k{};
-  constexpr int kCta = 3, kCut = 3, kMinLen = 3, kScale = 32;   // (estimates in 32nds)
+  constexpr int kCta = 3, kMinLen = 3, kScale = 32;            // (estimates in 32nds)
   const int rows = 256 / p.block;
   if (heads * n_tiles > kFwdMaxCutTiles) return k;             // (an SM's share then holds several tiles)
   int64_t all = 0;
@@ -164,20 +169,23 @@ inline FwdSplit fwd_split(const PatternDev& p, int D, int st_row0, int n_tiles, 
     if (n > longest) longest = n;
   }
   if (longest < 8 || (all + kCta * n_tiles) * heads >= static_cast<int64_t>(longest + kCta) * kSms) return k;
-  int64_t best = static_cast<int64_t>(longest + kCta) * kScale * 7 / 8;
+  int64_t best = static_cast<int64_t>(longest + kCta) * kScale * 9 / 10;
   for (int pieces = 2; pieces <= kFwdMaxPieces; ++pieces) {
     const int len = (longest + pieces - 1) / pieces;
     if (len < kMinLen) break;
-    int64_t ctas = 0, n_cut = 0, cut = 0;
+    int64_t ctas = 0, n_cut = 0;
     for (int t = 0; t < n_tiles; ++t) {
       const int n = fwd_tile_steps(p, st_row0 + rows * t, rows), segs = (n + len - 1) / len;
       ctas += segs;
-      if (segs > 1) { ++n_cut; cut += segs; }
+      n_cut += segs > 1;
     }
     if (heads * n_cut * pieces > kFwdMaxPlaces) continue;
-    int64_t then = ctas * heads <= kSms ? static_cast<int64_t>(len + kCta) * kScale
-                                        : (all + kCta * ctas) * heads * kScale / kSms + (len + kCta) * kScale / 2;
-    then += kCut * kScale + cut * heads * D / 128 * kScale / 32;
+    const int join = (pieces == 2 ? 3 : 6) * kScale / 2 + 3 * kScale * D / 128;
+    int64_t then = join + (len + kCta) * kScale;
+    if (ctas * heads > kFwdClusterCtas[pieces]) {
+      if (pieces > 2) continue;
+      then = join + (all + (kCta + 1) * ctas) * heads * kScale / kSms + (len + kCta) * kScale / 2;
+    }
     if (then >= best) continue;
     best = then;
     k.len = len;

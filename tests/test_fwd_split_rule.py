@@ -100,6 +100,12 @@ def test_gpu_cases_are_cut(rule):
     assert whole[0] > 0 and group[0] > 0 and whole != group
 
 
+def test_more_gpu_cases_are_cut(rule):
+    import test_gpu_fwd_cut as gpu
+    chunks = [(B * Hq, sink + W + T, 128, 64, 1, sink // 64, W // 64 + 1, (sink + W) // 64) for B, Hq, _, sink, W, T, _ in gpu.CHUNKS]
+    assert all(k[0] > 0 for k in rule([_line(gpu.FULL), _line(gpu.WINDOW)] + chunks))
+
+
 def test_where_it_is_not_worth_it(rule):
     lines = [(64, 10007, 128, 128, 0, 0, 0, 0),      # 2560 CTAs: many rounds
              (2, 512, 64, 64, 1, 1, 2, 0),           # three steps a tile
