@@ -27,6 +27,8 @@ struct __align__(16) TileRec {
 constexpr int kDqEntInts = 5;   // ints per entry of the schedule of the dQ pass that reads dS back (dq_entries)
 constexpr unsigned long long kWsMagic = 0x4c47575348445231ull;   // "LGWSHDR1"
 static_assert(sizeof(WsHeader) == 256, "header size");
+// a word that a kernel can have left (0 included): a code of 1 to 4 and a site
+__device__ __forceinline__ bool is_status(unsigned int w) { return w == 0 || ((w >> 24) >= 1 && (w >> 24) <= 4 && (w & 0xffffffu) < 256); }
 
 // A call that was told its workspace holds prepared lists checks, before it reads any of them,
 // that the header carries a fingerprint it accepts; otherwise the CTA records code 3 and returns.

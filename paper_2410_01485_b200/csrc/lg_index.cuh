@@ -78,8 +78,9 @@ struct SchedArgs {
 // error word nobody has read yet moves to `latched`, and the fingerprint is withdrawn until the
 // lists are whole again.
 __device__ __forceinline__ void header_begin(WsHeader* h) {
-  if (h->magic != kWsMagic) { h->magic = kWsMagic; h->latched = 0; }
-  else if (h->error_word != 0 && h->latched == 0) h->latched = h->error_word;
+  // (memory that was a workspace before may hold the magic between words that were written over since)
+  if (h->magic != kWsMagic || !is_status(h->latched)) { h->magic = kWsMagic; h->latched = 0; }
+  else if (h->latched == 0 && is_status(h->error_word)) h->latched = h->error_word;
   h->error_word = 0;
   h->fingerprint = 0;
 }
