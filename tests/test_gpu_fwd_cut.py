@@ -106,3 +106,24 @@ def test_checked_build(lg, cfg):
         out.append(b.lg_sparse_attn_fwd(p, inp["q"], inp["k"], inp["v"], workspace=ws))
         assert b.lg_last_status(ws) == 0
     assert all(torch.equal(x, y) for x, y in zip(*out))
+
+
+def test_captured(lg):
+    """One kernel node, replayed on other inputs."""
+    p = lg.params_of(FULL)
+    ws = lg.attn_workspace(p, False)
+    lg.lg_sparse_attn_prepare(p, ws, False)
+    p.lists_prepared = 1
+    inp, other = (synth.make_attn_inputs(FULL, "cuda", seed=s) for s in (7, 8))
+    o, lse = lg.lg_sparse_attn_fwd(p, inp["q"], inp["k"], inp["v"], workspace=ws)
+    graph = torch.cuda.CUDAGraph()
+    before = lg.kernel_launches()
+    with torch.cuda.graph(graph):
+        lg.lg_sparse_attn_fwd(p, inp["q"], inp["k"], inp["v"], o=o, lse=lse, workspace=ws)
+    assert lg.kernel_launches() == before + 1
+    for x in ("q", "k", "v"):
+        inp[x].copy_(other[x])
+    graph.replay()
+    torch.cuda.synchronize()
+    ref = lg.lg_sparse_attn_fwd(lg.params_of(FULL), other["q"], other["k"], other["v"])
+    assert torch.equal(o, ref[0]) and torch.equal(lse, ref[1]) and lg.lg_last_status(ws) == 0
