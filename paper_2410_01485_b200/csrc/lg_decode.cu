@@ -474,9 +474,9 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
     while (c > 0 && start_of(c) > f) --c;
     return static_cast<int>(c);
   };
-  // the segment of my slice that starts at tile pos: n tiles from tile t0 on of unit (b, k), which CTAs c_lo .. c_hi share,
-  // `pieces` of them with a record
-  int b = 0, k = 0, t0 = 0, n = 0, nt = 0, c_lo = 0, c_hi = 0, pieces = 0;
+  // the segment of my slice that starts at tile pos: n tiles from tile t0 on of unit (b, k), whose nt tiles start at `first`
+  int b = 0, k = 0, t0 = 0, n = 0, nt = 0;
+  int64_t first = 0;
   auto segment = [&](int64_t pos) {
     while (static_cast<int64_t>(cum[b + 1]) * ups <= pos) ++b;          // skip finished / empty sequences
     nt = cum[b + 1] - cum[b];
@@ -484,7 +484,11 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
     k = narrow ? static_cast<int>(static_cast<uint32_t>(rel) / static_cast<uint32_t>(nt)) : static_cast<int>(rel / nt);
     t0 = static_cast<int>(rel - static_cast<int64_t>(k) * nt);
     n = static_cast<int>(min(static_cast<int64_t>(nt - t0), f1 - pos));
-    const int64_t first = before + static_cast<int64_t>(k) * nt;
+    first = before + static_cast<int64_t>(k) * nt;
+  };
+  // the CTAs c_lo .. c_hi that share the segment's unit, `pieces` of them with a record
+  int c_lo = 0, c_hi = 0, pieces = 0;
+  auto sharers = [&]() {
     c_lo = (t0 == 0) ? static_cast<int>(blockIdx.x) : cta_of(first);
     c_hi = (t0 + n == nt) ? static_cast<int>(blockIdx.x) : cta_of(first + nt - 1);
     pieces = c_hi - c_lo + 1;
@@ -515,22 +519,33 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
   // releasing ticket: append + decode of one sequence over 4224 slots, 64 / 8 heads,
   // 12.7 -> 11.6 us, of 16 sequences 47.2 -> 46.2 us (13.7 and 49.2 us before the hint).
   // With more sequences than threads a count would be read twice and the readings could differ: no plan and no hint.
-  if (a.B <= kDecThreads) plan();
-  if (f0 < f1 && (threadIdx.x & 31) < 2) {
-    const int tb = t0 + static_cast<int>(static_cast<int64_t>(n) * warp / kDecWarps);
-    const int te = min(t0 + static_cast<int>(static_cast<int64_t>(n) * (warp + 1) / kDecWarps), tb + kDecHintTiles);
-    const int slot0 = tb * kDecTile, rows = min(te * kDecTile, a.C) - slot0;
-    if (rows > 0) {
-      const __nv_bfloat16* base = (threadIdx.x & 1) ? a.v_cache : a.k_cache;
-      prefetch_l2(base + ((static_cast<int64_t>(b) * a.Hkv + k / a.HG) * a.C + slot0) * D, rows * D * 2);
-    }
-  }
-  pdl_wait();
-  int nvalid = f0 < f1 ? decode_valid_of(a, b) : 0;        // (travels with the counts)
-  const bool changed = a.B > kDecThreads || (threadIdx.x < a.B && decode_tiles_of(a, threadIdx.x) != tiles);
-  if (__syncthreads_or(changed)) {
+  // The plan's code is there once, and the hint leaves as soon as its addresses are known: behind a kernel that does not let
+  // its successors start early, with code and counts out of the L2, instructions fetched ahead of the first load are what
+  // a decode waits for.  Alone behind a flushed L2: one sequence over 4224 slots 20.5 us without plan and hint ahead, 28.7 with two
+  // copies of the plan, 22.5 now; 8 x 2 heads over 1088 18.4 / 20.5 / 18.4; 32 x 8 over 1024 43.0 / 49.2 / 43.0.
+  int nvalid = 0;
+  bool planned = false;                    // the first segment's sharers and nvalid are known
+#pragma unroll 1
+  for (bool ahead = a.B <= kDecThreads;; ahead = false) {
+    if (!ahead) pdl_wait();
     plan();
-    if (f0 < f1) nvalid = decode_valid_of(a, b);
+    if (!ahead) break;
+    if (f0 < f1) {
+      if ((threadIdx.x & 31) < 2) {
+        const int tb = t0 + static_cast<int>(static_cast<int64_t>(n) * warp / kDecWarps);
+        const int te = min(t0 + static_cast<int>(static_cast<int64_t>(n) * (warp + 1) / kDecWarps), tb + kDecHintTiles);
+        const int slot0 = tb * kDecTile, rows = min(te * kDecTile, a.C) - slot0;
+        if (rows > 0) {
+          const __nv_bfloat16* base = (threadIdx.x & 1) ? a.v_cache : a.k_cache;
+          prefetch_l2(base + ((static_cast<int64_t>(b) * a.Hkv + k / a.HG) * a.C + slot0) * D, rows * D * 2);
+        }
+      }
+      sharers();
+    }
+    pdl_wait();
+    if (f0 < f1) nvalid = decode_valid_of(a, b);           // (travels with the counts)
+    planned = !__syncthreads_or(threadIdx.x < a.B && decode_tiles_of(a, threadIdx.x) != tiles);
+    if (planned) break;
   }
   __shared__ int s_last;
   // units of sequences without tokens get their (empty) result here, spread over the CTAs
@@ -542,10 +557,8 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
     }
   }
   for (int64_t pos = f0; pos < f1;) {
-    if (pos != f0) {
-      segment(pos);
-      nvalid = decode_clamped(a, a.n_tokens[b]);
-    }
+    if (pos != f0) segment(pos);
+    if (!planned) nvalid = decode_clamped(a, a.n_tokens[b]);
     const int tb = t0 + static_cast<int>(static_cast<int64_t>(n) * warp / kDecWarps);
     const int te = t0 + static_cast<int>(static_cast<int64_t>(n) * (warp + 1) / kDecWarps);
     const int64_t u = static_cast<int64_t>(b) * ups + k;
@@ -554,6 +567,8 @@ __global__ void __launch_bounds__(kDecWarps * 32) decode_stream_kernel(const Dec
     decode_run_segment<D>(a, dsmem, b, k / a.HG, k % a.HG, nvalid, tb, te,
                           a.part + (blockIdx.x + u) * (kDecHeads * kRec), direct);
     pos += n;
+    if (!direct && !planned) sharers();
+    planned = false;
     if (direct) continue;
     // The CTA that delivers the last record of a unit merges it (records are read in index
     // order, so the result does not depend on which CTA that is) and re-arms the counter.  The ticket releases the CTA's
