@@ -131,7 +131,11 @@ lg_status lg_sparse_attn_prepare(const lg_attn_params* p, void* workspace, size_
 
 /* O = softmax(scale * Q K^T + mask) V;  LSE_i = ln sum_j exp(scale * q_i . k_j) over the
  * visible keys.  q [B,Hq,L,D], k, v [B,Hkv,L,D], o [B,Hq,L,D] bf16 (device);
- * lse [B,Hq,L] fp32 contiguous (device).  workspace: device, 256-byte aligned.           */
+ * lse [B,Hq,L] fp32 contiguous (device).  workspace: device, 256-byte aligned.
+ * With few heads and long rows a row's keys are worked in pieces; how many follows from B * Hq, L
+ * and the pattern, so the last bits of a head's results may differ between calls with other head
+ * counts.  With lists_prepared = 1 the call only reads the workspace (and reports through its
+ * status word): forwards on several streams may share prepared lists.                     */
 lg_status lg_sparse_attn_fwd(const lg_attn_params* p, const void* q, const void* k, const void* v,
                              void* o, float* lse, void* workspace, size_t workspace_bytes,
                              void* stream);

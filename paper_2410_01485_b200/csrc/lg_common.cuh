@@ -326,7 +326,9 @@ __device__ __forceinline__ float4 cluster_ld128(uint32_t addr) {
 // A kernel launched with `overlap` (launch_kernel, lg_host.h) may start while the kernel before it on the stream drains:
 // its CTAs take the SMs that fall free, and everything up to pdl_wait() -- which returns when that kernel has
 // finished and its writes are visible -- runs beside the other's tail.  Nothing global may be touched before the
-// wait, and what it reads may still be written while it already runs: no `const __restrict__` inputs (loads through those
+// wait (one exception: decode_stream_kernel looks at the token counts and asks cache lines into the L2; it reads the counts
+// through the L2, uses them for addresses that lie inside the caches whatever they hold, and reads them again behind the wait),
+// and what it reads may still be written while it already runs: no `const __restrict__` inputs (loads through those
 // may be moved above the wait) and no loads by the non-coherent path, which is for data nobody writes during the kernel's
 // lifetime.  Every thread that goes on to touch something calls the wait.  pdl_trigger() lets the next kernel start
 // once every CTA has called it (or left); without it the next one starts when this one has finished.

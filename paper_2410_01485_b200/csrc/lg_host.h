@@ -36,7 +36,8 @@ void note_launch();
 
 constexpr int kMaxDevices = 64;   // devices whose properties are looked up once
 
-// Launch of a kernel that calls pdl_wait() (lg_common.cuh) before it touches global memory: with `overlap` it may
+// Launch of a kernel that calls pdl_wait() (lg_common.cuh) before it touches global memory (or
+// only for a hint, as the decode does): with `overlap` it may
 // start while the kernel before it on the stream drains.  A failed launch is reported by the result alone: it does not
 // stay behind as the runtime's last error, which a later call would take for its own.
 template <typename... Params, typename... Args>
@@ -115,7 +116,7 @@ lg_status resolve(const lg_attn_params* p, Resolved* r, bool want_bwd = false, i
 
 // Layout of the attention workspace (all offsets 256-byte aligned).
 struct WsLayout {
-  // per schedule: start of each tile's entries, their number, the entries, launch rank -> tile
+  // per schedule: start of each tile's entries, their number, the entries, by launch rank a TileRec of the tile
   size_t sq_off, sq_cnt, sq_ent, sq_order;       // super-tiles (forward)
   size_t qt_off, qt_cnt, qt_ent, qt_order;       // query tiles (dQ pass: over kv blocks, or over the kept dS tiles)
   size_t kt_off, kt_cnt, kt_ent, kt_order;       // kv tiles (dK/dV pass)

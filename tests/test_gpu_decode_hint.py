@@ -1,7 +1,6 @@
-"""Decode launched overlapped looks at the token counts before the kernel ahead of it has finished, as a hint of what to ask
-into the L2.  The counts that hold are those after that kernel: steps whose counts are written by the kernel just
-ahead (other lengths, empty and negative ones among them) give what the same steps give one by one, also for batches
-of more sequences than a block has threads."""
+"""Decode steps whose counts are written by an ordinary kernel just ahead (other lengths, empty and negative ones among them) give what the
+same steps give one by one, also for batches of more sequences than a block has threads.  (That kernel does not let the decode
+start early; counts that change behind the decode's early look at them are in test_gpu_decode_counts.py.)"""
 import pytest
 import torch
 
