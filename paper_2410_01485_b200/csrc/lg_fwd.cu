@@ -47,8 +47,9 @@ lg_status launch_fwd(const Resolved& r, const WsLayout& w, const void* q, const 
   const bool pairs = fwd_two_ctas(r);
 #define LG_FWD_CASE(DD, BB, NN) \
   if (r.D == DD && r.block == BB && pairs == (NN == 1)) return launch_fwd_t<DD, BB, NN, false>(r, w, q, k, v, o, lse, ws, stream);
+  // (where a part of a device cannot hold a cluster the launch is refused, and the tiles stay whole)
 #define LG_FWD_CUT_CASE(DD, BB) \
-  if (r.fsplit.len > 0 && r.D == DD && r.block == BB) return launch_fwd_t<DD, BB, 2, true>(r, w, q, k, v, o, lse, ws, stream);
+  if (r.fsplit.len > 0 && r.D == DD && r.block == BB && launch_fwd_t<DD, BB, 2, true>(r, w, q, k, v, o, lse, ws, stream) == LG_OK) return LG_OK;
   LG_FWD_CUT_CASE(128, 128)
   LG_FWD_CUT_CASE(128, 64)
   LG_FWD_CUT_CASE(64, 128)
